@@ -190,7 +190,9 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A,
  *                       M >= 256, N >= 2048 and at least a round and a half of 256 x 256 tiles
  *                       on the SM pairs: the CTA-pair tensor-core kernel; else the one-CTA
  *                       tensor-core kernel
- *   BITPLANES operands  N <= 16: one warp per weight row over the planes; else the tiled
+ *   BITPLANES operands  N <= 16: one warp per weight row over the planes; else tiled: the planes
+ *                       are expanded to bytes inside the tensor-core kernel, or (QNN_PATH_BITSERIAL,
+ *                       skip_planes, sixteen plane pairs up to 2^30 multiply-accumulates) the
  *                       AND/POPC kernel
  *   FIELDS weights      N <= 16 only: one or two columns: one warp per
  *                       packed weight row, an AND and a 4-way byte dot product per word and
@@ -253,7 +255,7 @@ qnn_status qnn_im2col(const qnn_conv_desc *d, const void *in, void *lowered, voi
  * activations with pad > 0 are UNSUPPORTED (zero is not representable).
  * The lowered matrix of Section 3.2 is written to `workspace` only where the GEMM
  * kernel cannot form its tiles itself.  Bit-plane maps are lowered on the fly by the
- * staging code of the tiled AND/POPC kernel (word-granular, as in Section 3.2).
+ * loading code of the tiled kernels (word-granular, as in Section 3.2).
  * 8-bit maps are lowered inside the tensor-core kernel: by its tensor-map loader
  * when C and in_pitch are multiples of 16 (the CTA-pair kernel for large layers,
  * the one-CTA kernel otherwise); by lowering warps when pixels are contiguous and

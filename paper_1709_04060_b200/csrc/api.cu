@@ -98,6 +98,16 @@ static void conv_to_gemm(const qnn_conv_desc *d, qnn_gemm_desc *g) {
     g->skip_planes = 0;
 }
 
+// Bit planes with more columns than the few-column kernel takes go through the tensor cores, expanded
+// to bytes inside the kernel, unless the caller asks for the bit-serial path or leaves plane pairs
+// out.  Sixteen plane pairs (W4A4) up to 2^30 multiply-accumulates keep the AND/POPC kernel although
+// dense operands take longer there (1024^3: 156 us against 15): that a call gets faster with
+// skip_planes and with empty plane tiles is what this format promises at these sizes.
+static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
+    if (d->path != QNN_PATH_AUTO || d->skip_planes != 0) return false;
+    return d->w_bits * d->a_bits < 16 || (double)d->M * d->N * d->K > double(1 << 30);
+}
+
 }  // namespace qnn
 
 using namespace qnn;
@@ -208,6 +218,10 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
     }
     // a handful of columns: stream the weight planes once, one warp per row
     if (gemv_planes_fits(d)) return gemv_planes_launch(d, W, A, thr, out, (cudaStream_t)stream);
+    if (planes_on_tensor_cores(d)) {
+        st = gemm_tc_planes_launch(nullptr, d, W, A, thr, out, (cudaStream_t)stream);
+        if (st != QNN_ERR_UNSUPPORTED) return st;
+    }
     return gemm_bitserial_launch(d, W, A, thr, out, (cudaStream_t)stream);
 }
 
@@ -282,6 +296,10 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
     // bit-plane maps on the tiled bit-serial kernel: its staging code lowers on the fly (a handful
     // of output pixels goes through the lowered matrix and the few-column kernel instead)
     if (path == QNN_PATH_BITSERIAL && !(explicit_env && explicit_env[0] == '1') && !gemv_planes_fits(&g)) {
+        if (planes_on_tensor_cores(&g)) {
+            st = gemm_tc_planes_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
+            if (st != QNN_ERR_UNSUPPORTED) return st;
+        }
         st = gemm_bitserial_conv_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
         if (st != QNN_ERR_UNSUPPORTED) return st;
     }

@@ -44,6 +44,7 @@
 #include <stdlib.h>
 
 #include "common.cuh"
+#include "planes.cuh"
 #include "tc_ptx.cuh"
 
 namespace qnn {
@@ -109,6 +110,14 @@ struct TcParams {
     int lw_step;           // stride*C: bytes between the runs of neighbouring output pixels
     int lw_run, lw_vecs;   // bytes of a run (KW*C) and its 16-byte pieces
     int lw_stage_bytes;    // bytes of one staging buffer
+    // Bit-plane operands (LOWER == 3): expanded to bytes inside the kernel, both of them.  Weights
+    // uint32 [pl_wb][M][pl_kw], activations uint32 [pl_ab][N][pl_kw] or (pl_conv) the
+    // channel-interleaved map [pl_ab][B][H][W][pl_cw], lowered on the fly.
+    const uint32_t *pl_W, *pl_A;
+    long long pl_wplane, pl_aplane;    // words per plane of the two operands
+    int pl_wb, pl_ab, pl_wkind, pl_akind, pl_kw;    // planes, PL_* kinds, depth words per row
+    int pl_conv, pl_cw;                // 1: implicit convolution; words per pixel
+    int pl_kbs, pl_vec;                // k-blocks per ring slot (2 or 4); 1: copies of 16 bytes
     // CTA-pair kernel with a split last round (see qgemm_tc2_kernel): the depth of each of the last
     // split_rem tiles is shared by two neighbouring CTA pairs, which exchange int32 partial sums
     // through global memory.
@@ -523,6 +532,174 @@ __device__ __forceinline__ bool epilogue_tile(const TcParams &p, const int *thr_
     return true;
 }
 
+// ------------------------------------------------------- bit planes expanded to bytes
+// The LOWER == 3 kernels take both operands as bit planes and multiply them on the tensor cores:
+// an expanding thread reads one 32-element word of every plane of a row and writes the 32 bytes
+// those elements stand for into the operand tile.
+constexpr int PL_WARPS = 4;        // expanding warps of the LOWER == 3 kernels, and as many loading warps
+// ROWS words of this thread (rows 8 PL_WARPS apart) into an operand tile.  src: shared-memory address
+// of the first row's word in the first plane, rows and planes that many bytes apart; piece0, piece1:
+// the two 16-byte pieces of the first row, already swizzled (the later rows' swizzle is the same).
+template <int ROWS, int B, int KIND>
+__device__ __forceinline__ void expand_rows(uint32_t src, uint32_t row_step, uint32_t plane_step, uint32_t keep, uint32_t piece0, uint32_t piece1) {
+    uint32_t w[ROWS][B];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w[i][b]) : "r"(src + (uint32_t)i * row_step + (uint32_t)b * plane_step));
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        uint32_t o[8];
+        expand_word<B, KIND>(w[i], o);
+        if (KIND == PL_BIPOLAR && keep != 0xFFFFFFFFu) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[j] &= ((keep >> j) & 0x01010101u) * 0xFFu;
+        }
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                     ::"r"(piece0 + (uint32_t)(i * 8 * PL_WARPS * TC_BK)), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                     ::"r"(piece1 + (uint32_t)(i * 8 * PL_WARPS * TC_BK)), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
+    }
+}
+template <int ROWS>
+__device__ __forceinline__ void expand_rows_of(int planes, int kind, uint32_t src, uint32_t row_step, uint32_t plane_step, uint32_t keep,
+                                               uint32_t piece0, uint32_t piece1) {
+    if (kind == PL_BIPOLAR) { expand_rows<ROWS, 1, PL_BIPOLAR>(src, row_step, plane_step, keep, piece0, piece1); return; }
+#define QNN_PL_CASE(B_)                                                                                                \
+    case B_:                                                                                                           \
+        if (kind == PL_SIGNED) expand_rows<ROWS, B_, PL_SIGNED>(src, row_step, plane_step, keep, piece0, piece1);      \
+        else expand_rows<ROWS, B_, PL_UNSIGNED>(src, row_step, plane_step, keep, piece0, piece1);                      \
+        break;
+    switch (planes) { QNN_PL_CASE(1) QNN_PL_CASE(2) QNN_PL_CASE(3) QNN_PL_CASE(4) }
+#undef QNN_PL_CASE
+}
+
+// Asynchronous copy of WORDS (1 or 4) words into shared memory; zeros where they lie outside.
+template <int WORDS>
+__device__ __forceinline__ void copy_words(uint32_t dst, const uint32_t *src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(4 * WORDS), "r"(ok ? 4 * WORDS : 0) : "memory");
+}
+
+// Ring of plane words of a LOWER == 3 kernel: two slots of pl_kbs k-blocks (2 or 4), each
+// [weight plane][row], [activation plane][row] with 4 pl_kbs words a row; the 16-byte units of a row
+// (one k-block each) are swizzled by its index, so that the eight rows a warp expands at a time fall
+// into different banks.
+struct PlRing {
+    uint32_t row_b, w_plane, a_plane, a_off, slot_b, umask, ushift;
+    __device__ __forceinline__ PlRing(const TcParams &p, int bn) {
+        row_b = 16u * (uint32_t)p.pl_kbs; w_plane = (uint32_t)bn * row_b; a_plane = TC_BP * row_b;
+        a_off = (uint32_t)p.pl_wb * w_plane; slot_b = a_off + (uint32_t)p.pl_ab * a_plane;
+        umask = (uint32_t)p.pl_kbs - 1u; ushift = p.pl_kbs == 4 ? 1u : 2u;
+    }
+    __device__ __forceinline__ uint32_t unit(uint32_t u, uint32_t row) const { return (u ^ ((row >> ushift) & umask)) << 4; }
+};
+
+// Loading warps: words of both operands into the ring, a slot at a time, so that one request touches
+// few rows (what a copy costs the load unit is the number of cache lines it touches).  They are
+// warps of their own because the expanding warps fence between their stores and the tensor core's
+// reads, and a fence would wait for the copies its thread has in flight.  UNIT: words per copy (4
+// where rows, or the pixels of a map, are whole 16-byte units).
+template <int BN, int UNIT, typename Smem>
+__device__ __forceinline__ void load_planes_loop(const TcParams &p, Smem &sm, uint32_t raw, int w, int lane, volatile int *abort_flag) {
+    const PlRing ring(p, BN);
+    const int ch = 4 * p.pl_kbs, lpr = ch / UNIT, rpi = 32 / lpr;      // words per row, lanes per row, rows per request
+    const int cw0 = (lane % lpr) * UNIT, crow = lane / lpr;            // first word of the slot, first row
+    uint32_t chunk = 0;
+    bool alive = true;
+    for (int u = blockIdx.x; alive && u < p.units; u += gridDim.x) {
+        const TcUnit un = tc_unit(p, u, BN);
+        int word = un.kb0 * 4 + cw0;
+        const int word_end = min(un.kb1 * 4, p.pl_kw);
+        // implicit convolution: lane l keeps the first tap of the warp's pixel l; the tap of the word
+        int pix_at = 0, pix_ih = 0, pix_iw = 0, kh = 0, kw = 0, cword = 0;
+        if (p.pl_conv) {
+            const int pix = min(un.p0 + 32 * w + lane, p.N - 1);
+            const int b = pix / p.cv_OHW, r = pix - b * p.cv_OHW, oh = r / p.cv_OW;
+            pix_ih = oh * p.cv_stride - p.cv_pad;
+            pix_iw = (r - oh * p.cv_OW) * p.cv_stride - p.cv_pad;
+            pix_at = (b * p.lw_H + pix_ih) * p.lw_W + pix_iw;
+            const int tap = word / p.pl_cw;
+            cword = word - tap * p.pl_cw;
+            kh = tap / p.cv_KW;
+            kw = tap - kh * p.cv_KW;
+        }
+        for (int kb0 = un.kb0; kb0 < un.kb1; kb0 += p.pl_kbs, ++chunk) {
+            const uint32_t slot = chunk & 1, dst = raw + slot * ring.slot_b;
+            if (!(alive = warp_wait(&sm.in_empty[slot], ((chunk >> 1) & 1) ^ 1, lane, abort_flag))) break;
+            const bool in = word < word_end;
+            for (int b = 0; b < p.pl_wb; ++b) {
+                const uint32_t *q = p.pl_W + (size_t)b * p.pl_wplane + word;
+#pragma unroll 4
+                for (int r = w * (BN / 4) + crow; r < (w + 1) * (BN / 4); r += rpi) {
+                    const bool ok = in && un.c0 + r < p.M;
+                    copy_words<UNIT>(dst + (uint32_t)b * ring.w_plane + (uint32_t)r * ring.row_b + ring.unit((uint32_t)cw0 >> 2, (uint32_t)r) + 4u * (cw0 & 3),
+                                     ok ? q + (size_t)(un.c0 + r) * p.pl_kw : p.pl_W, ok);
+                }
+            }
+#pragma unroll 4
+            for (int j = crow; j < 32; j += rpi) {
+                const int r = 32 * w + j, n = un.p0 + r;
+                bool ok = in && n < p.N;
+                size_t at = (size_t)n * p.pl_kw + word;
+                if (p.pl_conv) {
+                    const int ih = __shfl_sync(0xffffffffu, pix_ih, j) + kh, iw = __shfl_sync(0xffffffffu, pix_iw, j) + kw;
+                    const int base = __shfl_sync(0xffffffffu, pix_at, j);
+                    ok = ok && (unsigned)ih < (unsigned)p.lw_H && (unsigned)iw < (unsigned)p.lw_W;
+                    at = (size_t)(base + kh * p.lw_W + kw) * p.pl_cw + cword;
+                }
+                const uint32_t d = dst + ring.a_off + (uint32_t)r * ring.row_b + ring.unit((uint32_t)cw0 >> 2, (uint32_t)r) + 4u * (cw0 & 3);
+                for (int b = 0; b < p.pl_ab; ++b)
+                    copy_words<UNIT>(d + (uint32_t)b * ring.a_plane, ok ? p.pl_A + (size_t)b * p.pl_aplane + at : p.pl_A, ok);
+            }
+            // the barrier counts this thread once its copies have landed
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sm.in_full[slot])) : "memory");
+            word += ch;
+            if (p.pl_conv)
+                for (cword += ch; cword >= p.pl_cw; cword -= p.pl_cw)
+                    if (++kw == p.cv_KW) { kw = 0; ++kh; }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");               // nothing in flight when the CTA exits
+    __syncwarp();
+}
+
+// Expanding warps: lane l of warp w turns word l & 3 of a k-block, rows 8 w + l / 4 + 32 i, into bytes.
+// The 16-byte stores of eight lanes (two rows, the swizzle shifts them by one piece) fall into
+// different banks.
+template <int BN, int STAGES, typename Smem>
+__device__ __forceinline__ void expand_loop(const TcParams &p, Smem &sm, uint32_t raw, int w, int lane, volatile int *abort_flag) {
+    constexpr int RS = 8 * PL_WARPS, WR = BN / RS, AR = TC_BP / RS;
+    const PlRing ring(p, BN);
+    const uint32_t c = lane & 3, r0 = 8 * w + (lane >> 2), x = r0 & 7;
+    const uint32_t off0 = r0 * TC_BK + (((2 * c) ^ x) << 4), off1 = r0 * TC_BK + (((2 * c + 1) ^ x) << 4);
+    uint32_t it = 0, chunk = 0;
+    for (int u = blockIdx.x; u < p.units; u += gridDim.x) {
+        const TcUnit un = tc_unit(p, u, BN);
+        for (int kb0 = un.kb0; kb0 < un.kb1; kb0 += p.pl_kbs, ++chunk) {
+            const uint32_t slot = chunk & 1;
+            if (!warp_wait(&sm.in_full[slot], (chunk >> 1) & 1, lane, abort_flag)) return;
+            const int kb1 = min(kb0 + p.pl_kbs, un.kb1);
+            for (int kb = kb0; kb < kb1; ++kb, ++it) {
+                const int s = it % STAGES;
+                const uint32_t ph = (it / STAGES) & 1;
+                if (!warp_wait(&sm.empty[s], ph ^ 1, lane, abort_flag)) return;
+                const uint32_t wt = smem_u32(sm.wgt[s]), at = smem_u32(sm.act[s]);
+                const uint32_t src = raw + slot * ring.slot_b + r0 * ring.row_b + ring.unit((uint32_t)(kb - kb0), r0) + 4u * c;
+                expand_rows_of<WR>(p.pl_wb, p.pl_wkind, src, RS * ring.row_b, ring.w_plane, 0xFFFFFFFFu, wt + off0, wt + off1);
+                // +-1 has no zero: activation elements past the end of the depth have to become zero bytes
+                const int left = p.K - 32 * (kb * 4 + (int)c);
+                const uint32_t keep = left >= 32 ? 0xFFFFFFFFu : (left <= 0 ? 0u : (1u << left) - 1u);
+                expand_rows_of<AR>(p.pl_ab, p.pl_akind, src + ring.a_off, RS * ring.row_b, ring.a_plane, keep, at + off0, at + off1);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core's reads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.full[s]);
+            }
+            if (lane == 0) mbar_arrive(&sm.in_empty[slot]);
+        }
+    }
+}
+
 // ------------------------------------------------------- kernel A: one CTA per tile
 template <int BN, int STAGES, int OUT_BITS>
 struct TcSmem {
@@ -538,8 +715,8 @@ struct TcSmem {
     uint64_t ring_free;
     uint64_t landed[4 * 4];
     uint64_t w_full;           // LOWER: the resident weights have landed
-    uint64_t in_full[2];       // LOWER: image rows of a unit have landed in staging buffer b
-    uint64_t in_empty[2];      // LOWER: the lowering warps are done with staging buffer b
+    uint64_t in_full[2];       // LOWER: image rows of a unit (bit planes: words of a ring slot) have landed in buffer b
+    uint64_t in_empty[2];      // LOWER: the lowering warps are done with buffer b
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -562,11 +739,11 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_consta
 
     if (threadIdx.x == 0) {
         // LOWER: a stage is full when every lowering thread has written its row of the activation tile
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&sm.full[s], LOWER == 1 ? LW_THREADS : (LOWER == 2 ? LW_THREADS + 1 : 1)); mbar_init(&sm.empty[s], 1); }
+        for (int s = 0; s < STAGES; ++s) { mbar_init(&sm.full[s], LOWER == 3 ? PL_WARPS : LOWER == 1 ? LW_THREADS : (LOWER == 2 ? LW_THREADS + 1 : 1)); mbar_init(&sm.empty[s], 1); }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&sm.tmem_full[b], 1); mbar_init(&sm.tmem_empty[b], EPI_WARPS);
             mbar_init(&sm.thr_full[b], 1); mbar_init(&sm.thr_empty[b], EPI_WARPS);
-            mbar_init(&sm.in_full[b], 1); mbar_init(&sm.in_empty[b], LW_WARPS);
+            mbar_init(&sm.in_full[b], LOWER == 3 ? 32 * PL_WARPS : 1); mbar_init(&sm.in_empty[b], LOWER == 3 ? PL_WARPS : LW_WARPS);
         }
         mbar_init(&sm.w_full, 1);
         mbar_init(&sm.ring_free, 1);
@@ -593,7 +770,9 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_consta
     uint8_t *const w_extra = reinterpret_cast<uint8_t *>(&sm) + ((sizeof(Smem) + 1023) & ~size_t(1023));
     uint8_t *const stage_in = w_extra + (LOWER == 1 && p.num_kb > STAGES ? (size_t)(p.num_kb - STAGES) * BN * TC_BK : 0);
     auto w_block = [&](int kb) -> uint8_t * { return kb < STAGES ? sm.wgt[kb] : w_extra + (size_t)(kb - STAGES) * BN * TC_BK; };
-    if (LOWER && warp == 0) {
+    if (LOWER == 3 && warp == 0) {
+        // bit planes: the loading and expanding warps fill the operand tiles
+    } else if (LOWER && warp == 0) {
         // ------------------- producer of the LOWER kernels: the weights once, then image rows
         if (lane == 0) {
             uint32_t staged = 0;                               // staging copies issued
@@ -648,6 +827,15 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_consta
                 if (staged > 0) mbar_wait(&sm.in_full[(staged - 1) & 1], ((staged - 1) >> 1) & 1, abort_flag);
             }
         }
+        __syncwarp();
+    } else if (LOWER == 3 && warp > STAGER_WARP) {
+        if constexpr (LOWER == 3) {
+            if (p.pl_vec) load_planes_loop<BN, 4>(p, sm, smem_u32(w_extra), warp - (STAGER_WARP + 1), lane, abort_flag);
+            else load_planes_loop<BN, 1>(p, sm, smem_u32(w_extra), warp - (STAGER_WARP + 1), lane, abort_flag);
+        }
+    } else if (LOWER == 3 && warp >= 2 + EPI_WARPS / 2 && warp < STAGER_WARP) {
+        // four of the usual epilogue warps expand instead
+        if constexpr (LOWER == 3) expand_loop<BN, STAGES>(p, sm, smem_u32(w_extra), warp - (2 + EPI_WARPS / 2), lane, abort_flag);
         __syncwarp();
     } else if (LOWER && warp > STAGER_WARP) {
         // ------------------------------------------------------------ lowering warps
@@ -843,17 +1031,24 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_consta
         // ------------------------------------------------------------ epilogue
         uint32_t tcount = 0;
         TcExchange xc;
-        xc.zone = smem_u32(&sm.wgt[0][0]);
+        // the exchange's slabs take 512 bytes per channel: the weight ring of four stages or more, or
+        // (bit planes, three stages) both operand rings, which are adjacent and idle by then
+        static_assert(LOWER == 3 ? STAGES * (TC_BP + BN) >= 4 * BN : (LOWER != 0 || STAGES >= 4), "exchange slabs overrun the ring");
+        xc.zone = LOWER == 3 ? smem_u32(&sm.act[0][0]) : smem_u32(&sm.wgt[0][0]);
         xc.ring_free = &sm.ring_free; xc.landed = sm.landed;
         xc.rank = p.share ? cluster_ctarank() : 0u;
         for (int u = blockIdx.x; u < p.units; u += gridDim.x, ++tcount) {
             const TcUnit un = tc_unit(p, u, BN);
             const uint32_t buf = tcount & 1, acc_ph = (tcount >> 1) & 1;
-            if (!epilogue_tile<OUT_MODE, OUT_BITS>(p, sm.thr[buf], &sm.thr_full[buf], &sm.thr_empty[buf], acc_ph,
-                                                   &sm.tmem_full[buf], acc_ph, tmem_base + buf * BN, BN,
-                                                   un.p0, un.c0, un.shared, xc, warp, lane, abort_flag, (int)tcount))
-                break;
-            if (lane == 0) mbar_arrive(&sm.tmem_empty[buf]);     // one arrival per warp
+            // with bit planes a warp also takes the part of the warp four further on
+            bool ok = true;
+            for (int e = warp; ok && e <= (LOWER == 3 ? warp + EPI_WARPS / 2 : warp); e += EPI_WARPS / 2) {
+                ok = epilogue_tile<OUT_MODE, OUT_BITS>(p, sm.thr[buf], &sm.thr_full[buf], &sm.thr_empty[buf], acc_ph,
+                                                       &sm.tmem_full[buf], acc_ph, tmem_base + buf * BN, BN,
+                                                       un.p0, un.c0, un.shared, xc, e, lane, abort_flag, (int)tcount);
+                if (ok && lane == 0) mbar_arrive(&sm.tmem_empty[buf]);     // one arrival per warp's part
+            }
+            if (!ok) break;
         }
     }
 
@@ -1270,15 +1465,22 @@ template <int BN, int STAGES, int OUT_BITS>
 constexpr size_t tc_lower_base_smem() { return ((sizeof(TcSmem<BN, STAGES, OUT_BITS>) + 1023) & ~size_t(1023)) + 1024; }
 constexpr size_t TC_SMEM_LIMIT = 227 * 1024;
 
+// The ring of plane words of a LOWER == 3 kernel: two slots of kbs k-blocks of both operands.
+static size_t pl_ring_bytes(const TcParams &p, int bn, int kbs) {
+    return (size_t)2 * kbs * 16 * (bn * p.pl_wb + TC_BP * p.pl_ab);
+}
+
 template <int BN, int STAGES, int OUT_MODE, int OUT_BITS, int LOWER = 0>
 static qnn_status launch_cfg(const CUtensorMap &ma, const CUtensorMap &mw, const TcParams &p, cudaStream_t s) {
     auto kern = qgemm_tc_kernel<BN, STAGES, OUT_MODE, OUT_BITS, LOWER>;
     size_t smem = sizeof(TcSmem<BN, STAGES, OUT_BITS>) + 1024;
-    if (LOWER) {
+    if (LOWER == 3) {
+        smem = tc_lower_base_smem<BN, STAGES, OUT_BITS>() + pl_ring_bytes(p, BN, p.pl_kbs);
+    } else if (LOWER) {
         smem = tc_lower_base_smem<BN, STAGES, OUT_BITS>() + 2 * (size_t)p.lw_stage_bytes +
                (LOWER == 1 && p.num_kb > STAGES ? (size_t)(p.num_kb - STAGES) * BN * TC_BK : 0);
-        if (smem > TC_SMEM_LIMIT) return QNN_ERR_UNSUPPORTED;
     }
+    if (smem > TC_SMEM_LIMIT) return QNN_ERR_UNSUPPORTED;
     // per instantiation and device: the largest size configured so far
     static size_t attr_smem[QNN_MAX_DEVICES] = {0};
     const int dev = current_device();
@@ -1395,7 +1597,9 @@ struct TcPlan {
     bool share;
 };
 
-static bool tc_plan(const qnn_gemm_desc *d, int sms, int num_kb, TcPlan *pl) {
+// planes: the LOWER == 3 kernels, whose k-block time is set by the expansion (measured: about 1100
+// cycles and 75 per word that an expanding thread takes).
+static bool tc_plan(const qnn_gemm_desc *d, int sms, int num_kb, TcPlan *pl, bool planes = false) {
     const char *no_share = getenv("QNN_TC_NO_SHARE");
     const bool allowed = !(no_share && no_share[0] == '1');
     // Channel tile.  An MMA costs about the same for every N (measured: the 128 x 32-byte
@@ -1411,10 +1615,10 @@ static bool tc_plan(const qnn_gemm_desc *d, int sms, int num_kb, TcPlan *pl) {
     const int forced = force_bn ? atoi(force_bn) : 0;
     for (int ci = 0; ci < 3; ++ci) {
         const int b = cand[ci];
-        if (forced && b != forced) continue;
-        if (b > 32 && b / 2 >= round_up(d->M, 32)) continue;        // wider than the channels need
+        if (planes ? (b == 32 || (b == 256 && (d->w_bits > 2 || d->w_bits + d->a_bits > 4))) : (forced && b != forced)) continue;
+        if (b > (planes ? 128 : 32) && b / 2 >= round_up(d->M, 32)) continue;        // wider than the channels need
         const long long t = (long long)tiles_p * ceil_div(d->M, b);
-        const double main_loop = 640.0 * num_kb, epi = 2000.0 * (b >= 64 ? b / 64 : 1);
+        const double main_loop = (planes ? 1100.0 + 75.0 * (b / 32 * d->w_bits + TC_BP / 32 * d->a_bits) : 640.0) * num_kb, epi = (planes ? 4000.0 : 2000.0) * (b >= 64 ? b / 64 : 1);
         double cost;
         if (allowed && 2 * t <= sms && num_kb >= 4) {
             cost = 0.5 * main_loop + 1000.0 + epi;                   // every tile shared by a CTA pair
@@ -1648,6 +1852,55 @@ qnn_status gemm_tc_lower_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g,
     // shared memory is checked per instantiation (it depends on the number of thresholds)
     if (mode == 1) return launch_out<LW_BN, LW_STAGES, 1>(out_mode, g->out_bits, mw, mw, p, s);
     return launch_out<LW2_BN, LW2_STAGES, 2>(out_mode, g->out_bits, mw, mw, p, s);
+}
+
+// Bit-plane operands on the tensor cores: the tiled product (N too wide for the few-column kernels)
+// and, with cv, the convolution on a channels-last bit-plane map.  g: the (lowered) GEMM.
+qnn_status gemm_tc_planes_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *A,
+                                 const int32_t *thr, void *out, cudaStream_t s) {
+    TcParams p = {};
+    p.thr = thr; p.out = out; p.M = g->M; p.N = g->N; p.K = g->K;
+    p.pl_kw = ceil_div(g->K, 32);
+    p.num_kb = ceil_div(g->K, TC_BK);
+    p.ld_out = round_up(g->M, 16);
+    p.cchunks = 1; p.cv_C = p.cv_KW = p.cv_OW = p.cv_OHW = p.cv_stride = 1;
+    p.pl_W = (const uint32_t *)W; p.pl_A = (const uint32_t *)A;
+    p.pl_wb = g->w_bits; p.pl_ab = g->a_bits;
+    p.pl_wkind = plane_kind(g->w_enc); p.pl_akind = plane_kind(g->a_enc);
+    p.pl_wplane = (long long)g->M * p.pl_kw; p.pl_aplane = (long long)g->N * p.pl_kw;
+    if (cv) {
+        p.pl_conv = 1; p.pl_cw = ceil_div(cv->C, 32);
+        p.lw_H = cv->H; p.lw_W = cv->W; p.cv_KW = cv->KW; p.cv_stride = cv->stride; p.cv_pad = cv->pad;
+        p.cv_OW = qnn_conv_out_w(cv); p.cv_OHW = qnn_conv_out_h(cv) * p.cv_OW;
+        p.pl_aplane = (long long)cv->B * cv->H * cv->W * p.pl_cw;
+    }
+    TcPlan pl;
+    if (!tc_plan(g, sm_count(), p.num_kb, &pl, true)) return QNN_ERR_UNSUPPORTED;
+    p.tiles_p = pl.tiles_p; p.tiles_c = pl.tiles_c;
+    const int tiles = pl.tiles_p * pl.tiles_c;
+    p.units = p.full_units = tiles;
+    if (pl.share) {
+        p.share = 1;
+        p.full_units = tiles - pl.rem;
+        p.units = p.full_units + 2 * pl.rem;
+        p.kb_half = (p.num_kb + 1) / 2;
+    }
+    const double wmax = g->w_enc == QNN_ENC_BIPOLAR ? 1.0 : double(1 << g->w_bits);
+    const double amax = g->a_enc == QNN_ENC_BIPOLAR ? 1.0 : double(1 << g->a_bits);
+    p.fp_count = (double(g->K) * wmax * amax < double(FP_LIMIT)) ? 1 : 0;
+    p.idesc = (2u << 4) | ((g->a_enc == QNN_ENC_UNSIGNED ? 0u : 1u) << 7) | ((g->w_enc == QNN_ENC_UNSIGNED ? 0u : 1u) << 10) |
+              ((uint32_t)(pl.bn >> 3) << 17) | ((uint32_t)(TC_BP >> 4) << 24);
+    const int mode = !thr ? OUT_RAW : (g->out_fmt == QNN_FMT_INT8 ? OUT_U8 : OUT_PLANES);
+    const CUtensorMap none = {};                               // nothing is loaded through a tensor map
+    // Ring slots of four k-blocks where they fit beside the operand stages and the thresholds, else of
+    // two; 256-channel tiles only with up to two weight and four planes in all (other rings do not fit).
+    constexpr int STAGES_256 = 3, STAGES_128 = 4;
+    const size_t stages = pl.bn == 256 ? (size_t)STAGES_256 * (TC_BP + 256) * TC_BK : (size_t)STAGES_128 * (TC_BP + 128) * TC_BK;
+    const size_t used = stages + (size_t)2 * pl.bn * thr_slots(thr ? g->out_bits : 0) * 4 + 3072;
+    p.pl_kbs = used + pl_ring_bytes(p, pl.bn, 4) <= TC_SMEM_LIMIT ? 4 : 2;
+    p.pl_vec = (cv ? p.pl_cw : p.pl_kw) % 4 == 0 ? 1 : 0;
+    if (pl.bn == 256) return launch_out<256, STAGES_256, 3>(mode, g->out_bits, none, none, p, s);
+    return launch_out<128, STAGES_128, 3>(mode, g->out_bits, none, none, p, s);
 }
 
 #ifdef QNN_TC_TRACE
