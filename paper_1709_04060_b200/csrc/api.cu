@@ -101,11 +101,14 @@ static void conv_to_gemm(const qnn_conv_desc *d, qnn_gemm_desc *g) {
 // Bit planes with more columns than the few-column kernel takes go through the tensor cores, expanded
 // to bytes inside the kernel, unless the caller asks for the bit-serial path or leaves plane pairs
 // out.  Sixteen plane pairs (W4A4) up to 2^30 multiply-accumulates keep the AND/POPC kernel although
-// dense operands take longer there (1024^3: 156 us against 15): that a call gets faster with
+// dense operands take longer there (1024^3: 156 us against 20): that a call gets faster with
 // skip_planes and with empty plane tiles is what this format promises at these sizes.
 static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
     if (d->path != QNN_PATH_AUTO || d->skip_planes != 0) return false;
-    return d->w_bits * d->a_bits < 16 || (double)d->M * d->N * d->K > double(1 << 30);
+    const double macs = (double)d->M * d->N * d->K;
+    // a single plane pair at middle sizes (512^3: 7.6 us against 10.9; 1024^3: 16.0 against 13.5)
+    if (d->w_bits * d->a_bits == 1 && macs > double(1 << 24) && macs <= double(1 << 27)) return false;
+    return d->w_bits * d->a_bits < 16 || macs > double(1 << 30);
 }
 
 }  // namespace qnn

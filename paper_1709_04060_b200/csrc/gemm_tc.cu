@@ -117,7 +117,7 @@ struct TcParams {
     long long pl_wplane, pl_aplane;    // words per plane of the two operands
     int pl_wb, pl_ab, pl_wkind, pl_akind, pl_kw;    // planes, PL_* kinds, depth words per row
     int pl_conv, pl_cw;                // 1: implicit convolution; words per pixel
-    int pl_kbs, pl_vec;                // k-blocks per ring slot (2 or 4); 1: copies of 16 bytes
+    int pl_kbs, pl_mode;               // k-blocks per ring slot (2 or 4); copies of 0: words, 1: 16 bytes, 2: the 16-byte units rows lie in
     // CTA-pair kernel with a split last round (see qgemm_tc2_kernel): the depth of each of the last
     // split_rem tiles is shared by two neighbouring CTA pairs, which exchange int32 partial sums
     // through global memory.
@@ -540,17 +540,24 @@ constexpr int PL_WARPS = 4;        // expanding warps of the LOWER == 3 kernels,
 // ROWS words of this thread (rows 8 PL_WARPS apart) into an operand tile.  src: shared-memory address
 // of the first row's word in the first plane, rows and planes that many bytes apart; piece0, piece1:
 // the two 16-byte pieces of the first row, already swizzled (the later rows' swizzle is the same).
+// shift: words by which each plane's rows are off; live: 0 past the end of the rows.
 template <int ROWS, int B, int KIND>
-__device__ __forceinline__ void expand_rows(uint32_t src, uint32_t row_step, uint32_t plane_step, uint32_t keep, uint32_t piece0, uint32_t piece1) {
-    uint32_t w[ROWS][B];
+__device__ __forceinline__ void expand_rows(uint32_t src, uint32_t row_step, uint32_t plane_step, const uint32_t (&shift)[4], uint32_t live, uint32_t keep, uint32_t piece0, uint32_t piece1) {
+    // two rows at a time, not unrolled further: the expanding warps run this code over and over, and
+    // the shorter it is the less they wait for instructions
+#pragma unroll 1
+    for (int i0 = 0; i0 < ROWS; i0 += 2, src += 2 * row_step, piece0 += 2 * 8 * PL_WARPS * TC_BK, piece1 += 2 * 8 * PL_WARPS * TC_BK) {
+    uint32_t w[2][B];
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int b = 0; b < B; ++b)
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w[i][b]) : "r"(src + (uint32_t)i * row_step + (uint32_t)b * plane_step));
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w[i][b]) : "r"(src + (uint32_t)i * row_step + (uint32_t)b * plane_step + 4u * shift[b]));
 #pragma unroll
-    for (int i = 0; i < ROWS; ++i) {
+    for (int i = 0; i < 2; ++i) {
         uint32_t o[8];
+#pragma unroll
+        for (int b = 0; b < B; ++b) w[i][b] &= live;
         expand_word<B, KIND>(w[i], o);
         if (KIND == PL_BIPOLAR && keep != 0xFFFFFFFFu) {
 #pragma unroll
@@ -561,15 +568,17 @@ __device__ __forceinline__ void expand_rows(uint32_t src, uint32_t row_step, uin
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
                      ::"r"(piece1 + (uint32_t)(i * 8 * PL_WARPS * TC_BK)), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
     }
+    }
 }
 template <int ROWS>
-__device__ __forceinline__ void expand_rows_of(int planes, int kind, uint32_t src, uint32_t row_step, uint32_t plane_step, uint32_t keep,
+__device__ __forceinline__ void expand_rows_of(int planes, int kind, uint32_t src, uint32_t row_step, uint32_t plane_step,
+                                               const uint32_t (&shift)[4], uint32_t live, uint32_t keep,
                                                uint32_t piece0, uint32_t piece1) {
-    if (kind == PL_BIPOLAR) { expand_rows<ROWS, 1, PL_BIPOLAR>(src, row_step, plane_step, keep, piece0, piece1); return; }
+    if (kind == PL_BIPOLAR) { expand_rows<ROWS, 1, PL_BIPOLAR>(src, row_step, plane_step, shift, live, keep, piece0, piece1); return; }
 #define QNN_PL_CASE(B_)                                                                                                \
     case B_:                                                                                                           \
-        if (kind == PL_SIGNED) expand_rows<ROWS, B_, PL_SIGNED>(src, row_step, plane_step, keep, piece0, piece1);      \
-        else expand_rows<ROWS, B_, PL_UNSIGNED>(src, row_step, plane_step, keep, piece0, piece1);                      \
+        if (kind == PL_SIGNED) expand_rows<ROWS, B_, PL_SIGNED>(src, row_step, plane_step, shift, live, keep, piece0, piece1);      \
+        else expand_rows<ROWS, B_, PL_UNSIGNED>(src, row_step, plane_step, shift, live, keep, piece0, piece1);                      \
         break;
     switch (planes) { QNN_PL_CASE(1) QNN_PL_CASE(2) QNN_PL_CASE(3) QNN_PL_CASE(4) }
 #undef QNN_PL_CASE
@@ -584,13 +593,16 @@ __device__ __forceinline__ void copy_words(uint32_t dst, const uint32_t *src, bo
 // Ring of plane words of a LOWER == 3 kernel: two slots of pl_kbs k-blocks (2 or 4), each
 // [weight plane][row], [activation plane][row] with 4 pl_kbs words a row; the 16-byte units of a row
 // (one k-block each) are swizzled by its index, so that the eight rows a warp expands at a time fall
-// into different banks.
+// into different banks.  Rows of a matrix that are not whole 16-byte units are copied in the units
+// they lie in, one more per row (shifted: the odd number of units a row spreads the banks).
 struct PlRing {
     uint32_t row_b, w_plane, a_plane, a_off, slot_b, umask, ushift;
+    bool shifted;
     __device__ __forceinline__ PlRing(const TcParams &p, int bn) {
-        row_b = 16u * (uint32_t)p.pl_kbs; w_plane = (uint32_t)bn * row_b; a_plane = TC_BP * row_b;
+        shifted = p.pl_mode == 2;
+        row_b = 16u * (uint32_t)(p.pl_kbs + (shifted ? 1 : 0)); w_plane = (uint32_t)bn * row_b; a_plane = TC_BP * row_b;
         a_off = (uint32_t)p.pl_wb * w_plane; slot_b = a_off + (uint32_t)p.pl_ab * a_plane;
-        umask = (uint32_t)p.pl_kbs - 1u; ushift = p.pl_kbs == 4 ? 1u : 2u;
+        umask = shifted ? 0u : (uint32_t)p.pl_kbs - 1u; ushift = p.pl_kbs == 4 ? 1u : 2u;
     }
     __device__ __forceinline__ uint32_t unit(uint32_t u, uint32_t row) const { return (u ^ ((row >> ushift) & umask)) << 4; }
 };
@@ -664,13 +676,66 @@ __device__ __forceinline__ void load_planes_loop(const TcParams &p, Smem &sm, ui
     __syncwarp();
 }
 
+// The same for matrices whose rows are not whole 16-byte units: the units a row's words lie in.  Words
+// of neighbouring rows come along at both ends; those past the row's end meet activation words that
+// the expanding warps zero.
+template <int BN, typename Smem>
+__device__ __forceinline__ void load_shifted_loop(const TcParams &p, Smem &sm, uint32_t raw, int w, int lane, volatile int *abort_flag) {
+    const PlRing ring(p, BN);
+    const int upr = p.pl_kbs + 1;                                  // units per row: 3 or 5
+    const long long w_total = (long long)p.pl_wb * p.pl_wplane, a_total = (long long)p.pl_ab * p.pl_aplane;
+    uint32_t chunk = 0;
+    bool alive = true;
+    for (int u = blockIdx.x; alive && u < p.units; u += gridDim.x) {
+        const TcUnit un = tc_unit(p, u, BN);
+        for (int kb0 = un.kb0; kb0 < un.kb1; kb0 += p.pl_kbs, ++chunk) {
+            const uint32_t slot = chunk & 1, dst = raw + slot * ring.slot_b;
+            if (!(alive = warp_wait(&sm.in_empty[slot], ((chunk >> 1) & 1) ^ 1, lane, abort_flag))) break;
+            auto copy_rows = [&](const uint32_t *base, long long plane, long long total, int planes, int first, int limit, int rows, uint32_t at0,
+                                 uint32_t plane_b) {
+                const int n = (rows / 4) * upr;
+                for (int b = 0; b < planes; ++b) {
+#pragma unroll 2
+                    for (int i = lane; i < n; i += 32) {
+                        const int j = upr == 5 ? (i * 205) >> 10 : (i * 171) >> 9, k = i - j * upr;       // i / upr (i < 320)
+                        const int r = w * (rows / 4) + j;
+                        const long long at = ((b * plane + (long long)(first + r) * p.pl_kw + 4 * kb0) & ~3ll) + 4 * k;
+                        const bool ok = first + r < limit && at < total;
+                        const int bytes = ok ? 4 * (int)min(4ll, total - at) : 0;
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                                     ::"r"(dst + at0 + (uint32_t)b * plane_b + (uint32_t)r * ring.row_b + 16u * (uint32_t)k),
+                                       "l"(ok ? base + at : base), "r"(bytes) : "memory");
+                    }
+                }
+            };
+            copy_rows(p.pl_W, p.pl_wplane, w_total, p.pl_wb, un.c0, p.M, BN, 0u, ring.w_plane);
+            copy_rows(p.pl_A, p.pl_aplane, a_total, p.pl_ab, un.p0, p.N, TC_BP, ring.a_off, ring.a_plane);
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sm.in_full[slot])) : "memory");
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+}
+
 // Expanding warps: lane l of warp w turns word l & 3 of a k-block, rows 8 w + l / 4 + 32 i, into bytes.
 // The 16-byte stores of eight lanes (two rows, the swizzle shifts them by one piece) fall into
-// different banks.
+// different banks.  Every lane polls the barriers itself: these warps' serial time is what bounds the
+// kernel, and electing a lane and broadcasting its answer costs them twice as much.
+__device__ __forceinline__ bool lanes_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
 template <int BN, int STAGES, typename Smem>
 __device__ __forceinline__ void expand_loop(const TcParams &p, Smem &sm, uint32_t raw, int w, int lane, volatile int *abort_flag) {
     constexpr int RS = 8 * PL_WARPS, WR = BN / RS, AR = TC_BP / RS;
     const PlRing ring(p, BN);
+    // words before each plane's row in its first copied unit (rows of an operand that are not whole units)
+    uint32_t w_sh[4], a_sh[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const uint32_t r = (8 * w + (lane >> 2)) * (uint32_t)p.pl_kw;
+        w_sh[b] = ring.shifted ? (r + (uint32_t)b * (uint32_t)p.pl_wplane) & 3u : 0u;
+        a_sh[b] = ring.shifted ? (r + (uint32_t)b * (uint32_t)p.pl_aplane) & 3u : 0u;
+    }
     const uint32_t c = lane & 3, r0 = 8 * w + (lane >> 2), x = r0 & 7;
     const uint32_t off0 = r0 * TC_BK + (((2 * c) ^ x) << 4), off1 = r0 * TC_BK + (((2 * c + 1) ^ x) << 4);
     uint32_t it = 0, chunk = 0;
@@ -678,19 +743,19 @@ __device__ __forceinline__ void expand_loop(const TcParams &p, Smem &sm, uint32_
         const TcUnit un = tc_unit(p, u, BN);
         for (int kb0 = un.kb0; kb0 < un.kb1; kb0 += p.pl_kbs, ++chunk) {
             const uint32_t slot = chunk & 1;
-            if (!warp_wait(&sm.in_full[slot], (chunk >> 1) & 1, lane, abort_flag)) return;
+            if (!lanes_wait(&sm.in_full[slot], (chunk >> 1) & 1, abort_flag)) return;
             const int kb1 = min(kb0 + p.pl_kbs, un.kb1);
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
                 const int s = it % STAGES;
                 const uint32_t ph = (it / STAGES) & 1;
-                if (!warp_wait(&sm.empty[s], ph ^ 1, lane, abort_flag)) return;
+                if (!lanes_wait(&sm.empty[s], ph ^ 1, abort_flag)) return;
                 const uint32_t wt = smem_u32(sm.wgt[s]), at = smem_u32(sm.act[s]);
                 const uint32_t src = raw + slot * ring.slot_b + r0 * ring.row_b + ring.unit((uint32_t)(kb - kb0), r0) + 4u * c;
-                expand_rows_of<WR>(p.pl_wb, p.pl_wkind, src, RS * ring.row_b, ring.w_plane, 0xFFFFFFFFu, wt + off0, wt + off1);
+                expand_rows_of<WR>(p.pl_wb, p.pl_wkind, src, RS * ring.row_b, ring.w_plane, w_sh, 0xFFFFFFFFu, 0xFFFFFFFFu, wt + off0, wt + off1);
                 // +-1 has no zero: activation elements past the end of the depth have to become zero bytes
                 const int left = p.K - 32 * (kb * 4 + (int)c);
                 const uint32_t keep = left >= 32 ? 0xFFFFFFFFu : (left <= 0 ? 0u : (1u << left) - 1u);
-                expand_rows_of<AR>(p.pl_ab, p.pl_akind, src + ring.a_off, RS * ring.row_b, ring.a_plane, keep, at + off0, at + off1);
+                expand_rows_of<AR>(p.pl_ab, p.pl_akind, src + ring.a_off, RS * ring.row_b, ring.a_plane, a_sh, kb * 4 + (int)c < p.pl_kw ? 0xFFFFFFFFu : 0u, keep, at + off0, at + off1);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core's reads
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.full[s]);
@@ -830,7 +895,8 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_consta
         __syncwarp();
     } else if (LOWER == 3 && warp > STAGER_WARP) {
         if constexpr (LOWER == 3) {
-            if (p.pl_vec) load_planes_loop<BN, 4>(p, sm, smem_u32(w_extra), warp - (STAGER_WARP + 1), lane, abort_flag);
+            if (p.pl_mode == 2) load_shifted_loop<BN>(p, sm, smem_u32(w_extra), warp - (STAGER_WARP + 1), lane, abort_flag);
+            else if (p.pl_mode == 1) load_planes_loop<BN, 4>(p, sm, smem_u32(w_extra), warp - (STAGER_WARP + 1), lane, abort_flag);
             else load_planes_loop<BN, 1>(p, sm, smem_u32(w_extra), warp - (STAGER_WARP + 1), lane, abort_flag);
         }
     } else if (LOWER == 3 && warp >= 2 + EPI_WARPS / 2 && warp < STAGER_WARP) {
@@ -1040,15 +1106,24 @@ qgemm_tc_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_consta
         for (int u = blockIdx.x; u < p.units; u += gridDim.x, ++tcount) {
             const TcUnit un = tc_unit(p, u, BN);
             const uint32_t buf = tcount & 1, acc_ph = (tcount >> 1) & 1;
-            // with bit planes a warp also takes the part of the warp four further on
-            bool ok = true;
-            for (int e = warp; ok && e <= (LOWER == 3 ? warp + EPI_WARPS / 2 : warp); e += EPI_WARPS / 2) {
-                ok = epilogue_tile<OUT_MODE, OUT_BITS>(p, sm.thr[buf], &sm.thr_full[buf], &sm.thr_empty[buf], acc_ph,
+            const auto part = [&](int e) -> bool {
+                if (!epilogue_tile<OUT_MODE, OUT_BITS>(p, sm.thr[buf], &sm.thr_full[buf], &sm.thr_empty[buf], acc_ph,
                                                        &sm.tmem_full[buf], acc_ph, tmem_base + buf * BN, BN,
-                                                       un.p0, un.c0, un.shared, xc, e, lane, abort_flag, (int)tcount);
-                if (ok && lane == 0) mbar_arrive(&sm.tmem_empty[buf]);     // one arrival per warp's part
+                                                       un.p0, un.c0, un.shared, xc, e, lane, abort_flag, (int)tcount))
+                    return false;
+                if (lane == 0) mbar_arrive(&sm.tmem_empty[buf]);     // one arrival per warp's part
+                return true;
+            };
+            if constexpr (LOWER == 3) {
+                // four epilogue warps: two parts each, one copy of the code (a launch that runs a tile
+                // or two per SM waits for every instruction line it fetches)
+                bool ok = true;
+#pragma unroll 1
+                for (int e = warp; ok && e < warp + EPI_WARPS; e += EPI_WARPS / 2) ok = part(e);
+                if (!ok) break;
+            } else if (!part(warp)) {
+                break;
             }
-            if (!ok) break;
         }
     }
 
@@ -1467,7 +1542,7 @@ constexpr size_t TC_SMEM_LIMIT = 227 * 1024;
 
 // The ring of plane words of a LOWER == 3 kernel: two slots of kbs k-blocks of both operands.
 static size_t pl_ring_bytes(const TcParams &p, int bn, int kbs) {
-    return (size_t)2 * kbs * 16 * (bn * p.pl_wb + TC_BP * p.pl_ab);
+    return (size_t)2 * (kbs + (p.pl_mode == 2 ? 1 : 0)) * 16 * (bn * p.pl_wb + TC_BP * p.pl_ab);
 }
 
 template <int BN, int STAGES, int OUT_MODE, int OUT_BITS, int LOWER = 0>
@@ -1893,12 +1968,13 @@ qnn_status gemm_tc_planes_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g
     const int mode = !thr ? OUT_RAW : (g->out_fmt == QNN_FMT_INT8 ? OUT_U8 : OUT_PLANES);
     const CUtensorMap none = {};                               // nothing is loaded through a tensor map
     // Ring slots of four k-blocks where they fit beside the operand stages and the thresholds, else of
-    // two; 256-channel tiles only with up to two weight and four planes in all (other rings do not fit).
+    // two (word by word, without the extra units, where even those do not fit); 256-channel tiles only with up to two weight and four planes in all (other rings do not fit).
     constexpr int STAGES_256 = 3, STAGES_128 = 4;
     const size_t stages = pl.bn == 256 ? (size_t)STAGES_256 * (TC_BP + 256) * TC_BK : (size_t)STAGES_128 * (TC_BP + 128) * TC_BK;
     const size_t used = stages + (size_t)2 * pl.bn * thr_slots(thr ? g->out_bits : 0) * 4 + 3072;
+    p.pl_mode = (cv ? p.pl_cw : p.pl_kw) % 4 == 0 ? 1 : (cv ? 0 : 2);
+    if (p.pl_mode == 2 && used + pl_ring_bytes(p, pl.bn, 2) > TC_SMEM_LIMIT) p.pl_mode = 0;
     p.pl_kbs = used + pl_ring_bytes(p, pl.bn, 4) <= TC_SMEM_LIMIT ? 4 : 2;
-    p.pl_vec = (cv ? p.pl_cw : p.pl_kw) % 4 == 0 ? 1 : 0;
     if (pl.bn == 256) return launch_out<256, STAGES_256, 3>(mode, g->out_bits, none, none, p, s);
     return launch_out<128, STAGES_128, 3>(mode, g->out_bits, none, none, p, s);
 }
