@@ -111,6 +111,34 @@ static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
     return d->w_bits * d->a_bits < 16 || macs > double(1 << 30);
 }
 
+// Convolution on bit planes by way of 8-bit containers: the map and the filters are widened into the
+// workspace, which has room for them wherever a lowered matrix would be several times the map, and the
+// 8-bit convolution kernels run on that.  Expanding inside the GEMM kernel instead repeats the work
+// for every filter tap of the map and every pixel tile of the filters, and pays only where the extra
+// launch weighs more (27 x 27 x 96 -> 256, 5 x 5, W1A2 at batch 8: 15 us this way, 38 in the kernel).
+constexpr double WIDEN_MIN_MACS = double(1 << 28);
+static qnn_status widened_conv_launch(const qnn_conv_desc *d, const qnn_gemm_desc *g, const void *Wp, const void *in,
+                                      const int32_t *thr, void *out, void *ws, size_t ws_bytes, cudaStream_t s) {
+    const int Cp = round_up(d->C, 16);
+    const long long pixels = (long long)d->B * d->H * d->W, taps = (long long)d->OC * d->KH * d->KW;
+    if (pixels * Cp > 0x7fffffffffffll || taps > 0x7fffffffll || pixels > 0x7fffffffll) return QNN_ERR_UNSUPPORTED;
+    const size_t map_bytes = ((size_t)pixels * Cp + 255) / 256 * 256, w_bytes = (size_t)taps * Cp;
+    if (map_bytes + w_bytes > ws_bytes || (double)g->M * g->N * g->K < WIDEN_MIN_MACS) return QNN_ERR_UNSUPPORTED;
+    qnn_conv_desc c = *d;
+    c.C = Cp; c.in_pitch = Cp; c.fmt = QNN_FMT_INT8;
+    qnn_gemm_desc cg = *g;
+    cg.K = qnn_conv_lowered_k(&c); cg.w_fmt = cg.a_fmt = QNN_FMT_INT8;
+    // a pixel's words widen to one row of Cp bytes, and so do a filter tap's
+    const qnn_pack_desc pm = {(int)pixels, d->C, d->a_bits, d->a_enc, QNN_FMT_BITPLANES};
+    const qnn_pack_desc pw = {(int)taps, d->C, d->w_bits, d->w_enc, QNN_FMT_BITPLANES};
+    uint8_t *map = reinterpret_cast<uint8_t *>(ws), *filters = map + map_bytes;
+    if (!gemm_tc_conv_takes(&c)) return QNN_ERR_UNSUPPORTED;
+    qnn_status st = planes_to_int8_launch(&pm, in, map, s, &pw, Wp, filters);
+    if (st == QNN_OK) st = gemm_tc_lower_launch(&c, &cg, filters, map, thr, out, s);
+    if (st == QNN_ERR_UNSUPPORTED) st = gemm_tc_conv_launch(&c, &cg, filters, map, thr, out, true, s);
+    return st;
+}
+
 }  // namespace qnn
 
 using namespace qnn;
@@ -293,13 +321,15 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
         // channels: the first layer) or would waste k-blocks (channel count not a multiple of 128)
         st = gemm_tc_lower_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
         if (st != QNN_ERR_UNSUPPORTED) return st;
-        st = gemm_tc_conv_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
+        st = gemm_tc_conv_launch(d, &g, Wpacked, in, thr, out, false, (cudaStream_t)stream);
         if (st != QNN_ERR_UNSUPPORTED) return st;
     }
     // bit-plane maps on the tiled bit-serial kernel: its staging code lowers on the fly (a handful
     // of output pixels goes through the lowered matrix and the few-column kernel instead)
     if (path == QNN_PATH_BITSERIAL && !(explicit_env && explicit_env[0] == '1') && !gemv_planes_fits(&g)) {
         if (planes_on_tensor_cores(&g)) {
+            st = widened_conv_launch(d, &g, Wpacked, in, thr, out, workspace, workspace_bytes, (cudaStream_t)stream);
+            if (st != QNN_ERR_UNSUPPORTED) return st;
             st = gemm_tc_planes_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
             if (st != QNN_ERR_UNSUPPORTED) return st;
         }

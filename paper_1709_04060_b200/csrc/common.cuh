@@ -61,7 +61,8 @@ int sm_count();
 
 // Path implementations (one translation unit each).
 qnn_status pack_launch(const qnn_pack_desc *d, const void *logical, void *packed, cudaStream_t s);
-qnn_status planes_to_int8_launch(const qnn_pack_desc *d, const void *planes, void *packed, cudaStream_t s);
+qnn_status planes_to_int8_launch(const qnn_pack_desc *d, const void *planes, void *packed, cudaStream_t s,
+                                 const qnn_pack_desc *d2 = nullptr, const void *planes2 = nullptr, void *packed2 = nullptr);
 qnn_status gemm_bitserial_launch(const qnn_gemm_desc *d, const void *W, const void *A,
                                  const int32_t *thr, void *out, cudaStream_t s);
 qnn_status gemm_bitserial_conv_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W,
@@ -83,7 +84,8 @@ qnn_status gemm_tc_launch(const qnn_gemm_desc *d, const void *W, const void *A,
 size_t gemm_tc_workspace_bytes(const qnn_gemm_desc *d);   // optional scratch of the CTA-pair kernel (0: none)
 bool gemm_tc_uses_pair_kernel(const qnn_gemm_desc *d);
 qnn_status gemm_tc_conv_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
-                               const int32_t *thr, void *out, cudaStream_t s);
+                               const int32_t *thr, void *out, bool any_size, cudaStream_t s);
+bool gemm_tc_conv_takes(const qnn_conv_desc *cv);       // what the tensor-map loader can lower
 qnn_status gemm_tc_lower_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
                                 const int32_t *thr, void *out, cudaStream_t s);
 qnn_status gemm_tc_planes_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *A,

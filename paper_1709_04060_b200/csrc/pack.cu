@@ -74,39 +74,50 @@ __device__ __forceinline__ uint32_t container4(uint32_t x, int bits, int enc) {
     return low | ((sign << 1) * ((1u << (8 - bits)) - 1u));
 }
 
-// Bit planes -> 8-bit containers: one thread per 16 output bytes (16 consecutive depth indices,
-// one half of a plane word).  Four bits of a plane become four bytes by one multiplication
-// (bit b of the nibble lands in bit 0 of byte b); plane i adds them shifted by i.
-__global__ void __launch_bounds__(256) planes_to_int8_kernel(const uint32_t *__restrict__ planes,
-                                                             uint4 *__restrict__ packed, int rows, int K,
-                                                             int kw, int chunks, int bits, int enc) {
-    const long long total = (long long)rows * chunks;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(idx / chunks), c = (int)(idx - (long long)r * chunks);
-        const int k0 = 16 * c, word = k0 >> 5, shift = k0 & 31;
-        uint32_t o[4] = {0u, 0u, 0u, 0u};
-        for (int i = 0; i < bits; ++i) {
-            const uint32_t x = (planes[((size_t)i * rows + r) * kw + word] >> shift) & 0xFFFFu;
+// Bit planes -> 8-bit containers: one thread per plane word, i.e. 32 consecutive depth indices and two
+// 16-byte stores (one where the row ends in the word's first half).  Four bits of a plane become four
+// bytes by one multiplication (bit b of the nibble lands in bit 0 of byte b); plane i adds them shifted
+// by i.  One launch widens one operand, or two (the map and the filters of a convolution).
+struct WidenOp {
+    const uint32_t *planes;
+    uint4 *packed;
+    long long words;           // rows * kw
+    int K, kw, chunks, bits, enc;
+};
+__device__ __forceinline__ void widen_word(const WidenOp &p, long long idx) {
+    long long r;
+    if (p.words <= 0x7fffffffll) r = (unsigned)idx / (unsigned)p.kw; else r = idx / p.kw;
+    const int c = (int)(idx - r * p.kw), k0 = 32 * c;
+    uint32_t o[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t spread = (((x >> (4 * q)) & 0xFu) * 0x00204081u) & 0x01010101u;
-                // SIGNED: the top plane is the sign, which also fills the container's upper bits
-                const uint32_t mul = (enc == QNN_ENC_SIGNED && i == bits - 1) ? ((0xFFu << i) & 0xFFu) : (1u << i);
-                o[q] |= spread * mul;
-            }
-        }
-        if (enc == QNN_ENC_BIPOLAR) {
-            // bit 1 -> +1, bit 0 -> -1; pad bytes past K stay zero
+    for (int q = 0; q < 8; ++q) o[q] = 0u;
+#pragma unroll 4
+    for (int i = 0; i < p.bits; ++i) {
+        const uint32_t x = __ldg(p.planes + i * p.words + idx);
+        // SIGNED: the top plane is the sign, which also fills the container's upper bits
+        const uint32_t mul = (p.enc == QNN_ENC_SIGNED && i == p.bits - 1) ? ((0xFFu << i) & 0xFFu) : (1u << i);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t v = 0xFFFFFFFFu ^ (o[q] * 0xFEu);
-                const int left = K - (k0 + 4 * q);                 // elements of this word inside the row
-                if (left < 4) v &= left <= 0 ? 0u : (0xFFFFFFFFu >> (8 * (4 - left)));
-                o[q] = v;
-            }
+        for (int q = 0; q < 8; ++q) o[q] |= ((((x >> (4 * q)) & 0xFu) * 0x00204081u) & 0x01010101u) * mul;
+    }
+    if (p.enc == QNN_ENC_BIPOLAR) {
+        // bit 1 -> +1, bit 0 -> -1; pad bytes past K stay zero
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            uint32_t v = 0xFFFFFFFFu ^ (o[q] * 0xFEu);
+            const int left = p.K - (k0 + 4 * q);                   // elements of this register inside the row
+            if (left < 4) v &= left <= 0 ? 0u : (0xFFFFFFFFu >> (8 * (4 - left)));
+            o[q] = v;
         }
-        packed[idx] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    uint4 *dst = p.packed + r * p.chunks + 2 * c;
+    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    if (2 * c + 1 < p.chunks) dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+}
+__global__ void __launch_bounds__(256) planes_to_int8_kernel(const WidenOp a, const WidenOp b) {
+    pdl_trigger();        // a tensor-core kernel queued behind may set up while this one drains
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.words + b.words; i += step) {
+        if (i < a.words) widen_word(a, i); else widen_word(b, i - a.words);
     }
 }
 
@@ -186,14 +197,21 @@ __global__ void pack_fields_kernel(const uint8_t *__restrict__ logical, uint32_t
     packed[idx] = word;
 }
 
-qnn_status planes_to_int8_launch(const qnn_pack_desc *d, const void *planes, void *packed, cudaStream_t s) {
+static WidenOp widen_op(const qnn_pack_desc *d, const void *planes, void *packed) {
+    WidenOp p = {};
+    if (!d) return p;
+    p.planes = (const uint32_t *)planes; p.packed = (uint4 *)packed;
+    p.K = d->K; p.kw = ceil_div(d->K, 32); p.chunks = round_up(d->K, 16) / 16;
+    p.words = (long long)d->rows * p.kw;
+    p.bits = d->enc == QNN_ENC_BIPOLAR ? 1 : d->bits; p.enc = d->enc;
+    return p;
+}
+qnn_status planes_to_int8_launch(const qnn_pack_desc *d, const void *planes, void *packed, cudaStream_t s,
+                                 const qnn_pack_desc *d2, const void *planes2, void *packed2) {
     const int threads = 256;
-    const int kw = ceil_div(d->K, 32), chunks = round_up(d->K, 16) / 16;
-    const long long total = (long long)d->rows * chunks;
-    const long long want = (total + threads - 1) / threads, cap = (long long)sm_count() * 16;
-    planes_to_int8_kernel<<<(unsigned)(want < cap ? want : cap), threads, 0, s>>>(
-        (const uint32_t *)planes, (uint4 *)packed, d->rows, d->K, kw, chunks,
-        d->enc == QNN_ENC_BIPOLAR ? 1 : d->bits, d->enc);
+    const WidenOp a = widen_op(d, planes, packed), b = widen_op(d2, planes2, packed2);
+    const long long want = (a.words + b.words + threads - 1) / threads, cap = (long long)sm_count() * 16;
+    planes_to_int8_kernel<<<(unsigned)(want < cap ? want : cap), threads, 0, s>>>(a, b);
     count_launch();
     return launch_status();
 }
