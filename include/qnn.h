@@ -36,7 +36,7 @@
  *   QNN_CONV_LOWER=1|0         qnn_qconv uses the aligned lowering warps wherever they
  *                              apply | never
  *   QNN_FIELDS_KERNEL=dp4a|tensor  packed (FIELDS) weights: byte dot products on the CUDA
- *                              cores for up to 16 columns | always the tensor-core form
+ *                              cores for up to 16 columns | always the tcgen05 form
  *
  * Operand formats
  *   QNN_FMT_BITPLANES  uint32 [bits][rows][kw], kw = ceil(K/32): plane i holds
@@ -186,18 +186,21 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A,
  * chosen per layer shape).  The operand format is the caller's choice; on this GPU 8-bit
  * containers on the tensor cores are faster than bit planes for every size from 64 to 4096 per
  * dimension and every (w, a), so AUTO never converts between formats, it picks by shape:
- *   INT8 operands       N <= 8: byte dot products, one warp per weight row;
+ *   INT8 operands       N <= 8: weights streamed once: byte dot products, one warp per weight row,
+ *                       or (three columns on, large weights) warp-level tensor-core products;
  *                       M >= 256, N >= 2048 and at least a round and a half of 256 x 256 tiles
  *                       on the SM pairs: the CTA-pair tensor-core kernel; else the one-CTA
  *                       tensor-core kernel
- *   BITPLANES operands  N <= 16: one warp per weight row over the planes; else tiled: the planes
+ *   BITPLANES operands  N <= 16: weights streamed once: one warp per weight row over the planes, or
+ *                       (two columns on, or many plane pairs) warp-level tensor-core products
+ *                       on the planes widened in registers; else tiled: the planes
  *                       are expanded to bytes inside the tensor-core kernel, or (QNN_PATH_BITSERIAL,
  *                       skip_planes, sixteen plane pairs up to 2^30 multiply-accumulates) the
  *                       AND/POPC kernel
- *   FIELDS weights      N <= 16 only: one or two columns: one warp per
- *                       packed weight row, an AND and a 4-way byte dot product per word and
- *                       field position; more columns: packed weights expanded inside a
- *                       tensor-core kernel
+ *   FIELDS weights      N <= 16 only: one column: one warp per packed weight row, an AND and a 4-way
+ *                       byte dot product per word and field position; more: packed weights widened
+ *                       in registers for warp-level tensor-core products, or (columns beyond an
+ *                       SM's shared memory) inside a tcgen05 kernel
  * Returns a qnn_kernel value, or the (negative) qnn_status qnn_qgemm would return.  Host only. */
 typedef enum {
     QNN_KERNEL_TENSOR = 1, QNN_KERNEL_TENSOR_CTA_PAIR = 2, QNN_KERNEL_BYTES_FEW_COLUMNS = 3,

@@ -233,14 +233,18 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
     if (!aligned16(W) || !aligned16(A) || !aligned16(out) || (thr && (reinterpret_cast<uintptr_t>(thr) & 3u)))
         return QNN_ERR_ALIGNMENT;
     if (d->w_fmt == QNN_FMT_FIELDS) {
-        // a few columns: byte dot products on the CUDA cores; more: the tensor-core form
+        const char *force = getenv("QNN_FIELDS_KERNEL");
+        if (!force && gemv_mma_takes(d)) return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
+        // one column: byte dot products on the CUDA cores; columns that do not fit an SM's shared
+        // memory: the tcgen05 form
         if (gemv_fields_dp4a_fits(d)) return gemv_fields_dp4a_launch(d, W, A, thr, out, (cudaStream_t)stream);
         return gemv_fields_launch(d, W, A, thr, out, (cudaStream_t)stream);
     }
     // 8-bit containers with a handful of columns and no path forced: byte dot products,
     // one warp per weight row (a tensor-core tile would be almost empty)
     if (d->path == QNN_PATH_AUTO && d->w_fmt == QNN_FMT_INT8 && gemv_i8_fits(d))
-        return gemv_i8_launch(d, W, A, thr, out, (cudaStream_t)stream);
+        return gemv_mma_takes(d) ? gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream)
+                                : gemv_i8_launch(d, W, A, thr, out, (cudaStream_t)stream);
     if (path == QNN_PATH_TCGEN05_I8) {
         // the workspace is optional (see the header): used only when given, large enough and aligned
         const bool ws_ok = workspace && aligned16(workspace);
@@ -248,7 +252,12 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
                               (cudaStream_t)stream);
     }
     // a handful of columns: stream the weight planes once, one warp per row
-    if (gemv_planes_fits(d)) return gemv_planes_launch(d, W, A, thr, out, (cudaStream_t)stream);
+    if (gemv_planes_fits(d)) {
+        // ... on the tensor cores, unless the caller asks for the bit-serial path or leaves pairs out
+        if (d->path == QNN_PATH_AUTO && d->skip_planes == 0 && gemv_mma_takes(d))
+            return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
+        return gemv_planes_launch(d, W, A, thr, out, (cudaStream_t)stream);
+    }
     if (planes_on_tensor_cores(d)) {
         st = gemm_tc_planes_launch(nullptr, d, W, A, thr, out, (cudaStream_t)stream);
         if (st != QNN_ERR_UNSUPPORTED) return st;

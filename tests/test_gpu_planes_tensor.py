@@ -1,5 +1,5 @@
 """Bit planes multiplied on the tensor cores: the tiled product expands both operands to bytes inside the
-kernel.  Every output against the CPU oracle, at the sizes where a
+kernel, the few-column product in registers.  Every output against the CPU oracle, at the sizes where a
 tile, a ring slot, a step of the depth or a row of 32 ends; and against the AND/POPC kernels, which a
 forced bit-serial path still runs."""
 import numpy as np
@@ -60,6 +60,26 @@ def test_tiled_planes_with_a_shared_last_round(qb, w_bits, w_enc, a_bits, a_enc)
     two CTAs: their partial sums pass through the operand rings, 512 bytes per channel."""
     case = synth.gemm_case(7100 + w_bits, 256, 150 * 128 - 5, 256 if w_bits < 3 else 520, w_bits, a_bits, w_enc, a_enc, out_bits=2)
     check(qb, case, PLANES, INT8)
+
+
+@pytest.mark.parametrize("fmt", [PLANES, FIELDS, INT8])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (31, 16, 100), (33, 8, 513), (700, 9, 2048), (96, 3, 4096), (4800, 2, 300),
+                                   (65, 5, 8192), (64, 7, 9216), (40, 16, 9300), (50, 2, 70000)])
+def test_few_columns(qb, M, N, K, fmt):
+    """Tiles of 32 rows and steps of the depth that end early, one tile and several per CTA, loads of
+    one, two and four words, depths past what the columns' shared memory holds (other kernels)."""
+    if fmt == FIELDS and K == 70000:
+        pytest.skip("packed fields refuse this depth")
+    kinds = ENCODINGS if fmt == PLANES else [(w, we, a, ae) for (w, we, a, ae) in ENCODINGS if not (we == B and ae == B)]
+    for i, (w_bits, w_enc, a_bits, a_enc) in enumerate(kinds if M * K < 300000 else kinds[i0(M, K)::5]):
+        case = synth.gemm_case(7200 + M + N + K + i, M, N, K, w_bits, a_bits, w_enc, a_enc, out_bits=1 + (i + M) % 4)
+        check(qb, case, fmt, INT8)
+        check(qb, case, fmt, PLANES)
+        check(qb, case, fmt, INT8, raw=True)
+
+
+def i0(M, K):
+    return (M + K) % 5
 
 
 @pytest.mark.parametrize("N", [3, 40])
