@@ -135,18 +135,29 @@ def check(status: int) -> None:
 def _ptr(x):
     if x is None:
         return None
-    if isinstance(x, int):
-        return x
-    if isinstance(x, torch.Tensor):
+    if isinstance(x, _Tensor):
         assert x.is_contiguous(), "device buffers must be contiguous"
         return x.data_ptr()
+    if isinstance(x, int):
+        return x
     raise TypeError(type(x))
+
+
+_Tensor = torch.Tensor
+# The current stream's handle without building a torch.cuda.Stream around it (0.2 us
+# instead of 3.5 us a call).
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 def _stream(stream):
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        if not _initialized():
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_device())
     return int(stream)
+
+
+_initialized = torch.cuda.is_initialized
 
 
 # ---- one-to-one entry points -------------------------------------------------

@@ -282,8 +282,14 @@ qnn_status gemv_fields_dp4a_launch(const qnn_gemm_desc *d, const void *W, const 
     }
     // a persistent grid: as many CTAs as are resident at once, each staging its columns once and
     // then taking row blocks in turn
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, FD_THREADS, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    // (the occupancy query costs the host 2 us; its answer depends on the kernel and its shared memory)
+    static std::atomic<unsigned long long> occupancy[18][QNN_MAX_DEVICES];      // smem << 8 | CTAs per SM
+    const unsigned long long known = occupancy[fi][dev].load(std::memory_order_relaxed);
+    int per_sm = (int)(known & 0xFFu);
+    if (known == 0 || (known >> 8) != smem) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, FD_THREADS, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+        occupancy[fi][dev].store((unsigned long long)smem << 8 | (unsigned)per_sm, std::memory_order_relaxed);
+    }
     const int row_blocks = ceil_div(ceil_div(d->M, FD_THREADS / 32), fd_rows_at_a_time(F, nc));
     const int max_blocks = sm_count() * per_sm;
     dim3 grid(row_blocks < max_blocks ? row_blocks : max_blocks, ceil_div(d->N, nc));
