@@ -19,6 +19,10 @@
 // kernels with fewer than four plane pairs do not look (the bookkeeping costs 1-2 % of a dense
 // product with 4 to 16 pairs, but 6 % of one with two).
 //
+// The library's own choice takes this kernel for W4A4 up to 2^30 multiply-accumulates, for a single plane
+// pair at middle sizes and where plane pairs are left out; elsewhere the planes are expanded to bytes
+// for the tensor cores (gemm_tc.cu), which at 4096^3 W2A2 take 169 us against 1900 here.
+//
 // Tiling: one CTA (8 warps) per 64 x 64 output tile, depth staged 16 words at a
 // time.  Lanes run along the output-channel dimension (rows m0+lane, m0+32+lane)
 // so that (a) weight words are read conflict-free from a 17-word-pitch tile while

@@ -24,6 +24,8 @@
 //   warp 10    threshold stager: loads the thresholds of the next work unit's
 //              channels, sorts each channel's set (the count does not depend on
 //              their order) and writes them to one of two shared-memory buffers
+// (kernels that lower or expand their operands have four more warps, 480 threads; with bit
+// planes warps 2-5 are the epilogue, 6-9 expand and 11-14 load plane words)
 // Two accumulator buffers in tensor memory let the epilogue of tile t overlap the
 // main loop of tile t+1.  Every wait is bounded; on expiry the CTA records
 // QNN_ERR_DEVICE_TIMEOUT in the device status word, drains and exits.

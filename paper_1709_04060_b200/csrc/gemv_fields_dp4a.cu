@@ -17,9 +17,9 @@
 // Against the tensor-core form of the same product (gemv_fields.cu) this kernel has no serial
 // per-SM pipeline to fill, but every further column adds its shared-memory reads and dot products
 // to each warp's dependent chain (about 4 us per column at 8192 x 8192; the counters show load
-// latency, global and shared, not a saturated pipe), so it is the faster one for one column
-// (7.0 / 9.4 us against 12.5 / 14.7 us at 8192 x 8192 with 2- / 4-bit fields) and for two
-// (11.2 / 11.7 us against 12.7 / 15.0 us).
+// latency, global and shared, not a saturated pipe), so the library takes it for
+// one column (6.2 / 9.4 us against 12.5 / 14.7 us at 8192 x 8192 with 2- / 4-bit fields, and 7.8 / 11.3 us
+// in gemv_mma.cu, which takes over at two).
 #include <stdlib.h>
 
 #include "common.cuh"

@@ -9,7 +9,8 @@
 // One warp per weight row: lanes stride over the depth words, partial sums meet in
 // a shuffle reduction, then lane n counts the thresholds of column n (Section 2.1.1).
 // Columns are handled four at a time (blockIdx.y); more than four columns re-read
-// the weights from L2.
+// the weights from L2.  The library takes this kernel for one column and fewer than twelve plane pairs,
+// on the forced bit-serial path, and where plane pairs are left out; else gemv_mma.cu.
 #include "common.cuh"
 
 namespace qnn {
