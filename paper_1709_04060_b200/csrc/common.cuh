@@ -56,6 +56,21 @@ __device__ __forceinline__ void pdl_enter() {
 }
 #endif
 
+#ifdef __CUDACC__
+// Launch with programmatic stream serialization (see above): the launch gap overlaps the tail of the
+// kernel ahead.  For kernels that wait in griddepcontrol.wait before they touch global memory.
+template <typename Params>
+inline cudaError_t launch_pdl(void (*kern)(const Params), dim3 grid, int threads, size_t smem, cudaStream_t s, const Params &p) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
+#endif
+
 // Number of SMs of the current device (cached per device).
 int sm_count();
 
