@@ -183,10 +183,12 @@ __global__ void gemv_clear_kernel(uint32_t *out, long long words) {
         out[i] = 0u;
 }
 
+// Programmatic dependent launch: the kernel ahead releases its dependents at its end, so the CTAs
+// spread over all SMs (8192 x 8192 W1A2, one column, call after call: 8.1 -> 6.1 us).
 template <int WB, int AB, int MODE>
 static void gv_launch_one(const GvParams &p, dim3 grid, size_t smem, cudaStream_t s) {
-    if ((p.kw & 3) == 0) gemv_planes_kernel<WB, AB, MODE, true><<<grid, GV_THREADS, smem, s>>>(p);
-    else gemv_planes_kernel<WB, AB, MODE, false><<<grid, GV_THREADS, smem, s>>>(p);
+    if ((p.kw & 3) == 0) launch_pdl(gemv_planes_kernel<WB, AB, MODE, true>, grid, GV_THREADS, smem, s, p);
+    else launch_pdl(gemv_planes_kernel<WB, AB, MODE, false>, grid, GV_THREADS, smem, s, p);
 }
 
 template <int MODE>
