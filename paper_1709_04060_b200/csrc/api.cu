@@ -234,7 +234,7 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
         return QNN_ERR_ALIGNMENT;
     if (d->w_fmt == QNN_FMT_FIELDS) {
         const char *force = getenv("QNN_FIELDS_KERNEL");
-        if (!force && gemv_mma_takes(d)) return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
+        if (!force && gemv_mma_takes(d, thr != nullptr)) return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
         // one column: byte dot products on the CUDA cores; columns that do not fit an SM's shared
         // memory: the tcgen05 form
         if (gemv_fields_dp4a_fits(d)) return gemv_fields_dp4a_launch(d, W, A, thr, out, (cudaStream_t)stream);
@@ -243,7 +243,7 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
     // 8-bit containers with a handful of columns and no path forced: byte dot products,
     // one warp per weight row (a tensor-core tile would be almost empty)
     if (d->path == QNN_PATH_AUTO && d->w_fmt == QNN_FMT_INT8 && gemv_i8_fits(d))
-        return gemv_mma_takes(d) ? gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream)
+        return gemv_mma_takes(d, thr != nullptr) ? gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream)
                                 : gemv_i8_launch(d, W, A, thr, out, (cudaStream_t)stream);
     if (path == QNN_PATH_TCGEN05_I8) {
         // the workspace is optional (see the header): used only when given, large enough and aligned
@@ -254,7 +254,7 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
     // a handful of columns: stream the weight planes once, one warp per row
     if (gemv_planes_fits(d)) {
         // ... on the tensor cores, unless the caller asks for the bit-serial path or leaves pairs out
-        if (d->path == QNN_PATH_AUTO && d->skip_planes == 0 && gemv_mma_takes(d))
+        if (d->path == QNN_PATH_AUTO && d->skip_planes == 0 && gemv_mma_takes(d, thr != nullptr))
             return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
         return gemv_planes_launch(d, W, A, thr, out, (cudaStream_t)stream);
     }

@@ -82,7 +82,7 @@ qnn_status gemm_bitserial_launch(const qnn_gemm_desc *d, const void *W, const vo
                                  const int32_t *thr, void *out, cudaStream_t s);
 qnn_status gemm_bitserial_conv_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W,
                                       const void *in, const int32_t *thr, void *out, cudaStream_t s);
-bool gemv_mma_takes(const qnn_gemm_desc *d);
+bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr);
 qnn_status gemv_mma_launch(const qnn_gemm_desc *d, const void *W, const void *A,
                            const int32_t *thr, void *out, cudaStream_t s);
 bool gemv_i8_fits(const qnn_gemm_desc *d);

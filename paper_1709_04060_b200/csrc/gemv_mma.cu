@@ -372,13 +372,20 @@ static bool mv_plan(const qnn_gemm_desc *d, MvPlan *pl) {
 //   planes  two columns on, W2A2 N = 2 8.7 -> 8.3, N = 16 39 -> 14.9; one column where there are twelve or
 //           more plane pairs to count: W4A4 15.8 -> 14.9 (W2A2 6.2 -> 8.4)
 //   bytes   three columns on: N = 4 26 -> 17, N = 8 35 -> 18 (N = 2 15.9 -> 17.6), and not for small
-//           matrices (1000 x 4096, N = 7: 4.7 -> 4.9)
-bool gemv_mma_takes(const qnn_gemm_desc *d) {
+//           matrices (1000 x 4096, N = 7: 4.6 -> 4.9)
+//   any     where the others need a second launch that clears the output first (bit planes they set
+//           bit by bit; pad bytes they do not write), call after call: fields N = 1 10.2 -> 8.1, bytes
+//           4096 x 9216 N = 1 12.8 -> 11.4, planes 1000 x 4096 N = 1 7.9 -> 4.9; bytes only below 2^26
+//           elements (8192 x 8192: 16.1 there, 17 here), planes below 2^24 (from there on the two
+//           launches take less time on the device: 66.9 against 67.6 us for the batch-1 chain as a graph)
+bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr) {
     MvPlan pl;
     if (!mv_plan(d, &pl)) return false;
-    if (pl.src == MV_FIELDS) return d->N >= 2;
-    if (pl.src == MV_PLANES) return d->N >= 2 || d->w_bits * d->a_bits >= 12;
-    return d->N >= 3 && (long long)d->M * d->K >= (1ll << 23);
+    const bool clears = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (pl.src != MV_FIELDS && d->M % 16 != 0));
+    if (pl.src == MV_FIELDS) return d->N >= 2 || clears;
+    const long long size = (long long)d->M * d->K;
+    if (pl.src == MV_PLANES) return d->N >= 2 || d->w_bits * d->a_bits >= 12 || (clears && size < (1ll << 24));
+    return (d->N >= 3 && size >= (1ll << 23)) || (clears && size < (1ll << 26));
 }
 
 template <int SRC, int B, int V, int NT, bool W_SIGNED, bool A_SIGNED>
