@@ -57,6 +57,20 @@ __device__ __forceinline__ void pdl_enter() {
 #endif
 
 #ifdef __CUDACC__
+// Lets a kernel be launched with up to `limit` bytes of dynamic shared memory.  The attribute is set once
+// per kernel and device (`done`: static, one flag per device), always to the same limit: threads that
+// arrive here together write the same number, so no order of theirs leaves an attribute below what a
+// launch needs (one that followed the largest size seen so far could be lowered by a second thread).
+constexpr size_t SMEM_LIMIT = 227 * 1024;
+template <typename Kernel>
+inline bool allow_smem(Kernel *kern, size_t limit, std::atomic<bool> &done) {
+    if (done.load(std::memory_order_relaxed)) return true;
+    if (cudaFuncSetAttribute(reinterpret_cast<const void *>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess)
+        return false;
+    done.store(true, std::memory_order_relaxed);
+    return true;
+}
+
 // Launch with programmatic stream serialization (see above): the launch gap overlaps the tail of the
 // kernel ahead.  For kernels that wait in griddepcontrol.wait before they touch global memory.
 template <typename Params>

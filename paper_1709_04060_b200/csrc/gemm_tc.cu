@@ -1536,7 +1536,7 @@ static bool make_im2col_map(CUtensorMap *map, const void *base, const qnn_conv_d
 // Shared memory of a LOWER kernel besides its two staging buffers.
 template <int BN, int STAGES, int OUT_BITS>
 constexpr size_t tc_lower_base_smem() { return ((sizeof(TcSmem<BN, STAGES, OUT_BITS>) + 1023) & ~size_t(1023)) + 1024; }
-constexpr size_t TC_SMEM_LIMIT = 227 * 1024;
+constexpr size_t TC_SMEM_LIMIT = SMEM_LIMIT;
 
 // The ring of plane words of a LOWER == 3 kernel: two slots of kbs k-blocks of both operands.
 static size_t pl_ring_bytes(const TcParams &p, int bn, int kbs) {
@@ -1554,15 +1554,9 @@ static qnn_status launch_cfg(const CUtensorMap &ma, const CUtensorMap &mw, const
                (LOWER == 1 && p.num_kb > STAGES ? (size_t)(p.num_kb - STAGES) * BN * TC_BK : 0);
     }
     if (smem > TC_SMEM_LIMIT) return QNN_ERR_UNSUPPORTED;
-    // per instantiation and device: the largest size configured so far
-    static size_t attr_smem[QNN_MAX_DEVICES] = {0};
+    static std::atomic<bool> attr_done[QNN_MAX_DEVICES];    // per instantiation and device
     const int dev = current_device();
-    if (dev < 0) return QNN_ERR_CUDA;
-    if (smem > attr_smem[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return QNN_ERR_CUDA;
-        attr_smem[dev] = smem;
-    }
+    if (dev < 0 || !allow_smem(kern, TC_SMEM_LIMIT, attr_done[dev])) return QNN_ERR_CUDA;
     const int grid = p.units < sm_count() ? p.units : sm_count();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(LOWER ? TC_THREADS + LW_THREADS : TC_THREADS);
@@ -1594,14 +1588,9 @@ template <int OUT_MODE, int OUT_BITS, int KIND>
 static qnn_status launch_pair_cfg(const CUtensorMap &ma, const CUtensorMap &mw, const TcParams &p, cudaStream_t s) {
     auto kern = qgemm_tc2_kernel<OUT_MODE, OUT_BITS, KIND>;
     const size_t smem = sizeof(Tc2Smem<OUT_BITS>) + 1024;
-    static bool attr_done[QNN_MAX_DEVICES] = {false};       // per instantiation and device
+    static std::atomic<bool> attr_done[QNN_MAX_DEVICES];    // per instantiation and device
     const int dev = current_device();
-    if (dev < 0) return QNN_ERR_CUDA;
-    if (!attr_done[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return QNN_ERR_CUDA;
-        attr_done[dev] = true;
-    }
+    if (dev < 0 || !allow_smem(kern, smem, attr_done[dev])) return QNN_ERR_CUDA;
     const int tiles = p.tiles_p * p.tiles_c;
     const int max_pairs = sm_count() / 2;
     const int pairs = tiles < max_pairs ? tiles : max_pairs;

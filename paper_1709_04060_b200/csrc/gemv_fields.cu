@@ -500,13 +500,8 @@ qnn_status gemv_fields_launch(const qnn_gemm_desc *d, const void *W, const void 
     if (dev < 0) return QNN_ERR_CUDA;
     const void *fn = pl.F == 1 ? (const void *)gemv_fields_kernel<1>
                      : (pl.F == 2 ? (const void *)gemv_fields_kernel<2> : (const void *)gemv_fields_kernel<4>);
-    static size_t attr_smem[3][QNN_MAX_DEVICES] = {{0}};
-    const int fi = pl.F == 1 ? 0 : (pl.F == 2 ? 1 : 2);
-    if (smem > attr_smem[fi][dev]) {
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return QNN_ERR_CUDA;
-        attr_smem[fi][dev] = smem;
-    }
+    static std::atomic<bool> attr_done[3][QNN_MAX_DEVICES];
+    if (!allow_smem(fn, SMEM_LIMIT, attr_done[pl.F == 1 ? 0 : (pl.F == 2 ? 1 : 2)][dev])) return QNN_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(pl.nblocks * pl.sk)); cfg.blockDim = dim3(GF_THREADS);
     cfg.dynamicSmemBytes = smem; cfg.stream = s;

@@ -273,13 +273,9 @@ qnn_status gemv_fields_dp4a_launch(const qnn_gemm_desc *d, const void *W, const 
 #undef QNN_FD_PICK
     const int dev = current_device();
     if (dev < 0) return QNN_ERR_CUDA;
-    static size_t attr_smem[18][QNN_MAX_DEVICES] = {{0}};
+    static std::atomic<bool> attr_done[18][QNN_MAX_DEVICES];
     const int fi = ((F == 1 ? 0 : (F == 2 ? 1 : 2)) * 2 + (as ? 1 : 0)) * 3 + (nc == 1 ? 0 : (nc == 2 ? 1 : 2));
-    if (smem > 48 * 1024 && smem > attr_smem[fi][dev]) {
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return QNN_ERR_CUDA;
-        attr_smem[fi][dev] = smem;
-    }
+    if (!allow_smem(fn, SMEM_LIMIT, attr_done[fi][dev])) return QNN_ERR_CUDA;
     // a persistent grid: as many CTAs as are resident at once, each staging its columns once and
     // then taking row blocks in turn
     // (the occupancy query costs the host 2 us; its answer depends on the kernel and its shared memory)

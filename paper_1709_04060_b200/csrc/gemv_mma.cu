@@ -32,7 +32,7 @@ constexpr int MV_WARPS = 16, MV_THREADS = 32 * MV_WARPS;
 constexpr int MV_ROWS = 32;             // weight rows per tile
 constexpr int MV_COLS = 16;             // most columns
 constexpr int MV_PART_PITCH = 36;       // partial sums [column][row], row pitch without bank conflicts
-constexpr size_t MV_SMEM_MAX = 227 * 1024;
+constexpr size_t MV_SMEM_MAX = SMEM_LIMIT;
 
 enum { MV_PLANES = 0, MV_FIELDS = 1, MV_BYTES = 2 };
 
@@ -391,13 +391,9 @@ bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr) {
 template <int SRC, int B, int V, int NT, bool W_SIGNED, bool A_SIGNED>
 static qnn_status mv_launch(const MvParams &p, size_t smem, cudaStream_t s) {
     auto kern = gemv_mma_kernel<SRC, B, V, NT, W_SIGNED, A_SIGNED>;
-    static size_t attr_smem[QNN_MAX_DEVICES] = {0};                // per instantiation and device
+    static std::atomic<bool> attr_done[QNN_MAX_DEVICES];           // per instantiation and device
     const int dev = current_device();
-    if (dev < 0) return QNN_ERR_CUDA;
-    if (smem > 48 * 1024 && smem > attr_smem[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return QNN_ERR_CUDA;
-        attr_smem[dev] = smem;
-    }
+    if (dev < 0 || !allow_smem(kern, MV_SMEM_MAX, attr_done[dev])) return QNN_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.tiles < sm_count() ? p.tiles : sm_count())); cfg.blockDim = dim3(MV_THREADS);
     cfg.dynamicSmemBytes = smem; cfg.stream = s;

@@ -135,15 +135,11 @@ qnn_status qnn_peak_mma_i8(int mode, int n, int mmas_per_cta, double *ops, void 
     const size_t smem = sizeof(PeakSmem) + 1024;
     const int dev = current_device();
     if (dev < 0) return QNN_ERR_CUDA;
-    static bool attr_done[3][QNN_MAX_DEVICES] = {{false}};
-    if (!attr_done[mode][dev]) {
-        const void *fn = mode == PK_PAIR ? (const void *)peak_mma_i8_kernel<PK_PAIR>
-                         : (mode == PK_TMEM_A ? (const void *)peak_mma_i8_kernel<PK_TMEM_A>
-                                              : (const void *)peak_mma_i8_kernel<PK_SINGLE>);
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return QNN_ERR_CUDA;
-        attr_done[mode][dev] = true;
-    }
+    static std::atomic<bool> attr_done[3][QNN_MAX_DEVICES];
+    const void *fn = mode == PK_PAIR ? (const void *)peak_mma_i8_kernel<PK_PAIR>
+                     : (mode == PK_TMEM_A ? (const void *)peak_mma_i8_kernel<PK_TMEM_A>
+                                          : (const void *)peak_mma_i8_kernel<PK_SINGLE>);
+    if (!allow_smem(fn, smem, attr_done[mode][dev])) return QNN_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = smem; cfg.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[1];
