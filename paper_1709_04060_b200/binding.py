@@ -145,13 +145,15 @@ def _ptr(x):
 
 _Tensor = torch.Tensor
 # The current stream's handle without building a torch.cuda.Stream around it (0.2 us
-# instead of 3.5 us a call).
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# instead of 3.5 us a call), where this build of torch has these two functions: without
+# them the library can still be imported and queried on the host.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream):
     if stream is None:
-        if not _initialized():
+        if _raw_stream is None or _device is None or not _initialized():
             return torch.cuda.current_stream().cuda_stream
         return _raw_stream(_device())
     return int(stream)

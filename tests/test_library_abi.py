@@ -4,6 +4,8 @@ behaves as documented.  No kernel is launched here."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -192,3 +194,16 @@ def test_kernel_choice_follows_the_documented_rule(qb):
     assert k(8192, 16, 8192, FL, I8) == qb.QNN_KERNEL_FIELDS_FEW_COLUMNS
     assert k(8192, 17, 8192, FL, I8) == qb.QNN_ERR_UNSUPPORTED
     assert k(64, 64, 64, I8, PL) == qb.QNN_ERR_UNSUPPORTED                # mixed formats
+
+
+def test_import_does_not_need_private_functions_of_torch(qb):
+    """A torch build without the two functions behind the short way to the stream handle: the library
+    still imports and answers host queries."""
+    code = ("import torch\n"
+            "for n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "from paper_1709_04060_b200 import binding as qb\n"
+            "assert qb.qnn_packed_ld(576, qb.QNN_FMT_BITPLANES) == 18\n"
+            "assert qb.qnn_pack(qb.qnn_pack_desc(4, 64, 0, 0, 0), 16, 16, stream=0) == qb.QNN_ERR_INVALID_ARG\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-1500:]
