@@ -182,7 +182,7 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A,
                      const int32_t *thr, void *out,
                      void *workspace, size_t workspace_bytes, void *stream);
 
-/* Which kernel qnn_qgemm runs for this problem (Section 4.1.2 of the paper: the engine is
+/* Which kind of kernel qnn_qgemm runs for this problem (Section 4.1.2 of the paper: the engine is
  * chosen per layer shape).  The operand format is the caller's choice; on this GPU 8-bit
  * containers on the tensor cores are faster than bit planes for every size from 64 to 4096 per
  * dimension and every (w, a), so AUTO never converts between formats, it picks by shape:
@@ -201,12 +201,19 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A,
  *                       byte dot product per word and field position; more: packed weights widened
  *                       in registers for warp-level tensor-core products, or (columns beyond an
  *                       SM's shared memory) inside a tcgen05 kernel
- * Returns a qnn_kernel value, or the (negative) qnn_status qnn_qgemm would return.  Host only. */
+ * Returns a qnn_kernel value, or the (negative) qnn_status qnn_qgemm would return.  A value names the
+ * operand format and the kind of shape; several kernels share one (qnn_qgemm_kernel_name tells them
+ * apart).  Host only. */
 typedef enum {
     QNN_KERNEL_TENSOR = 1, QNN_KERNEL_TENSOR_CTA_PAIR = 2, QNN_KERNEL_BYTES_FEW_COLUMNS = 3,
     QNN_KERNEL_PLANES_FEW_COLUMNS = 4, QNN_KERNEL_PLANES_TILED = 5, QNN_KERNEL_FIELDS_FEW_COLUMNS = 6
 } qnn_kernel;
 int qnn_qgemm_kernel(const qnn_gemm_desc *d, int has_thresholds);
+
+/* The name of the kernel function qnn_qgemm runs for this problem, as a profiler shows it (qgemm_tc_kernel
+ * also for bit planes expanded inside it; without the clearing launch that some few-column kernels need
+ * first).  NULL where qnn_qgemm would return an error.  Host only. */
+const char *qnn_qgemm_kernel_name(const qnn_gemm_desc *d, int has_thresholds);
 
 /* ---- lowering and convolution (Section 3.2) ------------------------------- */
 

@@ -111,6 +111,31 @@ static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
     return d->w_bits * d->a_bits < 16 || macs > double(1 << 30);
 }
 
+// The kernel a valid problem runs on: the one place where qnn_qgemm and the host queries decide.
+enum Route {
+    ROUTE_FIELDS_MMA, ROUTE_FIELDS_DP4A, ROUTE_FIELDS_TENSOR,      // packed weights
+    ROUTE_BYTES_MMA, ROUTE_BYTES_DP4A, ROUTE_TENSOR,               // 8-bit containers
+    ROUTE_PLANES_MMA, ROUTE_PLANES_POPC, ROUTE_PLANES_TENSOR, ROUTE_PLANES_TILED
+};
+static Route gemm_route(const qnn_gemm_desc *d, bool has_thr, int path) {
+    if (d->w_fmt == QNN_FMT_FIELDS) {
+        if (!getenv("QNN_FIELDS_KERNEL") && gemv_mma_takes(d, has_thr)) return ROUTE_FIELDS_MMA;
+        // one column: byte dot products on the CUDA cores; columns that do not fit an SM's shared
+        // memory: the tcgen05 form
+        return gemv_fields_dp4a_fits(d) ? ROUTE_FIELDS_DP4A : ROUTE_FIELDS_TENSOR;
+    }
+    // 8-bit containers with a handful of columns and no path forced: the weights are streamed once
+    // (a tensor-core tile would be almost empty)
+    if (d->path == QNN_PATH_AUTO && d->w_fmt == QNN_FMT_INT8 && gemv_i8_fits(d))
+        return gemv_mma_takes(d, has_thr) ? ROUTE_BYTES_MMA : ROUTE_BYTES_DP4A;
+    if (path == QNN_PATH_TCGEN05_I8) return ROUTE_TENSOR;
+    // a handful of columns: stream the weight planes once ...
+    if (gemv_planes_fits(d))
+        // ... on the tensor cores, unless the caller asks for the bit-serial path or leaves pairs out
+        return d->path == QNN_PATH_AUTO && d->skip_planes == 0 && gemv_mma_takes(d, has_thr) ? ROUTE_PLANES_MMA : ROUTE_PLANES_POPC;
+    return planes_on_tensor_cores(d) ? ROUTE_PLANES_TENSOR : ROUTE_PLANES_TILED;
+}
+
 // Convolution on bit planes by way of 8-bit containers: the map and the filters are widened into the
 // workspace, which has room for them wherever a lowered matrix would be several times the map, and the
 // 8-bit convolution kernels run on that.  Expanding inside the GEMM kernel instead repeats the work
@@ -217,11 +242,30 @@ int qnn_qgemm_kernel(const qnn_gemm_desc *d, int has_thresholds) {
     int path = 0;
     const qnn_status st = check_gemm_desc(d, has_thresholds != 0, &path);
     if (st != QNN_OK) return (int)st;
-    if (d->w_fmt == QNN_FMT_FIELDS) return QNN_KERNEL_FIELDS_FEW_COLUMNS;
-    if (d->path == QNN_PATH_AUTO && d->w_fmt == QNN_FMT_INT8 && gemv_i8_fits(d)) return QNN_KERNEL_BYTES_FEW_COLUMNS;
-    if (path == QNN_PATH_TCGEN05_I8) return gemm_tc_uses_pair_kernel(d) ? QNN_KERNEL_TENSOR_CTA_PAIR : QNN_KERNEL_TENSOR;
-    if (gemv_planes_fits(d)) return QNN_KERNEL_PLANES_FEW_COLUMNS;
+    switch (gemm_route(d, has_thresholds != 0, path)) {
+        case ROUTE_FIELDS_MMA: case ROUTE_FIELDS_DP4A: case ROUTE_FIELDS_TENSOR: return QNN_KERNEL_FIELDS_FEW_COLUMNS;
+        case ROUTE_BYTES_MMA: case ROUTE_BYTES_DP4A: return QNN_KERNEL_BYTES_FEW_COLUMNS;
+        case ROUTE_TENSOR: return gemm_tc_uses_pair_kernel(d) ? QNN_KERNEL_TENSOR_CTA_PAIR : QNN_KERNEL_TENSOR;
+        case ROUTE_PLANES_MMA: case ROUTE_PLANES_POPC: return QNN_KERNEL_PLANES_FEW_COLUMNS;
+        case ROUTE_PLANES_TENSOR: case ROUTE_PLANES_TILED: break;
+    }
     return QNN_KERNEL_PLANES_TILED;
+}
+
+const char *qnn_qgemm_kernel_name(const qnn_gemm_desc *d, int has_thresholds) {
+    int path = 0;
+    if (check_gemm_desc(d, has_thresholds != 0, &path) != QNN_OK) return nullptr;
+    switch (gemm_route(d, has_thresholds != 0, path)) {
+        case ROUTE_FIELDS_MMA: case ROUTE_BYTES_MMA: case ROUTE_PLANES_MMA: return "gemv_mma_kernel";
+        case ROUTE_FIELDS_DP4A: return "gemv_fields_dp4a_kernel";
+        case ROUTE_FIELDS_TENSOR: return "gemv_fields_kernel";
+        case ROUTE_BYTES_DP4A: return "gemv_i8_kernel";
+        case ROUTE_TENSOR: return gemm_tc_uses_pair_kernel(d) ? "qgemm_tc2_kernel" : "qgemm_tc_kernel";
+        case ROUTE_PLANES_POPC: return "gemv_planes_kernel";
+        case ROUTE_PLANES_TENSOR: return "qgemm_tc_kernel";
+        case ROUTE_PLANES_TILED: break;
+    }
+    return "qgemm_bitserial_kernel";
 }
 
 qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const int32_t *thr,
@@ -232,37 +276,25 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
     if (!W || !A || !out) return QNN_ERR_INVALID_ARG;
     if (!aligned16(W) || !aligned16(A) || !aligned16(out) || (thr && (reinterpret_cast<uintptr_t>(thr) & 3u)))
         return QNN_ERR_ALIGNMENT;
-    if (d->w_fmt == QNN_FMT_FIELDS) {
-        const char *force = getenv("QNN_FIELDS_KERNEL");
-        if (!force && gemv_mma_takes(d, thr != nullptr)) return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
-        // one column: byte dot products on the CUDA cores; columns that do not fit an SM's shared
-        // memory: the tcgen05 form
-        if (gemv_fields_dp4a_fits(d)) return gemv_fields_dp4a_launch(d, W, A, thr, out, (cudaStream_t)stream);
-        return gemv_fields_launch(d, W, A, thr, out, (cudaStream_t)stream);
+    const cudaStream_t cs = (cudaStream_t)stream;
+    switch (gemm_route(d, thr != nullptr, path)) {
+        case ROUTE_FIELDS_MMA: case ROUTE_BYTES_MMA: case ROUTE_PLANES_MMA: return gemv_mma_launch(d, W, A, thr, out, cs);
+        case ROUTE_FIELDS_DP4A: return gemv_fields_dp4a_launch(d, W, A, thr, out, cs);
+        case ROUTE_FIELDS_TENSOR: return gemv_fields_launch(d, W, A, thr, out, cs);
+        case ROUTE_BYTES_DP4A: return gemv_i8_launch(d, W, A, thr, out, cs);
+        case ROUTE_TENSOR: {
+            // the workspace is optional (see the header): used only when given, large enough and aligned
+            const bool ws_ok = workspace && aligned16(workspace);
+            return gemm_tc_launch(d, W, A, thr, out, ws_ok ? workspace : nullptr, ws_ok ? workspace_bytes : 0, cs);
+        }
+        case ROUTE_PLANES_POPC: return gemv_planes_launch(d, W, A, thr, out, cs);
+        case ROUTE_PLANES_TENSOR:
+            st = gemm_tc_planes_launch(nullptr, d, W, A, thr, out, cs);
+            if (st != QNN_ERR_UNSUPPORTED) return st;
+            break;
+        case ROUTE_PLANES_TILED: break;
     }
-    // 8-bit containers with a handful of columns and no path forced: byte dot products,
-    // one warp per weight row (a tensor-core tile would be almost empty)
-    if (d->path == QNN_PATH_AUTO && d->w_fmt == QNN_FMT_INT8 && gemv_i8_fits(d))
-        return gemv_mma_takes(d, thr != nullptr) ? gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream)
-                                : gemv_i8_launch(d, W, A, thr, out, (cudaStream_t)stream);
-    if (path == QNN_PATH_TCGEN05_I8) {
-        // the workspace is optional (see the header): used only when given, large enough and aligned
-        const bool ws_ok = workspace && aligned16(workspace);
-        return gemm_tc_launch(d, W, A, thr, out, ws_ok ? workspace : nullptr, ws_ok ? workspace_bytes : 0,
-                              (cudaStream_t)stream);
-    }
-    // a handful of columns: stream the weight planes once, one warp per row
-    if (gemv_planes_fits(d)) {
-        // ... on the tensor cores, unless the caller asks for the bit-serial path or leaves pairs out
-        if (d->path == QNN_PATH_AUTO && d->skip_planes == 0 && gemv_mma_takes(d, thr != nullptr))
-            return gemv_mma_launch(d, W, A, thr, out, (cudaStream_t)stream);
-        return gemv_planes_launch(d, W, A, thr, out, (cudaStream_t)stream);
-    }
-    if (planes_on_tensor_cores(d)) {
-        st = gemm_tc_planes_launch(nullptr, d, W, A, thr, out, (cudaStream_t)stream);
-        if (st != QNN_ERR_UNSUPPORTED) return st;
-    }
-    return gemm_bitserial_launch(d, W, A, thr, out, (cudaStream_t)stream);
+    return gemm_bitserial_launch(d, W, A, thr, out, cs);
 }
 
 int qnn_conv_out_h(const qnn_conv_desc *d) {

@@ -207,3 +207,53 @@ def test_import_does_not_need_private_functions_of_torch(qb):
             "assert qb.qnn_pack(qb.qnn_pack_desc(4, 64, 0, 0, 0), 16, 16, stream=0) == qb.QNN_ERR_INVALID_ARG\n")
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-1500:]
+
+
+def test_kernel_names_on_both_sides_of_every_rule(qb):
+    """qnn_qgemm_kernel_name (host only) on both sides of each line the dispatch draws within a format;
+    qnn_qgemm takes its decision from the same function."""
+    I8, PL, FL = qb.QNN_FMT_INT8, qb.QNN_FMT_BITPLANES, qb.QNN_FMT_FIELDS
+    S, B = qb.QNN_ENC_SIGNED, qb.QNN_ENC_BIPOLAR
+
+    def k(M, N, K, fmt, w=2, a=2, out=I8, thr=True, path=0, skip=0, w_enc=S, a_enc=0):
+        d = qb.qnn_gemm_desc(M, N, K, w, a, 2, w_enc, a_enc, fmt, PL if fmt == PL else I8, out, path, skip)
+        return qb.qnn_qgemm_kernel_name(d, thr)
+
+    mma, popc, tiled, tc = "gemv_mma_kernel", "gemv_planes_kernel", "qgemm_bitserial_kernel", "qgemm_tc_kernel"
+    # packed weights: two columns on; one column where a clearing launch would be needed; depths that
+    # an SM's shared memory does not hold
+    assert k(8192, 1, 8192, FL) == "gemv_fields_dp4a_kernel"
+    assert k(8192, 1, 8192, FL, out=PL) == mma
+    assert k(8192, 1, 8192, FL, out=PL, thr=False) == "gemv_fields_dp4a_kernel"
+    assert k(8192, 2, 8192, FL) == mma
+    assert k(8192, 16, 9216, FL) == mma
+    assert k(8192, 16, 16384, FL) == "gemv_fields_kernel"
+    # bytes: three columns on from 2^23 weights; fewer where pad bytes need clearing, below 2^26 weights
+    assert k(2048, 3, 4096, I8) == mma
+    assert k(2048, 3, 4080, I8) == "gemv_i8_kernel"
+    assert k(4096, 2, 4096, I8) == "gemv_i8_kernel"
+    assert k(4100, 1, 4096, I8) == mma
+    assert k(4100, 1, 4096, I8, thr=False) == "gemv_i8_kernel"
+    assert k(8200, 1, 8192, I8, out=PL) == "gemv_i8_kernel"
+    assert k(4096, 9, 4096, I8) == tc
+    assert k(4096, 4096, 4096, I8) == "qgemm_tc2_kernel"
+    # planes, few columns: two columns on; one with twelve plane pairs, or cleared below 2^24 weights
+    assert k(8192, 1, 8192, PL) == popc
+    assert k(8192, 2, 8192, PL) == mma
+    assert k(8192, 1, 8192, PL, w=3, a=4) == mma
+    assert k(8192, 1, 8192, PL, w=3, a=3) == popc
+    assert k(4095, 1, 4096, PL) == mma
+    assert k(4096, 1, 4096, PL, out=PL) == popc
+    assert k(8192, 2, 8192, PL, path=qb.QNN_PATH_BITSERIAL) == popc
+    assert k(8192, 2, 8192, PL, skip=1) == popc
+    # planes, tiled: sixteen plane pairs up to 2^30, a single pair between 2^24 and 2^27, the forced path
+    # and skipped pairs stay with AND/POPC
+    assert k(1024, 1024, 1024, PL) == tc
+    assert k(1024, 1024, 1024, PL, w=4, a=4) == tiled
+    assert k(1024, 1024, 1025, PL, w=4, a=4) == tc
+    assert k(1024, 1024, 1024, PL, w=3, a=4) == tc
+    assert k(512, 512, 512, PL, w=1, a=1, w_enc=B, a_enc=B) == tiled
+    assert k(512, 512, 513, PL, w=1, a=1, w_enc=B, a_enc=B) == tc
+    assert k(1024, 1024, 1024, PL, path=qb.QNN_PATH_BITSERIAL) == tiled
+    assert k(1024, 1024, 1024, PL, skip=1) == tiled
+    assert k(64, 64, 64, I8, w=0) is None
