@@ -105,6 +105,10 @@ static void conv_to_gemm(const qnn_conv_desc *d, qnn_gemm_desc *g) {
 // skip_planes and with empty plane tiles is what this format promises at these sizes.
 static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
     if (d->path != QNN_PATH_AUTO || d->skip_planes != 0) return false;
+    // The roles of a tensor-core CTA wait for each other at most 2e9 cycles, and the epilogue waits for a
+    // whole tile: 3500 cycles per 128 elements of the depth (four planes each), 0.9e9 at 2^25.  AND/POPC
+    // waits for nothing.
+    if (d->K > (1 << 25)) return false;
     const double macs = (double)d->M * d->N * d->K;
     // a single plane pair at middle sizes (512^3: 7.6 us against 10.9; 1024^3: 16.0 against 13.5)
     if (d->w_bits * d->a_bits == 1 && macs > double(1 << 24) && macs <= double(1 << 27)) return false;

@@ -256,4 +256,7 @@ def test_kernel_names_on_both_sides_of_every_rule(qb):
     assert k(512, 512, 513, PL, w=1, a=1, w_enc=B, a_enc=B) == tc
     assert k(1024, 1024, 1024, PL, path=qb.QNN_PATH_BITSERIAL) == tiled
     assert k(1024, 1024, 1024, PL, skip=1) == tiled
+    # depths whose tiles would outlast the bounded waits of the tensor-core kernel
+    assert k(2, 17, 1 << 25, PL, w=1, a=2, w_enc=B) == tc
+    assert k(2, 17, (1 << 25) + 1, PL, w=1, a=2, w_enc=B) == tiled
     assert k(64, 64, 64, I8, w=0) is None
