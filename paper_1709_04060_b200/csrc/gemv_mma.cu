@@ -367,24 +367,49 @@ static bool mv_plan(const qnn_gemm_desc *d, MvPlan *pl) {
     return pl->smem <= MV_SMEM_MAX;
 }
 
+// Bit planes that need no clearing launch: whether this kernel beats the one that counts bits
+// (gemv_planes.cu), by an estimate of both in microseconds.  That one costs a load latency per staged
+// column and plane, one per depth step of a lane, its CTAs and its population counts; this one its fill
+// and drain, the columns it widens, the rounds of tiles and the weights.  Fitted to 3300 random problems
+// (1 to 16 columns, up to 12000 x 9216, every width and encoding, replayed as a graph): the choice costs
+// 0.8 % of the faster one's time on average, always this kernel 14 % (959 x 64, N = 5, W2A1: 2.7 us there,
+// 4.7 here), always the other 49 %.
+static bool mv_planes_faster(const qnn_gemm_desc *d) {
+    const int kw = ceil_div(d->K, 32), cols = d->N < 4 ? d->N : 4, pairs = d->w_bits * d->a_bits;
+    const double ctas = (double)ceil_div(d->M, 8) * ceil_div(d->N, 4), words = (double)d->M * kw;
+    const double staged = d->w_enc == QNN_ENC_BIPOLAR && d->a_enc != QNN_ENC_BIPOLAR ? 0.48 : 0.32;   // with column sums
+    const double counted = 0.89 + staged * d->a_bits * cols * ceil_div(kw, 256) +
+                           (kw % 4 == 0 ? 0.83 * ceil_div(kw, 128) : 0.23 * ceil_div(kw, 32)) +
+                           0.011 * pairs * cols * ceil_div(kw, 32) + 2.3e-7 * words * pairs * d->N + 2.44e-3 * ctas;
+    const double here = (d->w_bits <= 2 ? 4.8 : 4.0) + (d->N > 8 ? 0.25 : 0.0) + 1.9e-3 * d->N * kw +
+                        1.5 * ((ceil_div(d->M, MV_ROWS) - 1) / sm_count()) + 0.8e-6 * words * d->w_bits;
+    return counted > 0.96 * here;
+}
+
 // Where this kernel is the faster one of those that take the format (8192 x 8192, us, the other -> this):
 //   fields  two columns on: W2A2 N = 2 10.2 -> 8.0, N = 4 13.0 -> 8.0, N = 16 15.4 -> 12.3 (N = 1 6.2 -> 7.8)
-//   planes  two columns on, W2A2 N = 2 8.7 -> 8.3, N = 16 39 -> 14.9; one column where there are twelve or
-//           more plane pairs to count: W4A4 15.8 -> 14.9 (W2A2 6.2 -> 8.4)
+//   planes  two columns on, or one where there are twelve or more plane pairs to count (8192 x 8192 W2A2
+//           N = 2 8.7 -> 8.3, N = 16 39 -> 14.9; W4A4 N = 1 15.8 -> 14.9), but for small problems:
+//           mv_planes_faster
 //   bytes   three columns on: N = 4 26 -> 17, N = 8 35 -> 18 (N = 2 15.9 -> 17.6), and not for small
 //           matrices (1000 x 4096, N = 7: 4.6 -> 4.9)
 //   any     where the others need a second launch that clears the output first (bit planes they set
-//           bit by bit; pad bytes they do not write), call after call: fields N = 1 10.2 -> 8.1, bytes
-//           4096 x 9216 N = 1 12.8 -> 11.4, planes 1000 x 4096 N = 1 7.9 -> 4.9; bytes only below 2^26
-//           elements (8192 x 8192: 16.1 there, 17 here), planes below 2^24 (from there on the two
-//           launches take less time on the device: 66.9 against 67.6 us for the batch-1 chain as a graph)
+//           bit by bit; pad bytes they do not write), the host's second launch decides, call after call
+//           (planes: 4.6 us here, 7.3 there for everything small, and faster here for 677 of 700 random
+//           problems up to 12000 x 9216, although one in three takes up to 3 us longer on the device;
+//           fields N = 1 10.2 -> 8.1, bytes 4096 x 9216 N = 1 12.8 -> 11.4); bytes only below 2^26
+//           elements (8192 x 8192: 16.1 there, 17 here), planes with one column below 2^24 (from there on
+//           the two launches take less time on the device: 66.9 against 67.6 us for the batch-1 chain as
+//           a graph)
 bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr) {
     MvPlan pl;
     if (!mv_plan(d, &pl)) return false;
     const bool clears = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (pl.src != MV_FIELDS && d->M % 16 != 0));
     if (pl.src == MV_FIELDS) return d->N >= 2 || clears;
     const long long size = (long long)d->M * d->K;
-    if (pl.src == MV_PLANES) return d->N >= 2 || d->w_bits * d->a_bits >= 12 || (clears && size < (1ll << 24));
+    if (pl.src == MV_PLANES)
+        return clears ? d->N >= 2 || d->w_bits * d->a_bits >= 12 || size < (1ll << 24)
+                      : (d->N >= 2 || d->w_bits * d->a_bits >= 12) && mv_planes_faster(d);
     return (d->N >= 3 && size >= (1ll << 23)) || (clears && size < (1ll << 26));
 }
 

@@ -242,6 +242,15 @@ def test_kernel_names_on_both_sides_of_every_rule(qb):
     assert k(8192, 2, 8192, PL) == mma
     assert k(8192, 1, 8192, PL, w=3, a=4) == mma
     assert k(8192, 1, 8192, PL, w=3, a=3) == popc
+    # ... but not where little is counted: few activation planes, few rows, a shallow depth
+    assert k(960, 5, 64, PL, w=2, a=1) == popc
+    assert k(961, 5, 64, PL, w=2, a=1) == mma                 # pad bytes to clear
+    assert k(960, 5, 64, PL, w=2, a=1, out=PL) == mma         # bit-plane output
+    assert k(961, 5, 64, PL, w=2, a=1, thr=False) == popc
+    assert k(12000, 16, 64, PL, w=2, a=1) == mma
+    assert k(960, 5, 64, PL, w=2, a=4) == mma
+    assert k(5, 12, 647, PL, w=1, a=1, w_enc=B, thr=False) == popc
+    assert k(352, 1, 512, PL, w=4, a=4) == popc
     assert k(4095, 1, 4096, PL) == mma
     assert k(4096, 1, 4096, PL, out=PL) == popc
     assert k(8192, 2, 8192, PL, path=qb.QNN_PATH_BITSERIAL) == popc
