@@ -115,6 +115,35 @@ static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
     return d->w_bits * d->a_bits < 16 || macs > double(1 << 30);
 }
 
+// Whether the tensor-core kernel that expands planes inside beats the AND/POPC kernel, which it does not
+// where few plane pairs meet little work, raw sums or many thresholds: an estimate of both in microseconds.
+// AND/POPC: 64 x 64 tiles, two CTAs per SM, 512 elements of the depth a step; tensor cores: 128 x 128 tiles
+// whose depth two CTAs share when there are few, 128 elements a step, an epilogue that grows with the
+// thresholds and with raw rows that are not whole 16-byte units, and in a convolution word-by-word copies
+// unless pixels are whole 16-byte units.  Fitted to 4300 random products and 2900 convolutions of one to
+// four plane pairs, replayed as a graph: the choice costs 0.5 % of the faster one's time on average, always
+// the tensor cores 3.2 % (325 x 313 x 132 W1A1 raw sums: 14.5 us there, 6.2 with AND/POPC), always
+// AND/POPC 85 %.  From five plane pairs on the tensor cores were the faster ones everywhere.
+static bool planes_tensor_faster(const qnn_gemm_desc *d, const qnn_conv_desc *cv, bool has_thr) {
+    const int planes = d->w_bits + d->a_bits, pairs = d->w_bits * d->a_bits, sms = sm_count();
+    if (pairs > 4) return true;
+    const double ctas = (double)ceil_div(d->M, 64) * ceil_div(d->N, 64), waves = (double)(((long long)ctas + 2 * sms - 1) / (2 * sms));
+    const int steps = ceil_div(ceil_div(d->K, 32), 16);
+    const double counted = 2.9 + waves * steps * (2.7 * pairs + 0.14 * planes) + ctas * (8.5e-3 + 5.1e-3 * steps * pairs) +
+                           (has_thr ? 1.65 : 0.0) + (has_thr && d->out_fmt == QNN_FMT_BITPLANES ? 0.84 * d->out_bits : 0.0);
+    const long long tiles = (long long)ceil_div(d->M, 128) * ceil_div(d->N, 128);
+    const int kb = ceil_div(d->K, 128);
+    const bool share = 2 * tiles <= sms && kb >= 4, by_words = cv && ceil_div(cv->C, 32) % 4 != 0;
+    const double rounds = share ? 1.0 : (double)((tiles + sms - 1) / sms);
+    // epilogue of a tile by thresholds (1, 3, 7, 15) or raw sums, in the last round and in those before it
+    static const double last_us[5] = {0.0, 1.5, 2.4, 4.9, 6.9}, more_us[5] = {0.0, 0.0, 0.0, 3.3, 3.3};
+    const double last = has_thr ? last_us[d->out_bits] : (d->M % 4 ? 4.6 : 1.4), more = has_thr ? more_us[d->out_bits] : (d->M % 4 ? 8.3 : 2.5);
+    const double part = d->M < 128 ? ceil_div(d->M, 32) / 4.0 : 1.0;
+    const double tensor = 4.3 + (cv ? 0.9 : 0.0) + (by_words ? 3.3 : 0.0) + (share ? 2.7 : 0.0) + part * last + (rounds - 1.0) * (3.5 + part * more) +
+                          rounds * (share ? ceil_div(kb, 2) : kb) * (0.47 + (by_words ? 0.2 : 0.11) * planes);
+    return counted > 0.95 * tensor;
+}
+
 // The kernel a valid problem runs on: the one place where qnn_qgemm and the host queries decide.
 enum Route {
     ROUTE_FIELDS_MMA, ROUTE_FIELDS_DP4A, ROUTE_FIELDS_TENSOR,      // packed weights
@@ -137,7 +166,7 @@ static Route gemm_route(const qnn_gemm_desc *d, bool has_thr, int path) {
     if (gemv_planes_fits(d))
         // ... on the tensor cores, unless the caller asks for the bit-serial path or leaves pairs out
         return d->path == QNN_PATH_AUTO && d->skip_planes == 0 && gemv_mma_takes(d, has_thr) ? ROUTE_PLANES_MMA : ROUTE_PLANES_POPC;
-    return planes_on_tensor_cores(d) ? ROUTE_PLANES_TENSOR : ROUTE_PLANES_TILED;
+    return planes_on_tensor_cores(d) && planes_tensor_faster(d, nullptr, has_thr) ? ROUTE_PLANES_TENSOR : ROUTE_PLANES_TILED;
 }
 
 // Convolution on bit planes by way of 8-bit containers: the map and the filters are widened into the
@@ -375,8 +404,10 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
         if (planes_on_tensor_cores(&g)) {
             st = widened_conv_launch(d, &g, Wpacked, in, thr, out, workspace, workspace_bytes, (cudaStream_t)stream);
             if (st != QNN_ERR_UNSUPPORTED) return st;
-            st = gemm_tc_planes_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
-            if (st != QNN_ERR_UNSUPPORTED) return st;
+            if (planes_tensor_faster(&g, d, thr != nullptr)) {
+                st = gemm_tc_planes_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
+                if (st != QNN_ERR_UNSUPPORTED) return st;
+            }
         }
         st = gemm_bitserial_conv_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
         if (st != QNN_ERR_UNSUPPORTED) return st;

@@ -265,6 +265,14 @@ def test_kernel_names_on_both_sides_of_every_rule(qb):
     assert k(512, 512, 513, PL, w=1, a=1, w_enc=B, a_enc=B) == tc
     assert k(1024, 1024, 1024, PL, path=qb.QNN_PATH_BITSERIAL) == tiled
     assert k(1024, 1024, 1024, PL, skip=1) == tiled
+    # ... and so do few plane pairs with little work, raw sums or many thresholds
+    assert k(325, 313, 132, PL, w=1, a=1, thr=False) == tiled
+    assert k(325, 313, 132, PL, w=2, a=3, thr=False) == tc
+    assert k(133, 1948, 467, PL, w=2, a=1, thr=False) == tiled
+    assert k(133, 1948, 467, PL, w=2, a=1) == tc
+    assert k(325, 4000, 132, PL, w=2, a=2, thr=False) == tc
+    assert k(64, 256, 576, PL, w=1, a=2, w_enc=B) == tc
+    assert k(1000, 3025, 1363, PL, w=2, a=2, thr=False) == tc
     # depths whose tiles would outlast the bounded waits of the tensor-core kernel
     assert k(2, 17, 1 << 25, PL, w=1, a=2, w_enc=B) == tc
     assert k(2, 17, (1 << 25) + 1, PL, w=1, a=2, w_enc=B) == tiled
