@@ -1854,6 +1854,8 @@ qnn_status gemm_tc_lower_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g,
     const int pitch = cv->in_pitch ? cv->in_pitch : round_up(cv->C, 16);
     if (cv->fmt != QNN_FMT_INT8 || pitch != cv->C) return QNN_ERR_UNSUPPORTED;
     const int mode = (cv->C % 16) != 0 ? 1 : 2;
+    // whole image rows are staged; their size below is an int
+    if ((long long)cv->W * cv->C > (long long)TC_SMEM_LIMIT) return QNN_ERR_UNSUPPORTED;
     const int run = cv->KW * cv->C, runp = round_up(run, 16);
     if (g->K != cv->KH * runp) return QNN_ERR_UNSUPPORTED;
     const int OH = qnn_conv_out_h(cv), OW = qnn_conv_out_w(cv);
