@@ -307,7 +307,7 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A, const
     qnn_status st = check_gemm_desc(d, thr != nullptr, &path);
     if (st != QNN_OK) return st;
     if (!W || !A || !out) return QNN_ERR_INVALID_ARG;
-    if (!aligned16(W) || !aligned16(A) || !aligned16(out) || (thr && (reinterpret_cast<uintptr_t>(thr) & 3u)))
+    if (!aligned16(W) || !aligned16(A) || !aligned16(out) || !aligned4(thr))
         return QNN_ERR_ALIGNMENT;
     const cudaStream_t cs = (cudaStream_t)stream;
     switch (gemm_route(d, thr != nullptr, path)) {
@@ -384,7 +384,7 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
     if (st != QNN_OK) return st;
     if (!Wpacked || !in || !out) return QNN_ERR_INVALID_ARG;
     if (!workspace || workspace_bytes < qnn_conv_workspace_bytes(d)) return QNN_ERR_WORKSPACE;
-    if (!aligned16(Wpacked) || !aligned16(in) || !aligned16(out) || !aligned16(workspace))
+    if (!aligned16(Wpacked) || !aligned16(in) || !aligned16(out) || !aligned16(workspace) || !aligned4(thr))
         return QNN_ERR_ALIGNMENT;
     // 8-bit maps on the tensor-core path: the GEMM's loader does the lowering itself (im2col
     // tensor map) where the shape allows; QNN_CONV_EXPLICIT=1 in the environment keeps the
@@ -445,7 +445,7 @@ qnn_status qnn_qconv_static(const qnn_conv_desc *d, const void *Wpacked, const v
     if (st != QNN_OK) return st;
     if (qnn_conv_workspace_bytes(d) > (size_t)QNN_QCONV_STATIC_MAX_BYTES) return QNN_ERR_WORKSPACE;
     if (!Wpacked || !in || !out) return QNN_ERR_INVALID_ARG;
-    if (!aligned16(Wpacked) || !aligned16(in) || !aligned16(out)) return QNN_ERR_ALIGNMENT;
+    if (!aligned16(Wpacked) || !aligned16(in) || !aligned16(out) || !aligned4(thr)) return QNN_ERR_ALIGNMENT;
     void *lowered = nullptr;
     st = static_lowered_ptr(&lowered);
     if (st != QNN_OK) return st;

@@ -277,3 +277,13 @@ def test_kernel_names_on_both_sides_of_every_rule(qb):
     assert k(2, 17, 1 << 25, PL, w=1, a=2, w_enc=B) == tc
     assert k(2, 17, (1 << 25) + 1, PL, w=1, a=2, w_enc=B) == tiled
     assert k(64, 64, 64, I8, w=0) is None
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+def test_convolutions_refuse_misaligned_thresholds(qb, fmt):
+    """As qnn_qgemm does, on the host, whichever kernel the layer would run on (fake addresses)."""
+    P = 0x10000
+    d = qb.qnn_conv_desc(1, 13, 13, 96, 0, 256, 3, 3, 1, 1, 1, 2, 2, 2, 0, fmt, 1, 0)
+    for off in (1, 2, 3):
+        assert qb.qnn_qconv(d, P, P, P + off, P, P, 1 << 30, stream=0) == qb.QNN_ERR_ALIGNMENT
+        assert qb.qnn_qconv_static(d, P, P, P + off, P, stream=0) == qb.QNN_ERR_ALIGNMENT
