@@ -140,11 +140,13 @@ typedef struct {
                              conclusion names; it differs from the exact one by at
                              most K * sum_{i+j<s} 2^(i+j), and the bit-serial kernels
                              skip the AND/POPC work of those pairs.  A BIPOLAR
-                             operand counts as one plane (index 0).  (Apart from
-                             this, and exactly: the tiled bit-plane kernel skips a
-                             plane pair wherever one of its 64-row x 512-bit plane
-                             tiles holds no set bit -- the bit-level sparsity the
-                             same sentence of the paper names.)                   */
+                             operand counts as one plane (index 0).  Such calls
+                             always run the bit-serial kernels and can take longer
+                             than the exact product, which the library may put on the
+                             tensor cores.  (Apart from this, and exactly: the tiled
+                             AND/POPC kernel skips a plane pair wherever one of its
+                             64-row x 512-bit plane tiles holds no set bit -- the
+                             bit-level sparsity the same sentence of the paper names.) */
 } qnn_gemm_desc;
 
 /* Scratch bytes qnn_qgemm can use for this problem (0: none).  The workspace is OPTIONAL:
@@ -192,11 +194,11 @@ qnn_status qnn_qgemm(const qnn_gemm_desc *d, const void *W, const void *A,
  *                       on the SM pairs: the CTA-pair tensor-core kernel; else the one-CTA
  *                       tensor-core kernel
  *   BITPLANES operands  N <= 16: weights streamed once: one warp per weight row over the planes, or
- *                       (two columns on, or many plane pairs) warp-level tensor-core products
- *                       on the planes widened in registers; else tiled: the planes
- *                       are expanded to bytes inside the tensor-core kernel, or (QNN_PATH_BITSERIAL,
- *                       skip_planes, sixteen plane pairs up to 2^30 multiply-accumulates) the
- *                       AND/POPC kernel
+ *                       (two columns on, or many plane pairs, unless little is counted) warp-level
+ *                       tensor-core products on the planes widened in registers; else tiled: the
+ *                       planes are expanded to bytes inside the tensor-core kernel, or (QNN_PATH_BITSERIAL,
+ *                       skip_planes, sixteen plane pairs up to 2^30 multiply-accumulates, few
+ *                       pairs with little work) the AND/POPC kernel
  *   FIELDS weights      N <= 16 only: one column: one warp per packed weight row, an AND and a 4-way
  *                       byte dot product per word and field position; more: packed weights widened
  *                       in registers for warp-level tensor-core products, or (columns beyond an
@@ -263,9 +265,13 @@ qnn_status qnn_im2col(const qnn_conv_desc *d, const void *in, void *lowered, voi
  * weight operand in format d->fmt.  Output: as qnn_qgemm with N = B*OH*OW,
  * M = OC, i.e. a channels-last feature map [B][OH][OW][...].  BIPOLAR
  * activations with pad > 0 are UNSUPPORTED (zero is not representable).
- * The lowered matrix of Section 3.2 is written to `workspace` only where the GEMM
- * kernel cannot form its tiles itself.  Bit-plane maps are lowered on the fly by the
- * loading code of the tiled kernels (word-granular, as in Section 3.2).
+ * `workspace` is scratch of this call alone: any of its workspace_bytes may be written, and
+ * calls that can overlap (different streams) need workspaces of their own.  Which calls write
+ * it is not part of the contract; today it holds the lowered matrix of Section 3.2 where the
+ * GEMM kernel cannot form its tiles itself, and the map and filters of a bit-plane layer of
+ * 2^28 multiply-accumulates or more, widened to 8-bit containers (where they fit).  Smaller
+ * bit-plane maps are lowered on the fly by the loading code of the tiled kernels
+ * (word-granular, as in Section 3.2).
  * 8-bit maps are lowered inside the tensor-core kernel: by its tensor-map loader
  * when C and in_pitch are multiples of 16 (the CTA-pair kernel for large layers,
  * the one-CTA kernel otherwise); by lowering warps when pixels are contiguous and

@@ -8,13 +8,16 @@ arithmetic runs in the library's kernels.
 
 ``mode`` selects the operand format of the W1A2 layers' activations/weights:
   "tensor"     8-bit containers everywhere  (tcgen05 path for every layer)
-  "bitserial"  bit planes for the W1A2 layers (bit-serial path; conv1 writes bit
-               planes directly from its epilogue, fc7 writes 8-bit codes for fc8)
+  "bitserial"  bit planes for the W1A2 layers: the operands of the paper's bit-serial
+               product; conv1 writes bit planes directly from its epilogue, fc7
+               writes 8-bit codes for fc8.  The library picks the kernel by shape:
+               most of these layers are expanded for the tensor cores, some are
+               counted with AND/POPC (a descriptor with QNN_PATH_BITSERIAL forces that)
   "auto"       per layer, as Section 4.1 of the paper suggests choosing the engine
                by shape: 8-bit containers (tensor cores) for the convolutions,
                and, at batch <= 16, bit planes for the fully connected W1A2
                layers, whose packed weights are streamed once by the few-column
-               bit-serial kernel; at larger batch the same as "tensor"
+               kernels; at larger batch the same as "tensor"
 """
 import numpy as np
 import torch
