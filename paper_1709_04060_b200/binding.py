@@ -321,6 +321,15 @@ def _dev_bytes(n: int) -> torch.Tensor:
     return torch.empty(max(int(n), 16), dtype=torch.uint8, device="cuda")
 
 
+def _scratch(n: int, stream, zeroed: bool = False) -> torch.Tensor:
+    """Workspace of one call on ``stream``: allocated (and cleared) there, so that its memory is handed out
+    again only behind the call, whichever stream is the current one."""
+    if stream is None:
+        return torch.zeros(n, dtype=torch.uint8, device="cuda") if zeroed else _dev_bytes(n)
+    with torch.cuda.stream(torch.cuda.ExternalStream(int(stream))):
+        return _scratch(n, None, zeroed)
+
+
 def to_device_logical(x, enc: int) -> torch.Tensor:
     """numpy/torch logical integers -> contiguous device bytes (uint8 for
     UNSIGNED, int8 otherwise), the packer's input format."""
@@ -350,7 +359,7 @@ def qgemm(d: qnn_gemm_desc, W, A, thr, out=None, stream=None) -> torch.Tensor:
         out = _dev_bytes(qnn_gemm_out_bytes(d, thr is not None))
     # the optional workspace starts with flag words that must be zero before the first call
     ws_bytes = qnn_gemm_workspace_bytes(d)
-    ws = torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda") if ws_bytes else None
+    ws = _scratch(ws_bytes, stream, zeroed=True) if ws_bytes else None
     check(qnn_qgemm(d, W, A, thr, out, ws, ws_bytes, stream))
     if thr is None:
         return out[: d.N * d.M * 4].view(torch.int32).view(d.N, d.M)
@@ -381,6 +390,6 @@ def qconv(d: qnn_conv_desc, Wpacked, inp, thr, out=None, workspace=None, stream=
         out = _dev_bytes(qnn_conv_out_bytes(d, thr is not None))
     ws_bytes = qnn_conv_workspace_bytes(d)
     if workspace is None:
-        workspace = _dev_bytes(ws_bytes)
+        workspace = _scratch(ws_bytes, stream)
     check(qnn_qconv(d, Wpacked, inp, thr, out, workspace, workspace.numel(), stream))
     return out

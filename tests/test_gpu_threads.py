@@ -1,4 +1,6 @@
-"""First use of the kernels from several host threads at once.  ctypes releases the interpreter lock, so
+"""Several host threads and several streams.
+
+First use of the kernels from several host threads at once: ctypes releases the interpreter lock, so
 the library's one-time set-up of a kernel runs in all of them together, with problems of the same kernel
 that need different amounts of shared memory."""
 import os
@@ -6,6 +8,7 @@ import subprocess
 import sys
 
 import pytest
+import torch
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +60,28 @@ def test_threads_that_use_a_kernel_first_together():
     for _ in range(3):
         r = subprocess.run([sys.executable, "-c", CHILD], cwd=ROOT, capture_output=True, text=True, timeout=300)
         assert r.returncode == 0, (r.stdout + r.stderr)[-2000:]
+
+
+def test_scratch_of_a_call_on_another_stream():
+    """binding.qconv on a stream that is still busy: the workspace it drops on return must not be handed to
+    the current stream's next tensor while the layer has yet to write it.  (Two layers: the widened bit
+    planes and, for the explicit lowering, 8-bit containers.)"""
+    from paper_1709_04060_b200 import binding as qb
+    side = torch.cuda.Stream()
+    for fmt in (qb.QNN_FMT_BITPLANES, qb.QNN_FMT_INT8):
+        C, k = (96, 5) if fmt == qb.QNN_FMT_BITPLANES else (20, 3)
+        d = qb.qnn_conv_desc(8, 27, 27, C, 0, 256, k, k, 1, k // 2, 1, 2, 2, 0, 0, fmt, qb.QNN_FMT_INT8, 0)
+        x = torch.ones(1 << 20, dtype=torch.uint8, device="cuda")
+        W = torch.ones(1 << 20, dtype=torch.uint8, device="cuda")
+        thr = torch.arange(256 * 3, dtype=torch.int32, device="cuda")
+        n = qb.qnn_conv_workspace_bytes(d)
+        out = torch.empty(qb.qnn_conv_out_bytes(d, True), dtype=torch.uint8, device="cuda")
+        for warm in range(2):                                  # the pools know the size
+            qb.qconv(d, W, x, thr, out, stream=side.cuda_stream)
+            torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(20_000_000)                      # about 10 ms
+        qb.qconv(d, W, x, thr, out, stream=side.cuda_stream)
+        mine = [torch.full((n,), 7, dtype=torch.uint8, device="cuda") for _ in range(2)]
+        torch.cuda.synchronize()
+        assert all(bool((t == 7).all()) for t in mine)
