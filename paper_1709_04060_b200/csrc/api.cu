@@ -121,15 +121,17 @@ static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
 // whose depth two CTAs share when there are few, 128 elements a step, an epilogue that grows with the
 // thresholds and with raw rows that are not whole 16-byte units, and in a convolution word-by-word copies
 // unless pixels are whole 16-byte units.  Fitted to 4300 random products and 2900 convolutions of one to
-// four plane pairs, replayed as a graph: the choice costs 0.5 % of the faster one's time on average, always
-// the tensor cores 3.2 % (325 x 313 x 132 W1A1 raw sums: 14.5 us there, 6.2 with AND/POPC), always
+// four plane pairs, replayed as a graph; call after call the AND/POPC kernel, which is launched normally,
+// takes 1.9 us more (the launch gap), the other 0.5, and 1.8 us are added so that neither kind of caller
+// loses.  The choice costs 0.7 % (graph) and 0.3 % (calls) of the faster one's time on average, always the
+// tensor cores 2.6 % and 1.2 % (325 x 313 x 132 W1A1 raw sums: 14.5 us there, 6.2 with AND/POPC), always
 // AND/POPC 85 %.  From five plane pairs on the tensor cores were the faster ones everywhere.
 static bool planes_tensor_faster(const qnn_gemm_desc *d, const qnn_conv_desc *cv, bool has_thr) {
     const int planes = d->w_bits + d->a_bits, pairs = d->w_bits * d->a_bits, sms = sm_count();
     if (pairs > 4) return true;
     const double ctas = (double)ceil_div(d->M, 64) * ceil_div(d->N, 64), waves = (double)(((long long)ctas + 2 * sms - 1) / (2 * sms));
     const int steps = ceil_div(ceil_div(d->K, 32), 16);
-    const double counted = 2.9 + waves * steps * (2.7 * pairs + 0.14 * planes) + ctas * (8.5e-3 + 5.1e-3 * steps * pairs) +
+    const double counted = 2.9 + 1.8 + waves * steps * (2.7 * pairs + 0.14 * planes) + ctas * (8.5e-3 + 5.1e-3 * steps * pairs) +
                            (has_thr ? 1.65 : 0.0) + (has_thr && d->out_fmt == QNN_FMT_BITPLANES ? 0.84 * d->out_bits : 0.0);
     const long long tiles = (long long)ceil_div(d->M, 128) * ceil_div(d->N, 128);
     const int kb = ceil_div(d->K, 128);
