@@ -827,7 +827,7 @@ def run_shapes(args):
     """Size sweep of Section 4.1.2 of the paper: every (rows, depth, cols) in {2^6 .. 2^12}^3, for
     every (w, a) in {1..4}^2 (--pairs restricts them; weights bipolar when w = 1, else signed;
     activations unsigned), GEMM+threshold on 8-bit containers (tensor cores) and on bit planes
-    (bit-serial kernels), each timed by replaying a CUDA graph of repeated calls.  Prints one JSON
+    (the library's own choice of kernel), each timed by replaying a CUDA graph of repeated calls.  Prints one JSON
     line per (w, a) with the per-shape times, the faster operand format and the kernel the library
     chose, and a summary line."""
     import torch

@@ -120,12 +120,12 @@ static bool planes_on_tensor_cores(const qnn_gemm_desc *d) {
 // AND/POPC: 64 x 64 tiles, two CTAs per SM, 512 elements of the depth a step; tensor cores: 128 x 128 tiles
 // whose depth two CTAs share when there are few, 128 elements a step, an epilogue that grows with the
 // thresholds and with raw rows that are not whole 16-byte units, and in a convolution word-by-word copies
-// unless pixels are whole 16-byte units.  Fitted to 4300 random products and 2900 convolutions of one to
+// unless pixels are whole 16-byte units.  Fitted to 3800 random products and 2900 convolutions of one to
 // four plane pairs, replayed as a graph; call after call the AND/POPC kernel, which is launched normally,
 // takes 1.9 us more (the launch gap), the other 0.5, and 1.8 us are added so that neither kind of caller
-// loses.  The choice costs 0.7 % (graph) and 0.3 % (calls) of the faster one's time on average, always the
+// loses.  On 5762 others the choice costs 0.7 % (graph) and 0.3 % (calls) of the faster one's time on average, always the
 // tensor cores 2.6 % and 1.2 % (325 x 313 x 132 W1A1 raw sums: 14.5 us there, 6.2 with AND/POPC), always
-// AND/POPC 85 %.  From five plane pairs on the tensor cores were the faster ones everywhere.
+// AND/POPC 105 %.  From five plane pairs on the tensor cores were the faster ones everywhere.
 static bool planes_tensor_faster(const qnn_gemm_desc *d, const qnn_conv_desc *cv, bool has_thr) {
     const int planes = d->w_bits + d->a_bits, pairs = d->w_bits * d->a_bits, sms = sm_count();
     if (pairs > 4) return true;

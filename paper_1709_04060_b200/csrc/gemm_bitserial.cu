@@ -20,7 +20,8 @@
 // product with 4 to 16 pairs, but 6 % of one with two).
 //
 // The library's own choice takes this kernel for W4A4 up to 2^30 multiply-accumulates, for a single plane
-// pair at middle sizes and where plane pairs are left out; elsewhere the planes are expanded to bytes
+// pair at middle sizes, for few pairs with little work (planes_tensor_faster in api.cu), for depths beyond
+// 2^25 and where plane pairs are left out; elsewhere the planes are expanded to bytes
 // for the tensor cores (gemm_tc.cu), which at 4096^3 W2A2 take 169 us against 1900 here.
 //
 // Tiling: one CTA (8 warps) per 64 x 64 output tile, depth staged 16 words at a

@@ -22,7 +22,9 @@
 //
 // CTA = 16 warps, one CTA per SM, tiles of 32 weight rows (one word of the bit-plane output layout); the
 // warps split the depth of a tile, and meet in shared memory, where warp n finishes column n.  A
-// warp has two buffers of loads in flight, across tiles too (one at the start: 0.4 us slower).
+// warp has two buffers of loads in flight, across tiles too (one at the start: 0.4 us slower).  512
+// threads leave 128 registers each: bytes spill 24 bytes, planes with two blocks of columns 4 to 44
+// (one and two planes with four-word loads), fields none.
 #include "common.cuh"
 #include "planes.cuh"
 
@@ -388,15 +390,15 @@ static bool mv_planes_faster(const qnn_gemm_desc *d) {
 
 // Where this kernel is the faster one of those that take the format (8192 x 8192, us, the other -> this):
 //   fields  two columns on: W2A2 N = 2 10.2 -> 8.0, N = 4 13.0 -> 8.0, N = 16 15.4 -> 12.3 (N = 1 6.2 -> 7.8)
-//   planes  two columns on, or one where there are twelve or more plane pairs to count (8192 x 8192 W2A2
-//           N = 2 8.7 -> 8.3, N = 16 39 -> 14.9; W4A4 N = 1 15.8 -> 14.9), but for small problems:
-//           mv_planes_faster
+//   planes  two columns on, or one where there are twelve or more plane pairs to count (8192 x 8192, weights
+//           in L2: W2A2 N = 4 12.9 -> 8.8, N = 16 38 -> 14.6, N = 2 the same; W4A4 N = 1 14.6 -> 13.1, from
+//           HBM the same), but for small problems: mv_planes_faster
 //   bytes   three columns on: N = 4 26 -> 17, N = 8 35 -> 18 (N = 2 15.9 -> 17.6), and not for small
 //           matrices (1000 x 4096, N = 7: 4.6 -> 4.9)
 //   any     where the others need a second launch that clears the output first (bit planes they set
 //           bit by bit; pad bytes they do not write), the host's second launch decides, call after call
 //           (planes: 4.6 us here, 7.3 there for everything small, and faster here for 677 of 700 random
-//           problems up to 12000 x 9216, although one in three takes up to 3 us longer on the device;
+//           problems up to 12000 x 9216, although one in five takes longer on the device, up to 3 us;
 //           fields N = 1 10.2 -> 8.1, bytes 4096 x 9216 N = 1 12.8 -> 11.4); bytes only below 2^26
 //           elements (8192 x 8192: 16.1 there, 17 here), planes with one column below 2^24 (from there on
 //           the two launches take less time on the device: 66.9 against 67.6 us for the batch-1 chain as

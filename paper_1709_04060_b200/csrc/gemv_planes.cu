@@ -10,7 +10,8 @@
 // a shuffle reduction, then lane n counts the thresholds of column n (Section 2.1.1).
 // Columns are handled four at a time (blockIdx.y); more than four columns re-read
 // the weights from L2.  The library takes this kernel for one column and fewer than twelve plane pairs,
-// on the forced bit-serial path, and where plane pairs are left out; else gemv_mma.cu.
+// for small products where little is counted (mv_planes_faster in gemv_mma.cu), on the forced
+// bit-serial path, and where plane pairs are left out; else gemv_mma.cu.
 #include "common.cuh"
 
 namespace qnn {
