@@ -421,16 +421,10 @@ static qnn_status mv_launch(const MvParams &p, size_t smem, cudaStream_t s) {
     static std::atomic<bool> attr_done[QNN_MAX_DEVICES];           // per instantiation and device
     const int dev = current_device();
     if (dev < 0 || !allow_smem(kern, MV_SMEM_MAX, attr_done[dev])) return QNN_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.tiles < sm_count() ? p.tiles : sm_count())); cfg.blockDim = dim3(MV_THREADS);
-    cfg.dynamicSmemBytes = smem; cfg.stream = s;
     // programmatic dependent launch: a CTA has an SM's registers to itself, so early placement cannot
     // crowd several onto one SM; nothing is read before griddepcontrol.wait
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) return QNN_ERR_CUDA;
+    const dim3 grid((unsigned)(p.tiles < sm_count() ? p.tiles : sm_count()));
+    if (launch_pdl<MvParams>(kern, grid, MV_THREADS, smem, s, p) != cudaSuccess) return QNN_ERR_CUDA;
     count_launch();
     return launch_status();
 }
