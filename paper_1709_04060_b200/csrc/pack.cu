@@ -77,13 +77,20 @@ __device__ __forceinline__ uint32_t container4(uint32_t x, int bits, int enc) {
 // Bit planes -> 8-bit containers: one thread per plane word, i.e. 32 consecutive depth indices and two
 // 16-byte stores (one where the row ends in the word's first half).  Four bits of a plane become four
 // bytes by one multiplication (bit b of the nibble lands in bit 0 of byte b); plane i adds them shifted
-// by i.  One launch widens one operand, or two (the map and the filters of a convolution).
+// by i.  Bound by the stores at large sizes (16384 x 8192, four planes: 44 us = 4.6 TB/s) and by one
+// load's latency and the fetch of the code at small ones.  A lone operand has a kernel for each number of
+// planes, whose loads leave together, in CTAs of 128 threads (against one loop over the planes and 256
+// threads: 378 x 494, six planes 2.5 -> 1.9 us; 4096 x 4096, four planes 6.9 -> 5.9).  The map and the
+// filters of a convolution share a launch, which keeps the loop and the larger CTAs: the tensor-core
+// kernel behind it is placed while this one drains, and twice the CTAs (13 x 16 x 10 x 128 -> 149, 3 x 3,
+// W1A4, call after call: 10.5 -> 11.2 us) or more code (11.4) delay that.
 struct WidenOp {
     const uint32_t *planes;
     uint4 *packed;
     long long words;           // rows * kw
     int K, kw, chunks, bits, enc;
 };
+template <int BITS>       // p.bits, or 0: a loop over them
 __device__ __forceinline__ void widen_word(const WidenOp &p, long long idx) {
     long long r;
     if (p.words <= 0x7fffffffll) r = (unsigned)idx / (unsigned)p.kw; else r = idx / p.kw;
@@ -91,13 +98,22 @@ __device__ __forceinline__ void widen_word(const WidenOp &p, long long idx) {
     uint32_t o[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) o[q] = 0u;
-#pragma unroll 4
-    for (int i = 0; i < p.bits; ++i) {
-        const uint32_t x = __ldg(p.planes + i * p.words + idx);
+    auto load = [&](int i) { return __ldg(p.planes + i * p.words + idx); };
+    auto add = [&](int i, uint32_t x) {
         // SIGNED: the top plane is the sign, which also fills the container's upper bits
         const uint32_t mul = (p.enc == QNN_ENC_SIGNED && i == p.bits - 1) ? ((0xFFu << i) & 0xFFu) : (1u << i);
 #pragma unroll
         for (int q = 0; q < 8; ++q) o[q] |= ((((x >> (4 * q)) & 0xFu) * 0x00204081u) & 0x01010101u) * mul;
+    };
+    if (BITS > 0) {
+        uint32_t w[BITS > 0 ? BITS : 1];
+#pragma unroll
+        for (int i = 0; i < BITS; ++i) w[i] = load(i);
+#pragma unroll
+        for (int i = 0; i < BITS; ++i) add(i, w[i]);
+    } else {
+#pragma unroll 4
+        for (int i = 0; i < p.bits; ++i) add(i, load(i));
     }
     if (p.enc == QNN_ENC_BIPOLAR) {
         // bit 1 -> +1, bit 0 -> -1; pad bytes past K stay zero
@@ -113,11 +129,18 @@ __device__ __forceinline__ void widen_word(const WidenOp &p, long long idx) {
     dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
     if (2 * c + 1 < p.chunks) dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
 }
-__global__ void __launch_bounds__(256) planes_to_int8_kernel(const WidenOp a, const WidenOp b) {
+constexpr int WIDEN_THREADS = 128, WIDEN_PAIR_THREADS = 256;
+template <int BITS>
+__global__ void __launch_bounds__(WIDEN_THREADS) planes_to_int8_kernel(const WidenOp a) {
     pdl_trigger();        // a tensor-core kernel queued behind may set up while this one drains
     const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.words; i += step) widen_word<BITS>(a, i);
+}
+__global__ void __launch_bounds__(WIDEN_PAIR_THREADS) planes_to_int8_pair_kernel(const WidenOp a, const WidenOp b) {
+    pdl_trigger();
+    const long long step = (long long)gridDim.x * blockDim.x;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.words + b.words; i += step) {
-        if (i < a.words) widen_word(a, i); else widen_word(b, i - a.words);
+        if (i < a.words) widen_word<0>(a, i); else widen_word<0>(b, i - a.words);
     }
 }
 
@@ -208,10 +231,21 @@ static WidenOp widen_op(const qnn_pack_desc *d, const void *planes, void *packed
 }
 qnn_status planes_to_int8_launch(const qnn_pack_desc *d, const void *planes, void *packed, cudaStream_t s,
                                  const qnn_pack_desc *d2, const void *planes2, void *packed2) {
-    const int threads = 256;
     const WidenOp a = widen_op(d, planes, packed), b = widen_op(d2, planes2, packed2);
+    const int threads = d2 ? WIDEN_PAIR_THREADS : WIDEN_THREADS;
     const long long want = (a.words + b.words + threads - 1) / threads, cap = (long long)sm_count() * 16;
-    planes_to_int8_kernel<<<(unsigned)(want < cap ? want : cap), threads, 0, s>>>(a, b);
+    const unsigned grid = (unsigned)(want < cap ? want : cap);
+    if (d2) {
+        planes_to_int8_pair_kernel<<<grid, threads, 0, s>>>(a, b);
+    } else {
+#define QNN_WIDEN_CASE(B_) case B_: planes_to_int8_kernel<B_><<<grid, threads, 0, s>>>(a); break;
+        switch (a.bits) {
+            QNN_WIDEN_CASE(1) QNN_WIDEN_CASE(2) QNN_WIDEN_CASE(3) QNN_WIDEN_CASE(4)
+            QNN_WIDEN_CASE(5) QNN_WIDEN_CASE(6) QNN_WIDEN_CASE(7) QNN_WIDEN_CASE(8)
+            default: return QNN_ERR_UNSUPPORTED;
+        }
+#undef QNN_WIDEN_CASE
+    }
     count_launch();
     return launch_status();
 }

@@ -70,3 +70,10 @@ def test_packed_in_packed_out_pipeline(qb, w, a):
     torch.cuda.synchronize()
     got = decode_out(out.cpu().numpy().view(np.uint8).reshape(-1), BITPLANES, case.out_bits, N, M, False)
     assert np.array_equal(got, orc.qgemm(case.W, case.At, case.thr).T)
+
+
+@pytest.mark.parametrize("bits", [5, 6, 7])
+@pytest.mark.parametrize("enc", [synth.UNSIGNED, synth.SIGNED])
+def test_planes_to_containers_of_other_widths(qb, bits, enc):
+    """The kernel is compiled once per number of planes."""
+    test_planes_to_containers(qb, bits, enc)
