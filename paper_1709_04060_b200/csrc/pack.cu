@@ -77,10 +77,10 @@ __device__ __forceinline__ uint32_t container4(uint32_t x, int bits, int enc) {
 // Bit planes -> 8-bit containers: one thread per plane word, i.e. 32 consecutive depth indices and two
 // 16-byte stores (one where the row ends in the word's first half).  Four bits of a plane become four
 // bytes by one multiplication (bit b of the nibble lands in bit 0 of byte b); plane i adds them shifted
-// by i.  Bound by the stores at large sizes (16384 x 8192, four planes: 44 us = 4.6 TB/s) and by one
+// by i.  Bound by the stores at large sizes (16384 x 8192, four planes: 38 us = 5.3 TB/s) and by one
 // load's latency and the fetch of the code at small ones.  A lone operand has a kernel for each number of
 // planes, whose loads leave together, in CTAs of 128 threads (against one loop over the planes and 256
-// threads: 378 x 494, six planes 2.5 -> 1.9 us; 4096 x 4096, four planes 6.9 -> 5.9).  The map and the
+// threads: 378 x 494, six planes 2.5 -> 1.8 us; 4096 x 4096, four planes 6.9 -> 5.9).  The map and the
 // filters of a convolution share a launch, which keeps the loop and the larger CTAs: the tensor-core
 // kernel behind it is placed while this one drains, and twice the CTAs (13 x 16 x 10 x 128 -> 149, 3 x 3,
 // W1A4, call after call: 10.5 -> 11.2 us) or more code (11.4) delay that.
