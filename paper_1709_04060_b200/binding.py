@@ -1,4 +1,5 @@
-"""ctypes binding of the C ABI in ``include/qnn.h`` (argument marshalling only).
+"""Binding of the C ABI in ``include/qnn.h`` (argument marshalling only): ctypes, and for the calls that
+launch kernels an extension module (``csrc/fastcall.c``) in front of it.
 
 The ``qnn_*`` functions mirror the C entry points one to one and return the
 status code.  Pointer arguments accept a ``torch.Tensor`` (its ``data_ptr()``
@@ -163,6 +164,35 @@ def _stream(stream):
 
 _initialized = torch.cuda.is_initialized
 
+try:
+    from . import _fastcall
+except ImportError:              # a tree whose extension is not built: the same calls through ctypes
+    _fastcall = None
+
+
+def _entry(name, kinds, desc_type):
+    """The entry point ``name`` as a callable; kinds of its arguments: d descriptor, p pointer, n number,
+    s stream.  The extension takes the plain forms (0.8 us of host time instead of 2.2) and hands every
+    other one to the ctypes call below."""
+    fn = getattr(_lib, name)
+    convert = [{"d": ctypes.byref, "p": _ptr, "n": lambda x: x, "s": _stream}[k] for k in kinds]
+
+    def slow(*args):
+        return fn(*[c(x) for c, x in zip(convert, args)])
+
+    if _fastcall is None:
+        return slow
+    return _fastcall.bind(ctypes.cast(fn, _vp).value, kinds, desc_type, _Tensor, slow, _raw_stream, _device, _initialized)
+
+
+_pack = _entry("qnn_pack", "dpps", qnn_pack_desc)
+_planes_to_int8 = _entry("qnn_planes_to_int8", "dpps", qnn_pack_desc)
+_qgemm = _entry("qnn_qgemm", "dpppppns", qnn_gemm_desc)
+_im2col = _entry("qnn_im2col", "dpps", qnn_conv_desc)
+_qconv = _entry("qnn_qconv", "dpppppns", qnn_conv_desc)
+_qconv_static = _entry("qnn_qconv_static", "dpppps", qnn_conv_desc)
+_maxpool = _entry("qnn_maxpool", "dpps", qnn_pool_desc)
+
 
 # ---- one-to-one entry points -------------------------------------------------
 def qnn_version() -> int:
@@ -186,11 +216,11 @@ def qnn_packed_bytes(d: qnn_pack_desc) -> int:
 
 
 def qnn_pack(d, logical, packed, stream=None) -> int:
-    return _lib.qnn_pack(ctypes.byref(d), _ptr(logical), _ptr(packed), _stream(stream))
+    return _pack(d, logical, packed, stream)
 
 
 def qnn_planes_to_int8(d, planes, containers, stream=None) -> int:
-    return _lib.qnn_planes_to_int8(ctypes.byref(d), _ptr(planes), _ptr(containers), _stream(stream))
+    return _planes_to_int8(d, planes, containers, stream)
 
 
 def qnn_gemm_workspace_bytes(d) -> int:
@@ -217,8 +247,7 @@ def qnn_qgemm_kernel_name(d, has_thresholds: bool = True):
 
 
 def qnn_qgemm(d, W, A, thr, out, workspace=None, workspace_bytes=0, stream=None) -> int:
-    return _lib.qnn_qgemm(ctypes.byref(d), _ptr(W), _ptr(A), _ptr(thr), _ptr(out),
-                          _ptr(workspace), workspace_bytes, _stream(stream))
+    return _qgemm(d, W, A, thr, out, workspace, workspace_bytes, stream)
 
 
 def qnn_conv_out_h(d) -> int:
@@ -246,12 +275,11 @@ def qnn_conv_out_bytes(d, has_thresholds: bool) -> int:
 
 
 def qnn_im2col(d, inp, lowered, stream=None) -> int:
-    return _lib.qnn_im2col(ctypes.byref(d), _ptr(inp), _ptr(lowered), _stream(stream))
+    return _im2col(d, inp, lowered, stream)
 
 
 def qnn_qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream=None) -> int:
-    return _lib.qnn_qconv(ctypes.byref(d), _ptr(Wpacked), _ptr(inp), _ptr(thr), _ptr(out),
-                          _ptr(workspace), workspace_bytes, _stream(stream))
+    return _qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream)
 
 
 QNN_QCONV_STATIC_MAX_BYTES = 16 << 20
@@ -260,12 +288,11 @@ QNN_QCONV_STATIC_MAX_BYTES = 16 << 20
 def qnn_qconv_static(d, Wpacked, inp, thr, out, stream=None) -> int:
     """qnn_qconv without a workspace argument: the lowered matrix goes into a fixed
     array inside the library, so the call allocates nothing (see include/qnn.h)."""
-    return _lib.qnn_qconv_static(ctypes.byref(d), _ptr(Wpacked), _ptr(inp), _ptr(thr), _ptr(out),
-                                 _stream(stream))
+    return _qconv_static(d, Wpacked, inp, thr, out, stream)
 
 
 def qnn_maxpool(d, inp, out, stream=None) -> int:
-    return _lib.qnn_maxpool(ctypes.byref(d), _ptr(inp), _ptr(out), _stream(stream))
+    return _maxpool(d, inp, out, stream)
 
 
 def qnn_streamline(channels, qthr, acc_lo: int, acc_hi: int):

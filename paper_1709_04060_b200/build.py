@@ -1,4 +1,5 @@
-"""Compile the CUDA sources in ``csrc/`` into ``libqnn_b200.so`` (sm_100a only).
+"""Compile the CUDA sources in ``csrc/`` into ``libqnn_b200.so`` (sm_100a only), and
+``csrc/fastcall.c`` into the extension module the binding makes its calls through.
 
 nvcc cross-compiles without a GPU.  Objects are rebuilt only when their source
 (or a header) is newer; translation units compile in parallel.
@@ -6,6 +7,7 @@ nvcc cross-compiles without a GPU.  Objects are rebuilt only when their source
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -13,6 +15,7 @@ CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 OBJ_DIR = os.path.join(_HERE, "_build")
 LIB = os.path.join(_HERE, "libqnn_b200.so")
+FASTCALL = os.path.join(_HERE, "_fastcall.so")       # the binding's host path (csrc/fastcall.c)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -59,6 +62,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if todo or not os.path.exists(LIB):
         cmd = ["nvcc", "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"]
         subprocess.run(cmd, check=True)
+    src = os.path.join(CSRC, "fastcall.c")
+    if force or not os.path.exists(FASTCALL) or os.path.getmtime(FASTCALL) < os.path.getmtime(src):
+        subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"], src, "-o", FASTCALL], check=True)
     return LIB
 
 
