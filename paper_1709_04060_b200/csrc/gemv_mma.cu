@@ -5,35 +5,39 @@
 // instructions (mma.sync m16n8k32, int8 x int8 -> int32: exact, so the result is the integer that the
 // bit-serial sum of Section 3.1 equals); T(x, t) of Section 2.1.1 is applied before anything is stored.
 //
-// What bounds it: up to eight columns the weights' latency and the fill and drain of an SM (8192 x 8192
-// W2A2 fields, 16.8 MB: 8.0 us for 2 to 4 columns, against 10 to 13 in the other forms; 2.5 us at the copy
-// rate), beyond them also the int8 rate of mma.sync, which is no more than that of dp4a here (12.3 us
-// at 16).  The per-lane operand layout lets a loaded word feed the multiplication without a trip
-// through shared or tensor memory, so columns up to eight come at one price and an SM holds nothing but
-// loads in flight (16 warps x 8 x 16 bytes per lane, twice); tcgen05 would need every widened byte
-// written to shared or tensor memory first, and 128-row tiles.  Any order of the depth gives the same
-// sum, so weights and activations only have to agree on one:
+// Up to eight columns, sixteen weight rows are the instruction's first operand and the columns its second;
+// beyond, the columns are the first and eight weight rows the second.  A warp owns a slice of the depth for
+// all of its CTA's rows, so its part of the activations is loaded once, in the lane layout of the
+// instruction, and stays in registers (up to 64 a lane): no shared memory, no barrier and nothing else than
+// the weights' own loads between the start and the last row.  Rows are dealt in groups of eight, 8192 to 148
+// SMs as 7 groups each (99 % even); a group is one byte of a bit-plane row.  A depth that the registers of
+// 16 warps do not hold is walked in passes; a shallow one leaves warps over, which take other groups.
+// Partial sums of all groups meet in shared memory once, at the end.
+//
+// Any order of the depth gives the same sum, so weights and activations only have to agree on one:
 //   planes   a lane's word gives 32 elements, eight registers in the order of expand_word; the
-//            activation words are widened once per CTA by the same function
+//            activation words are widened by the same function
 //   fields   a word masked at field position s holds four consecutive depth elements
 //   bytes    a word is four elements as it stands
-// Weights enter as unsigned offsets from the encoding's minimum (a bipolar one as its bit); the column
-// sums of the activations correct for the offset, as in the packed-fields kernels.
+// A field that a mask leaves in the upper half of its byte pair is not shifted down: it counts 2^F times
+// and has accumulators of its own, which are shifted back (exactly) when a group ends.  That leaves one
+// AND a register with 4-bit fields and 1.25 to 1.4 instructions otherwise.
 //
-// CTA = 16 warps, one CTA per SM, tiles of 32 weight rows (one word of the bit-plane output layout); the
-// warps split the depth of a tile, and meet in shared memory, where warp n finishes column n.  A
-// warp has two buffers of loads in flight, across tiles too (one at the start: 0.4 us slower).  512
-// threads leave 128 registers each: bytes spill 24 bytes, planes with two blocks of columns 4 to 44
-// (one and two planes with four-word loads), fields none.
+// Weights enter as unsigned offsets from the encoding's minimum (a bipolar one as its bit); the column
+// sums of the activations, one more product with a column of ones, correct for the offset.
+//
+// What bounds it: two columns or so the weights (8192 x 8192 W2, 16.8 MB, 7.0 us; a plain read of as many bytes
+// call after call takes 3.0 from L2 and more from HBM); 16 columns of bytes the activations, which every SM
+// reads whole (131 KB each, 19 MB from L2).  8192 x 8192, us, activations staged through shared memory by the
+// whole CTA -> here: planes W2A2 N = 2 8.4 -> 7.0, 4 9.1 -> 7.2, 16 14.8 -> 9.1, W4A4 N = 1 13.5 -> 11.5;
+// fields W2 N = 2 7.8 -> 7.2, 16 12.3 -> 10.1, W4 N = 16 13.1 -> 11.9; bytes 1000 x 4096 N = 7 5.2 -> 3.3.
 #include "common.cuh"
 #include "planes.cuh"
 
 namespace qnn {
 
 constexpr int MV_WARPS = 16, MV_THREADS = 32 * MV_WARPS;
-constexpr int MV_ROWS = 32;             // weight rows per tile
 constexpr int MV_COLS = 16;             // most columns
-constexpr int MV_PART_PITCH = 36;       // partial sums [column][row], row pitch without bank conflicts
 constexpr size_t MV_SMEM_MAX = SMEM_LIMIT;
 
 enum { MV_PLANES = 0, MV_FIELDS = 1, MV_BYTES = 2 };
@@ -43,23 +47,36 @@ struct MvParams {
     const int32_t *thr;    // [M][n_thr] or null
     void *out;
     int M, N, K;
-    int tiles, steps;      // 32-row tiles; steps of the depth per row
-    int units;             // loads (of V words) per weight row, per plane
+    int groups, per;       // groups of eight weight rows, in all and per CTA
+    int units;             // loads (of V words) per weight row and plane
+    int dsplit, rsplit;    // warps that share a row's depth; products that a CTA works on at a time
+    int passes;            // parts of the depth, each held in registers as a whole
     long long w_pitch;     // bytes between weight rows
     long long w_plane;     // bytes between weight planes
     int a_bits, a_kind;    // planes: activation planes, PL_* kind
     int a_pitch;           // bytes between activation rows (planes: of one plane)
-    int col_pitch;         // shared-memory bytes between activation columns
-    int a_signed, w_scale, w_off;
+    int w_scale, w_off;
     uint32_t w_flip;       // planes: flips the top plane of a signed weight (offset binary)
     int out_bits, out_fmt, ld_out;
 };
 
 template <bool W_SIGNED, bool A_SIGNED>
-__device__ __forceinline__ void mv_mma(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ void mv_mma(int (&d)[4], uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, const uint32_t (&a)[2]) {
 #define QNN_MV_MMA(WT_, AT_)                                                                                              \
     asm volatile("mma.sync.aligned.m16n8k32.row.col.s32." WT_ "." AT_ ".s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};" \
-                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1))
+                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(w0), "r"(w1), "r"(w2), "r"(w3), "r"(a[0]), "r"(a[1]))
+    if (W_SIGNED && A_SIGNED) QNN_MV_MMA("s8", "s8");
+    else if (W_SIGNED) QNN_MV_MMA("s8", "u8");
+    else if (A_SIGNED) QNN_MV_MMA("u8", "s8");
+    else QNN_MV_MMA("u8", "u8");
+#undef QNN_MV_MMA
+}
+// The same with the activations as the 16-row operand (two blocks of columns) and eight weight rows.
+template <bool W_SIGNED, bool A_SIGNED>
+__device__ __forceinline__ void mv_mma16(int (&d)[4], const uint32_t (&a)[4], uint32_t w0, uint32_t w1) {
+#define QNN_MV_MMA(WT_, AT_)                                                                                              \
+    asm volatile("mma.sync.aligned.m16n8k32.row.col.s32." AT_ "." WT_ ".s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};" \
+                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(w0), "r"(w1))
     if (W_SIGNED && A_SIGNED) QNN_MV_MMA("s8", "s8");
     else if (W_SIGNED) QNN_MV_MMA("s8", "u8");
     else if (A_SIGNED) QNN_MV_MMA("u8", "s8");
@@ -67,315 +84,440 @@ __device__ __forceinline__ void mv_mma(int (&d)[4], uint32_t a0, uint32_t a1, ui
 #undef QNN_MV_MMA
 }
 
-__device__ __forceinline__ uint4 mv_lds(uint32_t a) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-    return v;
-}
-
-// V words of streamed weights (not kept in L1: nothing reads them again).
-template <int V>
+// V words of global memory.  volatile: the loads stay where they are written, all of a warp's first ones
+// ahead of everything that waits for one of them.  Whole 16-byte units of weights are streamed (nothing
+// reads them again); smaller ones leave the rest of their sector to the warp's next load.
+template <int V, bool STREAM>
 __device__ __forceinline__ void mv_load(uint32_t *w, const uint8_t *p) {
-    if (V == 4) {
-        const uint4 x = __ldcs(reinterpret_cast<const uint4 *>(p));
-        w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
-    } else if (V == 2) {
-        const uint2 x = __ldcs(reinterpret_cast<const uint2 *>(p));
-        w[0] = x.x; w[1] = x.y;
-    } else {
-        w[0] = __ldcs(reinterpret_cast<const uint32_t *>(p));
-    }
+    if (V == 4 && STREAM)
+        asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1 % V]), "=r"(w[2 % V]), "=r"(w[3 % V]) : "l"(p));
+    else if (V == 4)
+        asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1 % V]), "=r"(w[2 % V]), "=r"(w[3 % V]) : "l"(p));
+    else if (V == 2)
+        asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1 % V]) : "l"(p));
+    else
+        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w[0]) : "l"(p));
 }
 
-// Shared-memory offset of 16-byte unit u of an activation column (fields).  The four lanes of a row read
-// both halves of two neighbouring groups of 32 S bytes: where a group is a whole number of bank rows
-// (S = 4, 8) 32 pad bytes per group keep them apart.
-template <int S>
-__device__ __forceinline__ uint32_t mv_field_unit(uint32_t u) { return S == 2 ? 16u * u : 16u * u + 32u * (u / (2 * S)); }
+// A word of every plane of a weight row -> eight registers of four bytes, in pairs: pair k holds the
+// elements that registers mv_slot(k) and mv_slot(k) + mv_next of expand_word hold, times 2^F for the odd
+// pairs (F: 1, 2, 4 for 1, 2 and 3-4 planes).
+template <int B> constexpr int mv_field = B == 1 ? 1 : (B == 2 ? 2 : 4);
+template <int B> constexpr int mv_next = B == 1 ? 2 : 1;
+template <int B> __host__ __device__ constexpr int mv_slot(int k) {
+    return B == 1 ? (k & 1) + 4 * (k >> 1) : (B == 2 ? 2 * (k & 1) + 4 * (k >> 1) : 4 * (k & 1) + 2 * (k >> 1));
+}
+template <int B>
+__device__ __forceinline__ void mv_expand(const uint32_t *w, uint32_t (&o)[4][2]) {
+    if (B == 1) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) o[k][i] = (w[0] >> (4 * (k >> 1) + 2 * i)) & (k & 1 ? 0x02020202u : 0x01010101u);
+        return;
+    }
+    const uint32_t e[2] = {(w[0] & 0x55555555u) | ((w[1] << 1) & 0xAAAAAAAAu), ((w[0] >> 1) & 0x55555555u) | (w[1] & 0xAAAAAAAAu)};
+    if (B == 2) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) o[k][i] = (e[i] >> (4 * (k >> 1))) & (k & 1 ? 0x0C0C0C0Cu : 0x03030303u);
+        return;
+    }
+    const uint32_t w3 = B == 4 ? w[3] : 0u;
+    const uint32_t f[2] = {(w[2] & 0x55555555u) | ((w3 << 1) & 0xAAAAAAAAu), ((w[2] >> 1) & 0x55555555u) | (w3 & 0xAAAAAAAAu)};
+    const uint32_t x[4] = {(e[0] & 0x33333333u) | ((f[0] << 2) & 0xCCCCCCCCu), (e[1] & 0x33333333u) | ((f[1] << 2) & 0xCCCCCCCCu),
+                           ((e[0] >> 2) & 0x33333333u) | (f[0] & 0xCCCCCCCCu), ((e[1] >> 2) & 0x33333333u) | (f[1] & 0xCCCCCCCCu)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) o[k][i] = x[2 * (k >> 1) + i] & (k & 1 ? 0xF0F0F0F0u : 0x0F0F0F0Fu);
+}
 
-// SRC: MV_*; B: weight planes, or bits per field; V: words per load; NT: blocks of eight columns.
-// A step of the depth is what the four lanes of a row load at once: 4 V words of every plane, or 64
-// bytes.  U steps are in flight per warp and buffer.
-template <int SRC, int B, int V, int NT, bool W_SIGNED, bool A_SIGNED>
+// Activation registers of a product: for each half of its depth, the column g and (NT == 2) g + 8.
+#define MV_AT(HALF_, BLOCK_) ((HALF_) * NT + (BLOCK_))
+// Ints between the rows of a group's partial sums: two blocks of columns are stored column by column.
+__host__ __device__ constexpr int mv_part_pitch(int nt) { return nt == 2 ? 20 : 8; }
+
+// SRC: MV_*; B: weight planes, or bits per field; V: words per load; NT: blocks of eight columns; U: steps
+// of a warp per product and pass.  A step is what the four lanes of a row load at once: 4 V words of every
+// plane, or 64 bytes.
+template <int SRC, int B, int V, int NT, int U, bool W_SIGNED, bool A_SIGNED>
 __global__ void __launch_bounds__(MV_THREADS, 1)
 gemv_mma_kernel(const MvParams p) {
     constexpr int PL = SRC == MV_PLANES ? B : 1;                   // loads per row and step
-    constexpr int U = 8 / (PL * V) > 0 ? 8 / (PL * V) : 1;
-    constexpr int S = SRC == MV_FIELDS ? 8 / B : 1;
+    constexpr int S = SRC == MV_FIELDS ? 8 / B : 1;                // field positions of a byte
+    constexpr int RP = SRC == MV_PLANES ? 4 : 1;                   // activation planes as loaded
+    constexpr int AP = SRC == MV_PLANES ? 4 * V : 2 * S;           // products per step
+    constexpr int G = 3 - NT;                                      // groups per product: 16 weight rows, or 8 against 16 columns
+    constexpr int PITCH = mv_part_pitch(NT);
+    // two buffers of up to 16 registers a lane: steps per buffer, of one product's groups or of several
+    // (of few: a launch that runs a product or two per warp waits for every line of code it fetches, also of
+    // the products it skips)
+    constexpr int FIT = 16 / (G * PL * V), STEPS = FIT >= 8 ? 8 : (FIT >= 4 ? 4 : (FIT >= 2 ? 2 : 1)), MOST = AP >= 8 ? 2 : 4;
+    constexpr int UB = STEPS < U ? STEPS : U, Q = STEPS / UB < MOST ? STEPS / UB : MOST, NB = U / UB;
+    constexpr int TURN = NB == 1 ? 2 : NB;                         // buffers per turn of the loop (even)
+    constexpr int FIELD = SRC == MV_PLANES ? mv_field<B> : (SRC == MV_FIELDS ? B : 0);
     extern __shared__ __align__(16) uint8_t mv_smem[];
-    int *part = reinterpret_cast<int *>(mv_smem);                  // [warp][8 NT columns][MV_PART_PITCH]
-    uint8_t *cols = mv_smem + MV_WARPS * 8 * NT * MV_PART_PITCH * 4;
+    int *part = reinterpret_cast<int *>(mv_smem);                  // [group][depth slice][8 rows][PITCH: 8 NT columns]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int d = warp % p.dsplit, r0 = warp / p.dsplit;
+    const int g0 = blockIdx.x * p.per, ng = min(p.per, p.groups - g0);
+    const int n_thr = p.thr ? (1 << p.out_bits) - 1 : 0;
+    int *thr_s = part + (size_t)p.per * p.dsplit * 8 * PITCH;
     pdl_wait();
     pdl_trigger();
 
-    // ---- the warp's work: steps warp, warp + 16, ... of every tile of this CTA, U at a time
-    int ld_tile = blockIdx.x, ld_step = warp;
-    uint32_t w[2][U][4][PL][V];
-    auto load = [&](uint32_t (&x)[U][4][PL][V]) {
-        const bool live = ld_tile < p.tiles;
+    // thresholds of the CTA's rows, on their way while the weights stream
+    if (p.thr) {
+        const int32_t *first = p.thr + (size_t)g0 * 8 * n_thr;
+        const int count = min(ng * 8, p.M - g0 * 8) * n_thr;
+        for (int i = threadIdx.x; i < count; i += (int)blockDim.x)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(thr_s + i)), "l"(first + i) : "memory");
+    }
+
+    uint32_t w[2][Q][UB][G][PL][V];
+    // (warps past the plan's only help with the outputs)
+    for (int pass = r0 < p.rsplit ? 0 : p.passes; pass < p.passes; ++pass) {
+        const int unit0 = (pass * p.dsplit + d) * 4 * U + t;       // this lane's first load in a row
+        // steps nb UB .. of the products of ordinal gi .. gi + Q - 1 among this warp's.  No predicates: rows past
+        // the last one repeat it (their sums go nowhere), and loads past a row's end its last load (they meet
+        // activations that are zero).
+        auto load = [&](uint32_t (&x)[Q][UB][G][PL][V], int gi, int nb) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int unit = (ld_step + u * MV_WARPS) * 4 + t;
-            const bool in = live && unit < p.units;
+            for (int q = 0; q < Q; ++q) {
+                const int prod = r0 + (gi + q) * p.rsplit, m = (g0 + G * prod) * 8 + g;
+                if (G * prod >= ng) continue;                      // uniform
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int m = ld_tile * MV_ROWS + g + 8 * r;
-                const uint8_t *q = p.W + (size_t)m * p.w_pitch + (size_t)unit * (4 * V);
+                for (int i = 0; i < G; ++i) {
+                    const uint8_t *row = p.W + (size_t)min(m + 8 * i, p.M - 1) * p.w_pitch;
 #pragma unroll
-                for (int b = 0; b < PL; ++b) {
-                    if (in && m < p.M) {
-                        mv_load<V>(x[u][r][b], q + (size_t)b * p.w_plane);
-                    } else {
+                    for (int u = 0; u < UB; ++u) {
+                        const uint8_t *at = row + (uint32_t)min(unit0 + 4 * (nb * UB + u), p.units - 1) * (4u * V);
 #pragma unroll
-                        for (int v = 0; v < V; ++v) x[u][r][b][v] = 0u;
+                        for (int b = 0; b < PL; ++b) mv_load<V, true>(x[q][u][i][b], at + (size_t)b * p.w_plane);
                     }
                 }
             }
-        }
-        ld_step += U * MV_WARPS;
-        if (ld_step - warp >= p.steps) { ld_step = warp; ld_tile += gridDim.x; }
-    };
-    load(w[0]);
-    load(w[1]);
+        };
 
-    // ---- activation columns into shared memory, in the order the multiplication reads them
-    if (SRC == MV_PLANES) {
-        // word c of a column: step c / 4V, lane (c mod 4V) / V, word c mod V of the lane; 32 bytes each,
-        // the four lanes' words next to one another
-        const int words = p.steps * 4 * V, kw = p.a_pitch >> 2;
-        for (int i = threadIdx.x; i < p.N * words; i += MV_THREADS) {
-            const int n = i / words, c = i - n * words;
-            uint32_t a[4] = {0u, 0u, 0u, 0u}, o[8];
-            if (c < kw)
-                for (int b = 0; b < p.a_bits; ++b)
-                    a[b] = reinterpret_cast<const uint32_t *>(p.A)[((size_t)b * p.N + n) * kw + c];
-            if (p.a_kind == PL_BIPOLAR) {
-                expand_word<1, PL_BIPOLAR>(a, o);
-                const int left = p.K - 32 * c;                     // +-1 has no zero: nothing past the depth
-                const uint32_t keep = left >= 32 ? 0xFFFFFFFFu : (left <= 0 ? 0u : (1u << left) - 1u);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) o[j] &= ((keep >> j) & 0x01010101u) * 0xFFu;
-            } else if (p.a_kind == PL_SIGNED) {
-                switch (p.a_bits) {
-                    case 1: expand_word<1, PL_SIGNED>(a, o); break;
-                    case 2: expand_word<2, PL_SIGNED>(a, o); break;
-                    case 3: expand_word<3, PL_SIGNED>(a, o); break;
-                    default: expand_word<4, PL_SIGNED>(a, o); break;
-                }
-            } else {
-                expand_word<4, PL_UNSIGNED>(a, o);                 // planes past a_bits are zero
-            }
-            const int step = c / (4 * V), in = c % (4 * V), slot = step * 4 * V + (in % V) * 4 + in / V;
-            uint4 *dst = reinterpret_cast<uint4 *>(cols + (size_t)n * p.col_pitch + 32 * slot);
-            dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-            dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        // Weights that come from HBM go ahead of the activations, which all SMs read from L2 (fields, 8192 x 8192
+        // W2, N = 16: 13.2 -> 11.9 us; bytes, N = 8 13.1 -> 12.1); planes are few activation bytes, and their
+        // widening would have to wait for the weights
+        if (SRC != MV_PLANES) {
+            load(w[0], 0, 0);
+            load(w[1], NB == 1 ? Q : 0, NB == 1 ? 0 : 1);
         }
-    } else {
-        // plain bytes; what lies past the row meets zero weights, but has to be there
-        const int units = p.a_pitch >> 4;
-        for (int i = threadIdx.x; i < p.N * units; i += MV_THREADS) {
-            const int n = i / units, u = i - n * units;
-            *reinterpret_cast<uint4 *>(cols + (size_t)n * p.col_pitch + (SRC == MV_FIELDS ? mv_field_unit<S>(u) : 16u * u)) =
-                reinterpret_cast<const uint4 *>(p.A + (size_t)n * p.a_pitch)[u];
-        }
-    }
-    __syncthreads();
-    int colsum = 0;                                                // warp n: sum of column n
-    if (p.w_off != 0 && warp < p.N) {
-        const int units = SRC == MV_PLANES ? p.steps * 8 * V : p.a_pitch >> 4;
-        for (int u = lane; u < units; u += 32) {
-            const uint4 a = *reinterpret_cast<const uint4 *>(cols + (size_t)warp * p.col_pitch + (SRC == MV_FIELDS ? mv_field_unit<S>(u) : 16u * u));
-            if (A_SIGNED) {
-                colsum = __dp4a((int)a.x, 0x01010101, colsum); colsum = __dp4a((int)a.y, 0x01010101, colsum);
-                colsum = __dp4a((int)a.z, 0x01010101, colsum); colsum = __dp4a((int)a.w, 0x01010101, colsum);
-            } else {
-                colsum = (int)__dp4a(a.x, 0x01010101u, (unsigned)colsum); colsum = (int)__dp4a(a.y, 0x01010101u, (unsigned)colsum);
-                colsum = (int)__dp4a(a.z, 0x01010101u, (unsigned)colsum); colsum = (int)__dp4a(a.w, 0x01010101u, (unsigned)colsum);
-            }
-        }
+        // ---- this warp's slice of the activations, columns g and g + 8: as they lie in memory ...
+        uint32_t act[U][AP][2 * NT], raw[NT][U][RP][V];
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) colsum += __shfl_xor_sync(0xffffffffu, colsum, off);
-    }
-
-    // this lane's column of each block (columns past N read the last one; their sums are not used)
-    uint32_t col_at[NT];
+        for (int h = 0; h < NT; ++h) {
+            const int n = g + 8 * h;
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-        col_at[nt] = (uint32_t)__cvta_generic_to_shared(cols) + (uint32_t)min(8 * nt + g, p.N - 1) * (uint32_t)p.col_pitch;
-
-    const int n_thr = p.thr ? (1 << p.out_bits) - 1 : 0;
-    int acc[2][NT][4];
-    auto multiply = [&](const uint32_t (&x)[U][4][PL][V], int step0) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int step = step0 + u * MV_WARPS;
-            if (step < p.steps) {                                  // uniform
+            for (int u = 0; u < U; ++u) {
+                const int unit = unit0 + 4 * u;
+                const bool in = n < p.N && unit < p.units;
                 if (SRC == MV_PLANES) {
 #pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        uint32_t bq[NT][8];
+                    for (int b = 0; b < 4; ++b) {
 #pragma unroll
-                        for (int nt = 0; nt < NT; ++nt) {
-                            const uint32_t at = col_at[nt] + 32u * (uint32_t)(step * 4 * V + v * 4 + t);
-                            const uint4 lo = mv_lds(at), hi = mv_lds(at + 16u);
-                            bq[nt][0] = lo.x; bq[nt][1] = lo.y; bq[nt][2] = lo.z; bq[nt][3] = lo.w;
-                            bq[nt][4] = hi.x; bq[nt][5] = hi.y; bq[nt][6] = hi.z; bq[nt][7] = hi.w;
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            uint32_t o0[8], o1[8], wa[4], wb[4];
-#pragma unroll
-                            for (int b = 0; b < PL; ++b) {
-                                const uint32_t f = b == PL - 1 ? p.w_flip : 0u;
-                                wa[b] = x[u][2 * h][b][v] ^ f; wb[b] = x[u][2 * h + 1][b][v] ^ f;
-                            }
-                            expand_word<PL, PL_UNSIGNED>(wa, o0);
-                            expand_word<PL, PL_UNSIGNED>(wb, o1);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                                for (int nt = 0; nt < NT; ++nt)
-                                    mv_mma<false, A_SIGNED>(acc[h][nt], o0[2 * j], o1[2 * j], o0[2 * j + 1], o1[2 * j + 1],
-                                                            bq[nt][2 * j], bq[nt][2 * j + 1]);
-                        }
+                        for (int v = 0; v < V; ++v) raw[h][u][b % RP][v] = 0u;
+                        if (in && b < p.a_bits)
+                            mv_load<V, false>(raw[h][u][b % RP], p.A + ((size_t)b * p.N + n) * p.a_pitch + (size_t)unit * (4 * V));
                     }
+                } else if (SRC == MV_FIELDS && S >= 4) {
+                    // The four lanes' 4 S pieces of 16 elements lie one behind the other: lanes 0 and 1 meet the
+                    // even and odd ones of the first half, 2 and 3 of the second.  Loaded four neighbours at a time
+                    // (as many lines as columns, not twice that: 8192 x 8192 N = 16, W2 12.3 -> 10.1 us, W1 10.7 -> 8.8),
+                    // then half of them change places with lane t ^ 2.
+                    uint32_t y[S][4];
+#pragma unroll
+                    for (int s = 0; s < S; ++s) {
+                        const int au = (unit - t) * S + 4 * s + t;
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) y[s][v] = 0u;
+                        if (n < p.N && 16 * au < p.a_pitch) mv_load<4, false>(y[s], p.A + (size_t)n * p.a_pitch + 16 * (size_t)au);
+                    }
+#pragma unroll
+                    for (int s = 0; s < S / 2; ++s)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const uint32_t lo = y[s][v], hi = y[(s + S / 2) % S][v], got = __shfl_xor_sync(0xffffffffu, t < 2 ? hi : lo, 2);
+                            act[u][(4 * s + (v >> 1)) % AP][MV_AT(v & 1, h)] = t < 2 ? lo : got;
+                            act[u][(4 * s + 2 + (v >> 1)) % AP][MV_AT(v & 1, h)] = t < 2 ? got : hi;
+                        }
                 } else {
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
-                        constexpr uint32_t MASK = B == 1 ? 0x01010101u : (B == 2 ? 0x03030303u : (B == 4 ? 0x0F0F0F0Fu : 0xFFFFFFFFu));
-                        uint4 bq[NT];
+                        // fields: half (unit & 1) of 32-byte group unit / 2 meets S pieces of 16 elements
+                        const int au = SRC == MV_FIELDS ? (unit >> 1) * (2 * S) + 2 * s + (unit & 1) : unit;
+                        uint32_t y[4] = {0u, 0u, 0u, 0u};
+                        if (in && 16 * au < p.a_pitch) mv_load<4, false>(y, p.A + (size_t)n * p.a_pitch + 16 * (size_t)au);
 #pragma unroll
-                        for (int nt = 0; nt < NT; ++nt) {
-                            // fields: lane t holds half t & 1 of 32-byte group 2 step + t / 2
-                            const uint32_t unit = SRC == MV_FIELDS ? (uint32_t)((2 * step + (t >> 1)) * 2 * S + 2 * s + (t & 1)) : (uint32_t)(4 * step + t);
-                            bq[nt] = mv_lds(col_at[nt] + (SRC == MV_FIELDS ? mv_field_unit<S>(unit) : 16u * unit));
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            uint32_t o0[4], o1[4];
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) {
-                                o0[v] = SRC == MV_FIELDS ? (x[u][2 * h][0][v] >> (B * s)) & MASK : x[u][2 * h][0][v];
-                                o1[v] = SRC == MV_FIELDS ? (x[u][2 * h + 1][0][v] >> (B * s)) & MASK : x[u][2 * h + 1][0][v];
-                            }
-#pragma unroll
-                            for (int nt = 0; nt < NT; ++nt) {
-                                mv_mma<W_SIGNED, A_SIGNED>(acc[h][nt], o0[0], o1[0], o0[1], o1[1], bq[nt].x, bq[nt].y);
-                                mv_mma<W_SIGNED, A_SIGNED>(acc[h][nt], o0[2], o1[2], o0[3], o1[3], bq[nt].z, bq[nt].w);
-                            }
-                        }
+                        for (int v = 0; v < 4; ++v) act[u][(2 * s + (v >> 1)) % AP][MV_AT(v & 1, h)] = y[v];
                     }
                 }
             }
         }
-    };
+        if (SRC == MV_PLANES) {
+            load(w[0], 0, 0);
+            load(w[1], NB == 1 ? Q : 0, NB == 1 ? 0 : 1);
+        }
+        // ... and planes widened, in the pairs mv_expand forms
+        if (SRC == MV_PLANES) {
+            auto words = [&](auto &&f) {
+#pragma unroll
+                for (int h = 0; h < NT; ++h)
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+#pragma unroll
+                        for (int v = 0; v < V; ++v) f(h, u, v);
+            };
+            if (p.a_bits <= 2)
+                words([&](int h, int u, int v) {
+                    const uint32_t a[4] = {raw[h][u][0][v], raw[h][u][1 % RP][v], 0u, 0u};
+                    uint32_t o[8];
+                    expand_word<2, PL_UNSIGNED>(a, o);             // planes past a_bits are zero
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        act[u][(4 * v + k) % AP][MV_AT(0, h)] = o[mv_slot<B>(k)];
+                        act[u][(4 * v + k) % AP][MV_AT(1, h)] = o[mv_slot<B>(k) + mv_next<B>];
+                    }
+                });
+            else
+                words([&](int h, int u, int v) {
+                    uint32_t a[4], o[8];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) a[b] = raw[h][u][b % RP][v];
+                    expand_word<4, PL_UNSIGNED>(a, o);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        act[u][(4 * v + k) % AP][MV_AT(0, h)] = o[mv_slot<B>(k)];
+                        act[u][(4 * v + k) % AP][MV_AT(1, h)] = o[mv_slot<B>(k) + mv_next<B>];
+                    }
+                });
+            if (p.a_kind == PL_SIGNED) {
+                // two's complement: the lower planes less the top one
+                const uint32_t top = 0x01010101u << (p.a_bits - 1);
+                words([&](int h, int u, int v) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        uint32_t &x = act[u][(4 * v + (k >> 1)) % AP][MV_AT(k & 1, h)];
+                        x = (((x & ~top) | 0x80808080u) - (x & top)) ^ 0x80808080u;
+                    }
+                });
+            } else if (p.a_kind == PL_BIPOLAR) {
+                // +-1 has no zero: nothing past the depth, and nothing in an absent column
+                words([&](int h, int u, int v) {
+                    const int left = g + 8 * h < p.N ? p.K - 32 * ((unit0 + 4 * u) * V + v) : 0;
+                    const uint32_t keep = left >= 32 ? 0xFFFFFFFFu : (left <= 0 ? 0u : (1u << left) - 1u);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        uint32_t &x = act[u][(4 * v + (k >> 1)) % AP][MV_AT(k & 1, h)];
+                        x = ((2u * x | 0x80808080u) - 0x01010101u) ^ 0x80808080u;
+                        x &= ((keep >> (mv_slot<B>(k >> 1) + (k & 1) * mv_next<B>)) & 0x01010101u) * 0xFFu;
+                    }
+                });
+            }
+        }
+        int cs[4] = {0, 0, 0, 0};                                  // column sums, in the layout of the accumulators
+        if (p.w_off != 0) {
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int j = 0; j < AP; ++j) {
+                    if constexpr (NT == 2) mv_mma16<false, A_SIGNED>(cs, act[u][j], 0x01010101u, 0x01010101u);
+                    else mv_mma<false, A_SIGNED>(cs, 0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u, act[u][j]);
+                }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cs[e] *= p.w_off;
+        }
 
-    const int rounds = (p.steps + U * MV_WARPS - 1) / (U * MV_WARPS);      // buffers per tile
-    int cur = 0;
-    for (int tile = blockIdx.x; tile < p.tiles; tile += gridDim.x) {
+        int acc[2][4];                                             // even and odd pairs of registers
+        auto multiply = [&](const uint32_t (&x)[Q][UB][G][PL][V], int gi, int nb) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+            for (int q = 0; q < Q; ++q) {
+                const int prod = r0 + (gi + q) * p.rsplit;
+                if (G * prod >= ng) continue;                      // uniform
+                if (nb == 0) {
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
+                    for (int e = 0; e < 4; ++e) acc[0][e] = acc[1][e] = 0;
+                }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) acc[h][nt][e] = 0;
-        int step = warp;
-        for (int r = 0; r < rounds; ++r, step += U * MV_WARPS) {
-            if (cur == 0) { multiply(w[0], step); load(w[0]); }
-            else { multiply(w[1], step); load(w[1]); }
-            cur ^= 1;
-        }
-        // thresholds of this thread's row, on their way while the partial sums meet
-        const int m = tile * MV_ROWS + lane;
-        int th[15];
-        if (warp < p.N) {
+                for (int ub = 0; ub < UB; ++ub) {
+                    const int u = nb * UB + ub;
+                    if (SRC == MV_PLANES) {
 #pragma unroll
-            for (int q = 0; q < 15; ++q) th[q] = q < n_thr && m < p.M ? __ldg(p.thr + (size_t)m * n_thr + q) : 0x7fffffff;
-        }
-        int *mine = part + warp * (8 * NT * MV_PART_PITCH);
+                        for (int v = 0; v < V; ++v) {
+                            uint32_t o[G][4][2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+                            for (int i = 0; i < G; ++i) {
+                                uint32_t ww[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
+                                for (int b = 0; b < PL; ++b) ww[b] = b == PL - 1 ? x[q][ub][i][b][v] ^ p.w_flip : x[q][ub][i][b][v];
+                                mv_expand<B>(ww, o[i]);
+                            }
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    mine[(8 * nt + 2 * t + (e & 1)) * MV_PART_PITCH + 16 * h + g + 8 * (e >> 1)] = acc[h][nt][e];
-        __syncthreads();
-        if (warp < p.N) {
-            const int n = warp;
-            int x = 0;
+                            for (int k = 0; k < 4; ++k) {
+                                if constexpr (NT == 2) mv_mma16<false, true>(acc[k & 1], act[u][(4 * v + k) % AP], o[0][k][0], o[0][k][1]);
+                                else mv_mma<false, true>(acc[k & 1], o[0][k][0], o[G - 1][k][0], o[0][k][1], o[G - 1][k][1], act[u][(4 * v + k) % AP]);
+                            }
+                        }
+                    } else {
+                        constexpr uint32_t MASK = B == 1 ? 0x01010101u : (B == 2 ? 0x03030303u : (B == 4 ? 0x0F0F0F0Fu : 0xFFFFFFFFu));
 #pragma unroll
-            for (int v = 0; v < MV_WARPS; ++v) x += part[(v * 8 * NT + n) * MV_PART_PITCH + lane];
-            x = p.w_scale * x + p.w_off * colsum;
-            if (!p.thr) {
-                if (m < p.M) reinterpret_cast<int32_t *>(p.out)[(size_t)n * p.M + m] = x;
-            } else {
-                int code = 0;
+                        for (int s = 0; s < S; ++s) {
+                            uint32_t o[G][4];
 #pragma unroll
-                for (int q = 0; q < 15; ++q) code += q < n_thr && x >= th[q] ? 1 : 0;
-                if (m >= p.M) code = 0;
-                if (p.out_fmt == QNN_FMT_INT8) {
-                    if (m < p.ld_out) reinterpret_cast<uint8_t *>(p.out)[(size_t)n * p.ld_out + m] = (uint8_t)code;
-                } else {
-                    const int mw = (p.M + 31) >> 5;
-                    for (int b = 0; b < p.out_bits; ++b) {
-                        const uint32_t bits = __ballot_sync(0xffffffffu, (code >> b) & 1);
-                        if (lane == 0) reinterpret_cast<uint32_t *>(p.out)[((size_t)b * p.N + n) * mw + tile] = bits;
+                            for (int i = 0; i < G; ++i)
+#pragma unroll
+                                for (int v = 0; v < 4; ++v)
+                                    o[i][v] = SRC == MV_FIELDS ? (x[q][ub][i][0][v % V] >> (B * (s & ~1))) & (MASK << (B * (s & 1))) : x[q][ub][i][0][v % V];
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                int (&a)[4] = acc[SRC == MV_FIELDS ? s & 1 : k];
+                                if constexpr (NT == 2) mv_mma16<W_SIGNED, A_SIGNED>(a, act[u][(2 * s + k) % AP], o[0][2 * k], o[0][2 * k + 1]);
+                                else mv_mma<W_SIGNED, A_SIGNED>(a, o[0][2 * k], o[G - 1][2 * k], o[0][2 * k + 1], o[G - 1][2 * k + 1], act[u][(2 * s + k) % AP]);
+                            }
+                        }
+                    }
+                }
+                if (nb == NB - 1) {
+                    int y[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) y[e] = p.w_scale * (acc[0][e] + (acc[1][e] >> FIELD)) + cs[e];
+                    int *dst = part + (((size_t)(G * prod) * p.dsplit + d) * 8 + (NT == 2 ? 2 * t : g)) * PITCH + (NT == 2 ? g : 2 * t);
+                    if constexpr (NT == 2) {
+                        // rows 2 t and 2 t + 1, columns g and g + 8
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            int *q1 = dst + (e & 1) * PITCH + (e >> 1) * 8;
+                            *q1 = pass > 0 ? *q1 + y[e] : y[e];
+                        }
+                    } else {
+                        // rows g of two groups, columns 2 t and 2 t + 1
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            if (2 * prod + i >= ng) continue;
+                            int2 *q1 = reinterpret_cast<int2 *>(dst + i * p.dsplit * 8 * PITCH);
+                            int2 o = make_int2(y[2 * i], y[2 * i + 1]);
+                            if (pass > 0) { const int2 a = *q1; o.x += a.x; o.y += a.y; }
+                            *q1 = o;
+                        }
                     }
                 }
             }
+        };
+        for (int gi = 0; G * (r0 + gi * p.rsplit) < ng; gi += NB == 1 ? 2 * Q : 1) {
+#pragma unroll
+            for (int i = 0; i < TURN; ++i) {
+                multiply(w[i & 1], NB == 1 ? gi + i * Q : gi, NB == 1 ? 0 : i);
+                if (NB == 1) load(w[i & 1], gi + (i + 2) * Q, 0);
+                else load(w[i & 1], i + 2 < NB ? gi : gi + 1, (i + 2) % NB);
+            }
         }
-        __syncthreads();                                           // the partial sums have been read
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+
+    // ---- all partial sums of an output, its thresholds, its code; eight lanes are the rows of a group
+    const int total = ng * 8 * p.N;
+    for (int base = warp * 32; base < total; base += (int)blockDim.x) {
+        const int i = base + lane, row = i & 7, gn = (i >> 3) / p.N, gl = min(gn, ng - 1), n = (i >> 3) - gn * p.N;
+        const int m = (g0 + gl) * 8 + row;
+        const bool ok = i < total;
+        const int *src = part + ((size_t)gl * p.dsplit * 8 + row) * PITCH + n;
+        int x = 0;
+#pragma unroll 8
+        for (int v = 0; v < p.dsplit; ++v) x += src[v * 8 * PITCH];
+        if (!p.thr) {
+            if (ok && m < p.M) reinterpret_cast<int32_t *>(p.out)[(size_t)n * p.M + m] = x;
+            continue;
+        }
+        int code = 0;
+        if (m < p.M)
+            for (int q = 0; q < n_thr; ++q) code += x >= thr_s[(gl * 8 + row) * n_thr + q] ? 1 : 0;
+        if (p.out_fmt == QNN_FMT_INT8) {
+            if (ok && m < p.ld_out) reinterpret_cast<uint8_t *>(p.out)[(size_t)n * p.ld_out + m] = (uint8_t)code;
+        } else {
+            // a group is one byte of the row's words
+            const int mw = (p.M + 31) >> 5;
+            for (int b = 0; b < p.out_bits; ++b) {
+                const uint32_t bits = __ballot_sync(0xffffffffu, (code >> b) & 1) >> (lane & 24);
+                if (ok && row == 0) reinterpret_cast<uint8_t *>(p.out)[((size_t)b * p.N + n) * 4 * mw + g0 + gl] = (uint8_t)bits;
+            }
+        }
     }
 }
 
 // ------------------------------------------------------------------- host side
-struct MvPlan { int src, b, v, units, steps, col_pitch; size_t smem; };
+struct MvPlan { int src, b, v, units, u, dsplit, rsplit, passes, groups, per, threads; size_t smem; };
 
-static bool mv_plan(const qnn_gemm_desc *d, MvPlan *pl) {
+// Activation registers per lane and step, and the steps of a warp per product that kernels are built for:
+// as many as 64 such registers allow, and fewer for shallow depths and few rows.
+static int mv_act_regs(const MvPlan &pl, int nt) { return nt * (pl.src == MV_PLANES ? 8 * pl.v : 4 * (8 / pl.b)); }
+constexpr int mv_steps_least(int regs) { return regs >= 16 ? 1 : (regs == 8 ? 2 : 4); }
+constexpr int mv_steps_most(int regs) { return 64 / regs; }
+
+static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
     if (d->N > MV_COLS) return false;
-    const int nt = d->N > 8 ? 2 : 1;
-    long long col = 0;
+    const int nt = d->N > 8 ? 2 : 1, sms = sm_count();
     if (d->w_fmt == QNN_FMT_BITPLANES) {
         if (d->w_bits > 4 || d->a_bits > 4) return false;
         const int kw = ceil_div(d->K, 32);
         pl->src = MV_PLANES; pl->b = d->w_bits;
-        // Wide loads once they leave every warp a step of its own (and with few planes: registers);
-        // rows that are not whole units go word by word.
-        pl->v = kw % 4 == 0 && kw >= 16 * MV_WARPS && d->w_bits <= 2 ? 4 : (kw % 2 == 0 && kw >= 8 * MV_WARPS ? 2 : 1);
+        // 16-byte loads where rows are whole units of them and two rows' planes fit the registers, else 8-byte
+        // ones where they can be, else words
+        pl->v = kw % 4 == 0 && d->w_bits <= 2 ? 4 : (kw % 2 == 0 ? 2 : 1);
         pl->units = kw / pl->v;
-        pl->steps = ceil_div(pl->units, 4);
-        col = 128ll * pl->steps * pl->v;
-        pl->col_pitch = (int)(col + 16);                           // eight lanes (two columns) on different banks
     } else if (d->w_fmt == QNN_FMT_FIELDS) {
-        const int f = d->w_bits == 1 ? 1 : (d->w_bits == 2 ? 2 : 4), S = 8 / f;
-        const int ldf = 32 * ceil_div(d->K, 32 * S);
-        pl->src = MV_FIELDS; pl->b = f; pl->v = 4;
-        pl->units = ldf / 16;
-        pl->steps = ceil_div(pl->units, 4);
-        col = (long long)pl->steps * 2 * (32 * S + (S == 2 ? 0 : 32));
-        pl->col_pitch = (int)(col + 127) / 128 * 128 + (S == 2 ? 32 : 64);   // two columns on different banks
+        pl->src = MV_FIELDS; pl->b = d->w_bits == 1 ? 1 : (d->w_bits == 2 ? 2 : 4); pl->v = 4;
+        pl->units = 2 * ceil_div(d->K, 32 * (8 / pl->b));
     } else {
         if (d->N > 8) return false;                                // the tiled tensor-core kernel
         pl->src = MV_BYTES; pl->b = 8; pl->v = 4;
         pl->units = round_up(d->K, 16) / 16;
-        pl->steps = ceil_div(pl->units, 4);
-        col = (long long)pl->steps * 64;
-        pl->col_pitch = (int)(col + 127) / 128 * 128 + 64;
     }
-    if (col > (long long)MV_SMEM_MAX) return false;
-    pl->smem = (size_t)MV_WARPS * 8 * nt * MV_PART_PITCH * 4 + (size_t)d->N * pl->col_pitch;
-    return pl->smem <= MV_SMEM_MAX;
+    // rows in whole groups, and in what the output pads its rows to
+    pl->groups = ceil_div(d->M, 8);
+    if (has_thr) pl->groups = d->out_fmt == QNN_FMT_BITPLANES ? 4 * ceil_div(d->M, 32) : 2 * ceil_div(d->M, 16);
+    // depth and rows to warps: fewest steps for the warp with the most; a pass waits for its activations,
+    // which takes about as long as five steps (fields, us, five or more passes of one step -> two of four, W4
+    // 4101 x 9063 N = 11: 11.1 -> 10.2; three of one -> two of two, W2 6154 x 8805 N = 16: 10.8 -> 12.5)
+    const int steps = ceil_div(pl->units, 4), regs = mv_act_regs(*pl, nt), most = mv_steps_most(regs);
+    long long best = 0;
+    for (int u = mv_steps_least(regs); u <= most; u = u < most ? most : most + 1) {
+        const int passes = ceil_div(steps, MV_WARPS * u), ds = ceil_div(steps, u * passes), rs = MV_WARPS / ds;
+        const int fit = (int)((MV_SMEM_MAX - 1024) / (ds * 32 * mv_part_pitch(nt) + 8 * 15 * 4));
+        const int waves = ceil_div(pl->groups, sms * fit), per = ceil_div(pl->groups, sms * waves);
+        const int prods = ceil_div(per, 3 - nt);
+        const long long cost = (long long)waves * passes * (ceil_div(prods, rs) * u + 5);
+        if (best != 0 && cost >= best) continue;
+        best = cost;
+        pl->u = u; pl->passes = passes; pl->dsplit = ds; pl->rsplit = rs < prods ? rs : prods; pl->per = per;
+    }
+    // ... and enough warps for the outputs
+    const int outputs = pl->per * 8 * d->N, want = outputs < 256 ? round_up(outputs, 32) : 256;
+    pl->threads = 32 * pl->dsplit * pl->rsplit > want ? 32 * pl->dsplit * pl->rsplit : want;
+    pl->smem = (size_t)pl->per * (pl->dsplit * 32 * mv_part_pitch(nt) + 8 * 15 * 4);
+    return true;
+}
+
+// What this kernel is taken for: deeper products with several columns, whose activations would be loaded
+// in many passes, are left to the others.
+static bool mv_fits(const qnn_gemm_desc *d) {
+    if (d->N > (d->w_fmt == QNN_FMT_INT8 ? 8 : MV_COLS) || (d->w_fmt == QNN_FMT_BITPLANES && (d->w_bits > 4 || d->a_bits > 4))) return false;
+    return (long long)d->N * round_up(d->K, 32) <= 192 * 1024;
 }
 
 // Bit planes that need no clearing launch: whether this kernel beats the one that counts bits
-// (gemv_planes.cu), by an estimate of both in microseconds.  That one costs a load latency per staged
-// column and plane, one per depth step of a lane, its CTAs and its population counts; this one its fill
-// and drain, the columns it widens, the rounds of tiles and the weights.  Fitted to 3300 random problems
-// (1 to 16 columns, up to 12000 x 9216, every width and encoding, replayed as a graph): the choice costs
-// 0.8 % of the faster one's time on average, always this kernel 14 % (959 x 64, N = 5, W2A1: 2.7 us there,
-// 4.7 here), always the other 49 %.
+// (gemv_planes.cu), by an estimate of both.  That one costs a load latency per staged column and plane, one
+// per depth step of a lane, its CTAs and its population counts; this one its fill and drain, the columns it
+// widens, the rounds of tiles and the weights.  The terms' shares are fitted to random problems; the factor
+// is the point below which counting is the better choice: of 860 problems with 2 to 16 columns (up to 12000
+// x 9216, every width and encoding, replayed as a graph) the choice costs 1.0 % of the faster one's time (at
+// 0.96, as for one column, 10.5 %; always this kernel 0.6 %, but up to 1.4 times as long for little work, call
+// after call); 960 x 64, N = 5, W2A1: 2.7 us there, 2.9 here.
 static bool mv_planes_faster(const qnn_gemm_desc *d) {
     const int kw = ceil_div(d->K, 32), cols = d->N < 4 ? d->N : 4, pairs = d->w_bits * d->a_bits;
     const double ctas = (double)ceil_div(d->M, 8) * ceil_div(d->N, 4), words = (double)d->M * kw;
@@ -384,17 +526,19 @@ static bool mv_planes_faster(const qnn_gemm_desc *d) {
                            (kw % 4 == 0 ? 0.83 * ceil_div(kw, 128) : 0.23 * ceil_div(kw, 32)) +
                            0.011 * pairs * cols * ceil_div(kw, 32) + 2.3e-7 * words * pairs * d->N + 2.44e-3 * ctas;
     const double here = (d->w_bits <= 2 ? 4.8 : 4.0) + (d->N > 8 ? 0.25 : 0.0) + 1.9e-3 * d->N * kw +
-                        1.5 * ((ceil_div(d->M, MV_ROWS) - 1) / sm_count()) + 0.8e-6 * words * d->w_bits;
-    return counted > 0.96 * here;
+                        1.5 * ((ceil_div(d->M, 32) - 1) / sm_count()) + 0.8e-6 * words * d->w_bits;
+    return counted > (d->N >= 2 ? 0.65 : 0.96) * here;
 }
 
 // Where this kernel is the faster one of those that take the format (8192 x 8192, us, the other -> this):
-//   fields  two columns on: W2A2 N = 2 10.2 -> 8.0, N = 4 13.0 -> 8.0, N = 16 15.4 -> 12.3 (N = 1 6.2 -> 7.8)
+//   fields  two columns on: W2A2 N = 2 10.2 -> 7.2, N = 4 13.0 -> 7.3, N = 16 15.4 -> 9.5 (N = 1 6.0 -> 7.1)
 //   planes  two columns on, or one where there are twelve or more plane pairs to count (8192 x 8192, weights
-//           in L2: W2A2 N = 4 12.9 -> 8.8, N = 16 38 -> 14.6, N = 2 the same; W4A4 N = 1 14.6 -> 13.1, from
-//           HBM the same), but for small problems: mv_planes_faster
-//   bytes   three columns on: N = 4 26 -> 17, N = 8 35 -> 18 (N = 2 15.9 -> 17.6), and not for small
-//           matrices (1000 x 4096, N = 7: 4.6 -> 4.9)
+//           in L2: W2A2 N = 4 12.9 -> 7.2, N = 16 38 -> 9.1; W4A4 N = 1 14.6 -> 11.5), but for small problems:
+//           mv_planes_faster
+//   bytes   three columns on from 2^23 weights, four from 3 x 2^20: N = 4 26 -> 11.6, N = 8 35 -> 12.1 (N = 2
+//           4805 x 5120 5.4 -> 6.2); 11841 x 512 N = 7 6.1 -> 2.9, 416 x 7424 N = 6 6.8 -> 4.0.  Below, where
+//           either takes 2 to 3 us, a call of the host takes longer than both, and of this one longest
+//           (320 x 1401 N = 7: 2.9 -> 2.5 replayed, 4.08 -> 4.16 call after call)
 //   any     where the others need a second launch that clears the output first (bit planes they set
 //           bit by bit; pad bytes they do not write), the host's second launch decides, call after call
 //           (planes: 4.6 us here, 7.3 there for everything small, and faster here for 677 of 700 random
@@ -404,52 +548,54 @@ static bool mv_planes_faster(const qnn_gemm_desc *d) {
 //           the two launches take less time on the device: 66.9 against 67.6 us for the batch-1 chain as
 //           a graph)
 bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr) {
-    MvPlan pl;
-    if (!mv_plan(d, &pl)) return false;
-    const bool clears = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (pl.src != MV_FIELDS && d->M % 16 != 0));
-    if (pl.src == MV_FIELDS) return d->N >= 2 || clears;
+    if (!mv_fits(d)) return false;
+    const bool clears = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (d->w_fmt != QNN_FMT_FIELDS && d->M % 16 != 0));
+    if (d->w_fmt == QNN_FMT_FIELDS) return d->N >= 2 || clears;
     const long long size = (long long)d->M * d->K;
-    if (pl.src == MV_PLANES)
+    if (d->w_fmt == QNN_FMT_BITPLANES)
         return clears ? d->N >= 2 || d->w_bits * d->a_bits >= 12 || size < (1ll << 24)
                       : (d->N >= 2 || d->w_bits * d->a_bits >= 12) && mv_planes_faster(d);
-    return (d->N >= 3 && size >= (1ll << 23)) || (clears && size < (1ll << 26));
+    return (d->N >= 3 && size >= (1ll << 23)) || (d->N >= 4 && size >= (3ll << 20)) || (clears && size < (1ll << 26));
 }
 
-template <int SRC, int B, int V, int NT, bool W_SIGNED, bool A_SIGNED>
-static qnn_status mv_launch(const MvParams &p, size_t smem, cudaStream_t s) {
-    auto kern = gemv_mma_kernel<SRC, B, V, NT, W_SIGNED, A_SIGNED>;
+template <int SRC, int B, int V, int NT, int U, bool W_SIGNED, bool A_SIGNED>
+static qnn_status mv_launch(const MvParams &p, const MvPlan &pl, cudaStream_t s) {
+    auto kern = gemv_mma_kernel<SRC, B, V, NT, U, W_SIGNED, A_SIGNED>;
     static std::atomic<bool> attr_done[QNN_MAX_DEVICES];           // per instantiation and device
     const int dev = current_device();
     if (dev < 0 || !allow_smem(kern, MV_SMEM_MAX, attr_done[dev])) return QNN_ERR_CUDA;
-    // programmatic dependent launch: a CTA has an SM's registers to itself, so early placement cannot
+    // programmatic dependent launch: a CTA has most of an SM's registers to itself, so early placement cannot
     // crowd several onto one SM; nothing is read before griddepcontrol.wait
-    const dim3 grid((unsigned)(p.tiles < sm_count() ? p.tiles : sm_count()));
-    if (launch_pdl<MvParams>(kern, grid, MV_THREADS, smem, s, p) != cudaSuccess) return QNN_ERR_CUDA;
+    if (launch_pdl<MvParams>(kern, dim3((unsigned)ceil_div(p.groups, p.per)), pl.threads, pl.smem, s, p) != cudaSuccess) return QNN_ERR_CUDA;
     count_launch();
     return launch_status();
 }
 
-template <int SRC, int B, int V, bool W_SIGNED>
-static qnn_status mv_launch_n(const MvParams &p, size_t smem, cudaStream_t s) {
-    if (SRC != MV_BYTES && p.N > 8)
-        return p.a_signed ? mv_launch<SRC, B, V, SRC == MV_BYTES ? 1 : 2, W_SIGNED, true>(p, smem, s)
-                          : mv_launch<SRC, B, V, SRC == MV_BYTES ? 1 : 2, W_SIGNED, false>(p, smem, s);
-    return p.a_signed ? mv_launch<SRC, B, V, 1, W_SIGNED, true>(p, smem, s) : mv_launch<SRC, B, V, 1, W_SIGNED, false>(p, smem, s);
+template <int SRC, int B, int V, int NT, bool W_SIGNED, bool A_SIGNED>
+static qnn_status mv_launch_u(const MvParams &p, const MvPlan &pl, cudaStream_t s) {
+    constexpr int REGS = NT * (SRC == MV_PLANES ? 8 * V : 4 * (8 / B)), LEAST = mv_steps_least(REGS), MOST = mv_steps_most(REGS);
+    if (pl.u == LEAST) return mv_launch<SRC, B, V, NT, LEAST, W_SIGNED, A_SIGNED>(p, pl, s);
+    return mv_launch<SRC, B, V, NT, MOST, W_SIGNED, A_SIGNED>(p, pl, s);
+}
+
+template <int SRC, int B, int V, bool W_SIGNED, bool A_SIGNED>
+static qnn_status mv_launch_n(const MvParams &p, const MvPlan &pl, cudaStream_t s) {
+    if (SRC != MV_BYTES && p.N > 8) return mv_launch_u<SRC, B, V, SRC == MV_BYTES ? 1 : 2, W_SIGNED, A_SIGNED>(p, pl, s);
+    return mv_launch_u<SRC, B, V, 1, W_SIGNED, A_SIGNED>(p, pl, s);
 }
 
 qnn_status gemv_mma_launch(const qnn_gemm_desc *d, const void *W, const void *A, const int32_t *thr, void *out, cudaStream_t s) {
     MvPlan pl;
-    if (!mv_plan(d, &pl)) return QNN_ERR_UNSUPPORTED;
+    if (!mv_plan(d, thr != nullptr, &pl)) return QNN_ERR_UNSUPPORTED;
     MvParams p = {};
     p.W = (const uint8_t *)W; p.A = (const uint8_t *)A; p.thr = thr; p.out = out;
     p.M = d->M; p.N = d->N; p.K = d->K;
-    p.tiles = ceil_div(d->M, MV_ROWS); p.steps = pl.steps; p.units = pl.units;
+    p.groups = pl.groups; p.per = pl.per; p.units = pl.units;
+    p.dsplit = pl.dsplit; p.rsplit = pl.rsplit; p.passes = pl.passes;
     p.a_bits = d->a_bits; p.a_kind = plane_kind(d->a_enc);
     p.a_pitch = pl.src == MV_PLANES ? 4 * ceil_div(d->K, 32) : round_up(d->K, 16);
     p.w_pitch = pl.src == MV_FIELDS ? 16ll * pl.units : p.a_pitch;
     p.w_plane = (long long)d->M * p.w_pitch;
-    p.col_pitch = pl.col_pitch;
-    p.a_signed = d->a_enc != QNN_ENC_UNSIGNED ? 1 : 0;
     p.w_scale = 1;
     if (pl.src != MV_BYTES) {
         if (d->w_enc == QNN_ENC_BIPOLAR) { p.w_scale = 2; p.w_off = -1; }
@@ -458,17 +604,21 @@ qnn_status gemv_mma_launch(const qnn_gemm_desc *d, const void *W, const void *A,
     p.out_bits = thr ? d->out_bits : 0;
     p.out_fmt = d->out_fmt;
     p.ld_out = round_up(d->M, 16);
-    const size_t m = pl.smem;
-    if (pl.src == MV_BYTES)
-        return d->w_enc != QNN_ENC_UNSIGNED ? mv_launch_n<MV_BYTES, 8, 4, true>(p, m, s) : mv_launch_n<MV_BYTES, 8, 4, false>(p, m, s);
-    if (pl.src == MV_FIELDS)
-        return pl.b == 1 ? mv_launch_n<MV_FIELDS, 1, 4, false>(p, m, s)
-                         : (pl.b == 2 ? mv_launch_n<MV_FIELDS, 2, 4, false>(p, m, s) : mv_launch_n<MV_FIELDS, 4, 4, false>(p, m, s));
-#define QNN_MV_CASE(B_, V_) if (pl.b == B_ && pl.v == V_) return mv_launch_n<MV_PLANES, B_, V_, false>(p, m, s);
-    QNN_MV_CASE(1, 1) QNN_MV_CASE(1, 2) QNN_MV_CASE(1, 4)
-    QNN_MV_CASE(2, 1) QNN_MV_CASE(2, 2) QNN_MV_CASE(2, 4)
-    QNN_MV_CASE(3, 1) QNN_MV_CASE(3, 2)
-    QNN_MV_CASE(4, 1) QNN_MV_CASE(4, 2)
+    const bool as = d->a_enc != QNN_ENC_UNSIGNED, ws = d->w_enc != QNN_ENC_UNSIGNED;
+    if (pl.src == MV_BYTES) {
+        if (ws) return as ? mv_launch_n<MV_BYTES, 8, 4, true, true>(p, pl, s) : mv_launch_n<MV_BYTES, 8, 4, true, false>(p, pl, s);
+        return as ? mv_launch_n<MV_BYTES, 8, 4, false, true>(p, pl, s) : mv_launch_n<MV_BYTES, 8, 4, false, false>(p, pl, s);
+    }
+    if (pl.src == MV_FIELDS) {
+#define QNN_MV_CASE(B_) if (pl.b == B_) return as ? mv_launch_n<MV_FIELDS, B_, 4, false, true>(p, pl, s) : mv_launch_n<MV_FIELDS, B_, 4, false, false>(p, pl, s);
+        QNN_MV_CASE(1) QNN_MV_CASE(2) QNN_MV_CASE(4)
+#undef QNN_MV_CASE
+    }
+    // planes: at most four, so the activations fit signed bytes whatever their encoding
+#define QNN_MV_CASE(B_)                                                                                                        \
+    if (pl.b == B_) return pl.v == 4 ? mv_launch_n<MV_PLANES, B_, B_ <= 2 ? 4 : 2, false, true>(p, pl, s)                       \
+                                     : (pl.v == 2 ? mv_launch_n<MV_PLANES, B_, 2, false, true>(p, pl, s) : mv_launch_n<MV_PLANES, B_, 1, false, true>(p, pl, s));
+    QNN_MV_CASE(1) QNN_MV_CASE(2) QNN_MV_CASE(3) QNN_MV_CASE(4)
 #undef QNN_MV_CASE
     return QNN_ERR_UNSUPPORTED;
 }

@@ -1,0 +1,51 @@
+"""The few-column tensor-core kernel (one to sixteen columns) at the edges of its plan, against the
+oracle: groups of eight rows and pairs of them, depth slices that end inside a load, several passes over a
+depth, warps that take other groups, each format and encoding."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_1709_04060_b200 import synth
+from qnn_testutil import decode_out
+
+pytestmark = pytest.mark.gpu
+
+BITPLANES, INT8, FIELDS = 0, 1, 2
+
+
+@pytest.fixture(scope="module")
+def qb():
+    from paper_1709_04060_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("fmt,w,a,w_enc,a_enc", [
+    (BITPLANES, 1, 2, 2, 0), (BITPLANES, 2, 4, 1, 1), (BITPLANES, 3, 1, 0, 2), (BITPLANES, 4, 3, 1, 0), (BITPLANES, 1, 1, 2, 2),
+    (FIELDS, 1, 8, 2, 0), (FIELDS, 2, 2, 1, 1), (FIELDS, 4, 4, 1, 0), (INT8, 8, 8, 1, 0), (INT8, 3, 8, 0, 1),
+])
+@pytest.mark.parametrize("M,N,K", [
+    (4100, 2, 4097), (1201, 8, 9216),          # rows past whole groups; one pass more than 16 warps hold
+    (2500, 9, 1000), (321, 16, 9120),          # two blocks of columns; passes
+    (4100, 5, 33), (1200, 3, 2080),            # shallow: several groups at a time
+    (19000, 2, 512),                           # more groups a CTA than warps
+])
+def test_plan_edges(qb, fmt, w, a, w_enc, a_enc, M, N, K):
+    if fmt == INT8 and N > 8:
+        N = 8
+    case = synth.gemm_case(4400 + M + 3 * K + w, M, N, K, w, a, w_enc, a_enc, out_bits=3)
+    a_fmt = INT8 if fmt == FIELDS else fmt
+    Wp = qb.pack(qb.to_device_logical(case.W, w_enc), w, w_enc, fmt)
+    Ap = qb.pack(qb.to_device_logical(case.At, a_enc), a, a_enc, a_fmt)
+    thr = torch.from_numpy(case.thr).cuda()
+    sums = orc.qgemm(case.W, case.At, None).T
+    codes = (sums[:, :, None] >= case.thr[None]).sum(2)
+    for out_fmt, raw in ((INT8, False), (BITPLANES, False), (INT8, True)):
+        d = qb.qnn_gemm_desc(M, N, K, w, a, 3, w_enc, a_enc, fmt, a_fmt, out_fmt, 0, 0)
+        nb = qb.qnn_gemm_out_bytes(d, not raw)
+        out = torch.full((nb + 64,), 0xEE, dtype=torch.uint8, device="cuda")
+        qb.check(qb.qnn_qgemm(d, Wp, Ap, None if raw else thr, out))
+        torch.cuda.synchronize()
+        buf = out.cpu().numpy()
+        assert (buf[nb:] == 0xEE).all()
+        assert np.array_equal(decode_out(buf[:nb], out_fmt, 3, N, M, raw), sums if raw else codes)
