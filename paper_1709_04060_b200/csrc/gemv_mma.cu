@@ -510,7 +510,7 @@ static bool mv_fits(const qnn_gemm_desc *d) {
     return (long long)d->N * round_up(d->K, 32) <= 192 * 1024;
 }
 
-// Bit planes that need no clearing launch: whether this kernel beats the one that counts bits
+// Sums, and 8-bit codes without pad bytes: whether this kernel beats the one that counts bits
 // (gemv_planes.cu), by an estimate of both.  That one costs a load latency per staged column and plane, one
 // per depth step of a lane, its CTAs and its population counts; this one its fill and drain, the columns it
 // widens, the rounds of tiles and the weights.  The terms' shares are fitted to random problems; the factor
@@ -539,23 +539,22 @@ static bool mv_planes_faster(const qnn_gemm_desc *d) {
 //           4805 x 5120 5.4 -> 6.2); 11841 x 512 N = 7 6.1 -> 2.9, 416 x 7424 N = 6 6.8 -> 4.0.  Below, where
 //           either takes 2 to 3 us, a call of the host takes longer than both, and of this one longest
 //           (320 x 1401 N = 7: 2.9 -> 2.5 replayed, 4.08 -> 4.16 call after call)
-//   any     where the others need a second launch that clears the output first (bit planes they set
-//           bit by bit; pad bytes they do not write), the host's second launch decides, call after call
-//           (planes: 4.6 us here, 7.3 there for everything small, and faster here for 677 of 700 random
-//           problems up to 12000 x 9216, although one in five takes longer on the device, up to 3 us;
-//           fields N = 1 10.2 -> 8.1, bytes 4096 x 9216 N = 1 12.8 -> 11.4); bytes only below 2^26
-//           elements (8192 x 8192: 16.1 there, 17 here), planes with one column below 2^24 (from there on
-//           the two launches take less time on the device: 66.9 against 67.6 us for the batch-1 chain as
-//           a graph)
+//   codes   fields and bytes whose kernels need a second launch that clears the output first (bit planes that
+//           they set bit by bit; pad bytes that they do not write): the host's second launch decides, call
+//           after call (fields N = 1 10.2 -> 8.1, bytes 4096 x 9216 N = 1 12.8 -> 11.4); bytes only below 2^26
+//           elements (8192 x 8192: 16.1 there, 17 here)
+//   planes whose output is bit planes or padded: two columns on (240 random problems with two columns: 0.76 of
+//           the time on average, more columns 0.51); one column below 2^24 weights (210 problems: 0.95,
+//           between 0.4 and 1.6)
 bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr) {
     if (!mv_fits(d)) return false;
-    const bool clears = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (d->w_fmt != QNN_FMT_FIELDS && d->M % 16 != 0));
-    if (d->w_fmt == QNN_FMT_FIELDS) return d->N >= 2 || clears;
+    const bool padded = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (d->w_fmt != QNN_FMT_FIELDS && d->M % 16 != 0));
+    if (d->w_fmt == QNN_FMT_FIELDS) return d->N >= 2 || padded;
     const long long size = (long long)d->M * d->K;
     if (d->w_fmt == QNN_FMT_BITPLANES)
-        return clears ? d->N >= 2 || d->w_bits * d->a_bits >= 12 || size < (1ll << 24)
+        return padded ? d->N >= 2 || d->w_bits * d->a_bits >= 12 || size < (1ll << 24)
                       : (d->N >= 2 || d->w_bits * d->a_bits >= 12) && mv_planes_faster(d);
-    return (d->N >= 3 && size >= (1ll << 23)) || (d->N >= 4 && size >= (3ll << 20)) || (clears && size < (1ll << 26));
+    return (d->N >= 3 && size >= (1ll << 23)) || (d->N >= 4 && size >= (3ll << 20)) || (padded && size < (1ll << 26));
 }
 
 template <int SRC, int B, int V, int NT, int U, bool W_SIGNED, bool A_SIGNED>

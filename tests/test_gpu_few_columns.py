@@ -49,3 +49,30 @@ def test_plan_edges(qb, fmt, w, a, w_enc, a_enc, M, N, K):
         buf = out.cpu().numpy()
         assert (buf[nb:] == 0xEE).all()
         assert np.array_equal(decode_out(buf[:nb], out_fmt, 3, N, M, raw), sums if raw else codes)
+
+
+@pytest.mark.parametrize("w,a,w_enc,a_enc", [(1, 2, 2, 0), (2, 2, 1, 0), (3, 1, 0, 2)])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 31), (17, 5, 128), (4097, 1, 4096), (9700, 3, 96), (10001, 16, 70)])
+def test_counting_kernel_writes_whole_rows(qb, w, a, w_enc, a_enc, M, N, K):
+    """The AND/POPC kernel writes pad bytes and pad bits itself: rows past whole groups of eight, several
+    turns of a CTA."""
+    case = synth.gemm_case(4700 + M + w, M, N, K, w, a, w_enc, a_enc, out_bits=3)
+    Wp = qb.pack(qb.to_device_logical(case.W, w_enc), w, w_enc, BITPLANES)
+    Ap = qb.pack(qb.to_device_logical(case.At, a_enc), a, a_enc, BITPLANES)
+    thr = torch.from_numpy(case.thr).cuda()
+    sums = orc.qgemm(case.W, case.At, None).T
+    codes = (sums[:, :, None] >= case.thr[None]).sum(2)
+    for out_fmt in (INT8, BITPLANES):
+        d = qb.qnn_gemm_desc(M, N, K, w, a, 3, w_enc, a_enc, BITPLANES, BITPLANES, out_fmt, qb.QNN_PATH_BITSERIAL, 0)
+        assert qb.qnn_qgemm_kernel_name(d, True) == "gemv_planes_kernel"
+        nb = qb.qnn_gemm_out_bytes(d, True)
+        out = torch.full((nb + 64,), 0xEE, dtype=torch.uint8, device="cuda")
+        qb.check(qb.qnn_qgemm(d, Wp, Ap, thr, out))
+        torch.cuda.synchronize()
+        buf = out.cpu().numpy()
+        assert (buf[nb:] == 0xEE).all()
+        assert np.array_equal(decode_out(buf[:nb], out_fmt, 3, N, M, False), codes)
+        if out_fmt == INT8:
+            assert (buf[:nb].reshape(N, -1)[:, M:] == 0).all()
+        elif M % 32:
+            assert (buf[:nb].view(np.uint32).reshape(3 * N, -1)[:, -1] >> (M % 32) == 0).all()
