@@ -274,9 +274,10 @@ qnn_status qnn_im2col(const qnn_conv_desc *d, const void *in, void *lowered, voi
  * (word-granular, as in Section 3.2).
  * 8-bit maps are lowered inside the tensor-core kernel: by its tensor-map loader
  * when C and in_pitch are multiples of 16 (the CTA-pair kernel for large layers,
- * the one-CTA kernel otherwise); by lowering warps when pixels are contiguous and
- * either C is not a multiple of 16, pad == 0, OC <= 128 and the weights are not
- * BIPOLAR, or C is a multiple of 16 but not of 128, the layer has many tiles and
+ * the one-CTA kernel otherwise); by the operand descriptors of a kernel that keeps image rows
+ * in shared memory when C is 3, pixels are contiguous, pad == 0, OC <= 128, the stride is 1, 2
+ * or 4 and the layer has many tiles; by lowering warps when pixels are contiguous and either C
+ * is not a multiple of 16, pad == 0, OC <= 128 and the weights are not BIPOLAR, or C is a multiple of 16 but not of 128, the layer has many tiles and
  * the CTA-pair kernel does not apply.  All routes give the same integer results.
  * The pad columns of the weight rows (see qnn_conv_lowered_k) must be zero bytes
  * for the lowering warps' unmasked route: it leaves image bytes,
@@ -284,6 +285,17 @@ qnn_status qnn_im2col(const qnn_conv_desc *d, const void *in, void *lowered, voi
 qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in,
                      const int32_t *thr, void *out,
                      void *workspace, size_t workspace_bytes, void *stream);
+
+/* Convolution and the max-pool behind it (Section 4.2) in one kernel: the un-pooled map never reaches
+ * global memory.  Arguments as for qnn_qconv, without a workspace, thr required; `out` is the pooled map,
+ * [B][(OH-k)/stride+1][(OW-k)/stride+1][...] in d->out_fmt, i.e. what qnn_maxpool makes of qnn_qconv's output.
+ * Which layers fuse: qnn_conv_maxpool_fuses (host only; 1 or 0), i.e. large three-channel 8-bit maps
+ * with contiguous pixels and no padding, a filter stride of 1, 2 or 4 and rows of 33 to 64 units (output
+ * pixels plus ceil(KW / stride) - 1), with a 3 x 3 pool of stride 2.  The others return
+ * QNN_ERR_UNSUPPORTED: call qnn_qconv and qnn_maxpool. */
+int qnn_conv_maxpool_fuses(const qnn_conv_desc *d, int k, int stride);
+qnn_status qnn_qconv_maxpool(const qnn_conv_desc *d, int k, int stride, const void *Wpacked, const void *in,
+                             const int32_t *thr, void *out, void *stream);
 
 /* Largest lowered matrix, in bytes, that qnn_qconv_static accepts. */
 #define QNN_QCONV_STATIC_MAX_BYTES (16u << 20)

@@ -3,7 +3,8 @@
 Section 4.2 / Table 3 of the paper: conv1 and fc8 are 8-bit layers, the other
 matrix layers are W1A2 with per-channel threshold activations, 3x3 stride-2
 max-pools follow conv1, conv2 and conv5.  This module only sequences the calls
-(qnn_qconv, qnn_maxpool, qnn_qgemm) and owns the device buffers; all
+(qnn_qconv, qnn_maxpool, qnn_qgemm, and qnn_qconv_maxpool where the library has
+both layers in one kernel) and owns the device buffers; all
 arithmetic runs in the library's kernels.
 
 ``mode`` selects the operand format of the W1A2 layers' activations/weights:
@@ -94,13 +95,25 @@ class AlexNetPlan:
                 flat = L.OC
             fmt_in = out_fmt
         self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
+        # convolutions that run together with the pool behind them
+        self._fused = {i for i in range(len(self.steps) - 1)
+                       if self.steps[i][0] == "conv" and self.steps[i + 1][0] == "pool" and self.steps[i][3] is not None
+                       and qb.qnn_conv_maxpool_fuses(self.steps[i][1], self.steps[i + 1][1].k, self.steps[i + 1][1].stride)}
+        self._image = None       # input of the last forward pass
         self.n_classes = self.layers[-1].OC
 
     def forward(self, image: torch.Tensor, stream=None):
         """image: uint8 device tensor [B][H][W][3].  Returns int32 logits [B][n_classes]
         (a view of the plan's last buffer).  Enqueues only; does not synchronise."""
-        x = image
-        for kind, d, Wp, thr, out in self.steps:
+        x = self._image = image
+        for i, (kind, d, Wp, thr, out) in enumerate(self.steps):
+            if i in self._fused:
+                _, pool, _, _, pooled = self.steps[i + 1]
+                qb.check(qb.qnn_qconv_maxpool(d, pool.k, pool.stride, Wp, x, thr, pooled, stream))
+                x = pooled
+                continue
+            if i - 1 in self._fused:
+                continue
             if kind == "conv":
                 qb.check(qb.qnn_qconv(d, Wp, x, thr, out, self.workspace, self.workspace.numel(), stream))
             elif kind == "pool":
@@ -128,7 +141,14 @@ class AlexNetPlan:
         return graph, logits
 
     def intermediates(self):
-        """{step name: (output buffer, descriptor kind, descriptor)} for tests."""
+        """{step name: (output buffer, descriptor kind, descriptor)} for tests.  A convolution that runs
+        together with its pool leaves no map of its own: it is computed here from its present input (for
+        the first layer the image of the last forward pass)."""
+        for i in sorted(self._fused):
+            if i > 0 or self._image is not None:
+                _, d, Wp, thr, out = self.steps[i]
+                x = self.steps[i - 1][4] if i > 0 else self._image
+                qb.check(qb.qnn_qconv(d, Wp, x, thr, out, self.workspace, self.workspace.numel()))
         return {n: (s[4], s[0], s[1]) for n, s in zip(self.names, self.steps)}
 
     def launches_per_forward(self) -> int:

@@ -36,7 +36,7 @@ EXPORTS = (
     "qnn_packed_ld", "qnn_packed_bytes", "qnn_pack", "qnn_planes_to_int8", "qnn_gemm_workspace_bytes",
     "qnn_gemm_out_bytes", "qnn_qgemm", "qnn_qgemm_kernel", "qnn_qgemm_kernel_name", "qnn_conv_out_h", "qnn_conv_out_w",
     "qnn_conv_lowered_k", "qnn_conv_lowered_bytes", "qnn_conv_workspace_bytes",
-    "qnn_conv_out_bytes", "qnn_im2col", "qnn_qconv", "qnn_qconv_static", "qnn_maxpool",
+    "qnn_conv_out_bytes", "qnn_im2col", "qnn_qconv", "qnn_conv_maxpool_fuses", "qnn_qconv_maxpool", "qnn_qconv_static", "qnn_maxpool",
     "qnn_streamline", "qnn_peak_mma_i8", "qnn_peak_popc", "qnn_peak_popc_sink_bytes", "qnn_validate_thresholds", "qnn_device_status", "qnn_launch_count",
     "qnn_status_string", "qnn_version",
 )
@@ -99,6 +99,10 @@ _lib.qnn_im2col.restype = _ci
 _lib.qnn_im2col.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp]
 _lib.qnn_qconv.restype = _ci
 _lib.qnn_qconv.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp]
+_lib.qnn_conv_maxpool_fuses.restype = _ci
+_lib.qnn_conv_maxpool_fuses.argtypes = [_P(qnn_conv_desc), _ci, _ci]
+_lib.qnn_qconv_maxpool.restype = _ci
+_lib.qnn_qconv_maxpool.argtypes = [_P(qnn_conv_desc), _ci, _ci, _vp, _vp, _vp, _vp, _vp]
 _lib.qnn_qconv_static.restype = _ci
 _lib.qnn_qconv_static.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp, _vp, _vp]
 _lib.qnn_maxpool.restype = _ci
@@ -190,6 +194,7 @@ _planes_to_int8 = _entry("qnn_planes_to_int8", "dpps", qnn_pack_desc)
 _qgemm = _entry("qnn_qgemm", "dpppppns", qnn_gemm_desc)
 _im2col = _entry("qnn_im2col", "dpps", qnn_conv_desc)
 _qconv = _entry("qnn_qconv", "dpppppns", qnn_conv_desc)
+_qconv_maxpool = _entry("qnn_qconv_maxpool", "dnnpppps", qnn_conv_desc)
 _qconv_static = _entry("qnn_qconv_static", "dpppps", qnn_conv_desc)
 _maxpool = _entry("qnn_maxpool", "dpps", qnn_pool_desc)
 
@@ -280,6 +285,15 @@ def qnn_im2col(d, inp, lowered, stream=None) -> int:
 
 def qnn_qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream=None) -> int:
     return _qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream)
+
+
+def qnn_conv_maxpool_fuses(d, k: int, stride: int) -> bool:
+    """Whether qnn_qconv_maxpool takes this layer with this pool."""
+    return bool(_lib.qnn_conv_maxpool_fuses(ctypes.byref(d), k, stride))
+
+
+def qnn_qconv_maxpool(d, k: int, stride: int, Wpacked, inp, thr, out, stream=None) -> int:
+    return _qconv_maxpool(d, k, stride, Wpacked, inp, thr, out, stream)
 
 
 QNN_QCONV_STATIC_MAX_BYTES = 16 << 20

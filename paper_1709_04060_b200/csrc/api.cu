@@ -393,8 +393,11 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
     // lowered matrix (measurements, tests)
     const char *explicit_env = getenv("QNN_CONV_EXPLICIT");
     if (path == QNN_PATH_TCGEN05_I8 && !(explicit_env && explicit_env[0] == '1')) {
+        // three-channel maps whose rows shared memory holds: nothing is lowered
+        st = conv_direct_launch(d, &g, Wpacked, in, thr, out, false, (cudaStream_t)stream);
+        if (st != QNN_ERR_UNSUPPORTED) return st;
         // lowering warps inside the kernel where the tensor-map loader does not apply (few
-        // channels: the first layer) or would waste k-blocks (channel count not a multiple of 128)
+        // channels: other first layers) or would waste k-blocks (channel count not a multiple of 128)
         st = gemm_tc_lower_launch(d, &g, Wpacked, in, thr, out, (cudaStream_t)stream);
         if (st != QNN_ERR_UNSUPPORTED) return st;
         st = gemm_tc_conv_launch(d, &g, Wpacked, in, thr, out, false, (cudaStream_t)stream);
@@ -417,6 +420,29 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
     st = im2col_launch(d, in, workspace, (cudaStream_t)stream);
     if (st != QNN_OK) return st;
     return qnn_qgemm(&g, Wpacked, workspace, thr, out, nullptr, 0, stream);
+}
+
+int qnn_conv_maxpool_fuses(const qnn_conv_desc *d, int k, int stride) {
+    qnn_gemm_desc g;
+    int path = 0;
+    if (check_conv_desc(d) != QNN_OK || k != 3 || stride != 2) return 0;
+    conv_to_gemm(d, &g);
+    if (check_gemm_desc(&g, true, &path) != QNN_OK || path != QNN_PATH_TCGEN05_I8) return 0;
+    return conv_direct_takes(d, &g, true, true) ? 1 : 0;
+}
+
+qnn_status qnn_qconv_maxpool(const qnn_conv_desc *d, int k, int stride, const void *Wpacked, const void *in,
+                             const int32_t *thr, void *out, void *stream) {
+    qnn_status st = check_conv_desc(d);
+    if (st != QNN_OK) return st;
+    qnn_gemm_desc g;
+    conv_to_gemm(d, &g);
+    st = check_gemm_desc(&g, true, nullptr);
+    if (st != QNN_OK) return st;
+    if (!Wpacked || !in || !thr || !out || k <= 0 || stride <= 0) return QNN_ERR_INVALID_ARG;
+    if (!aligned16(Wpacked) || !aligned16(in) || !aligned16(out) || !aligned4(thr)) return QNN_ERR_ALIGNMENT;
+    if (!qnn_conv_maxpool_fuses(d, k, stride)) return QNN_ERR_UNSUPPORTED;
+    return conv_direct_launch(d, &g, Wpacked, in, thr, out, true, (cudaStream_t)stream);
 }
 
 // Lowered-matrix storage of qnn_qconv_static.  In host code this name is only a

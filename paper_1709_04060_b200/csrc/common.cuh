@@ -124,6 +124,9 @@ qnn_status gemm_tc_lower_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g,
                                 const int32_t *thr, void *out, cudaStream_t s);
 qnn_status gemm_tc_planes_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *A,
                                  const int32_t *thr, void *out, cudaStream_t s);
+bool conv_direct_takes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, bool pool);
+qnn_status conv_direct_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
+                              const int32_t *thr, void *out, bool pool, cudaStream_t s);
 qnn_status im2col_launch(const qnn_conv_desc *d, const void *in, void *lowered, cudaStream_t s);
 qnn_status maxpool_launch(const qnn_pool_desc *d, const void *in, void *out, cudaStream_t s);
 qnn_status validate_thresholds_launch(const int32_t *thr, int M, int n_thr, int *n_bad, cudaStream_t s);
