@@ -98,6 +98,10 @@ struct TcParams {
     // channels-last feature map itself: k-block kb = (filter tap, 128-byte channel chunk), and
     // the 128 pixels x 128 bytes of a stage are fetched by one im2col-mode TMA load.
     int taps, cchunks, cv_C, cv_KW, cv_OW, cv_OHW, cv_stride, cv_pad;
+    // ... or (CTA-pair kernel, bx_w != 0, stride 1) by one tiled load of a box of bx_w x bx_h output pixels of bx_n images,
+    // shifted by the tap: the tile's rows are then the box's pixels, columns fastest, nb_w x nb_h x nb_n
+    // boxes in all
+    int bx_w, bx_h, bx_n, nb_w, nb_h, nb_n;
     // Convolution lowered inside the kernel (LOWER kernels; 8-bit maps with contiguous pixels): the
     // map itself is the input, four lowering warps build the activation tiles in shared memory
     // from image rows staged there by bulk copies.  A lowered row is one run per filter row: the
@@ -142,6 +146,45 @@ __host__ __device__ inline void lw_range(const TcParams &p, int p0, int p1, long
     if (r1 > p.lw_H) r1 = p.lw_H;
     *lo = (((long long)b0 * p.lw_H + r0) * p.lw_rowbytes) & ~15ll;
     *hi = ((long long)b1 * p.lw_H + r1) * p.lw_rowbytes;
+}
+
+// Box b of an implicit convolution: its first output pixel (boxes past the last one: the last one's).
+__device__ __forceinline__ void tc_box(const TcParams &p, int b, int *ow, int *oh, int *img) {
+    // images first, so that the two boxes of a CTA pair are often the same pixels of other images
+    b = min(b, p.nb_w * p.nb_h * p.nb_n - 1);
+    const int q = b / p.nb_n;
+    *img = (b - q * p.nb_n) * p.bx_n;
+    *ow = q % p.nb_w * p.bx_w;
+    *oh = q / p.nb_w * p.bx_h;
+}
+// Output pixel of row r of the tile that starts at row p0 (N: none).
+__device__ __forceinline__ int tc_pixel(const TcParams &p, int p0, int r) {
+    if (p.bx_w == 0) return p0 + r;
+    const int b = p0 / TC_BP;
+    if (b >= p.nb_w * p.nb_h * p.nb_n || r >= p.bx_w * p.bx_h * p.bx_n) return p.N;
+    int ow, oh, img;
+    tc_box(p, b, &ow, &oh, &img);
+    const int q = r / p.bx_w;
+    ow += r - q * p.bx_w; oh += q % p.bx_h; img += q / p.bx_h;
+    if (ow >= p.cv_OW || oh * p.cv_OW >= p.cv_OHW || (long long)img * p.cv_OHW >= p.N) return p.N;
+    return img * p.cv_OHW + oh * p.cv_OW + ow;
+}
+// The filter taps of a CTA pair's tile (its first row: p0) that meet the image at all; at the border of a
+// padded map the others would only add zeros (27 x 27, 5 x 5 taps: 9 % of them; 13 x 13, 3 x 3: 10 %).
+struct TcTaps { int h0, h1, w0, w1; };
+__device__ __forceinline__ TcTaps tc_taps(const TcParams &p, int p0) {
+    const int KW = p.cv_KW, KH = p.taps / KW;
+    TcTaps t = {0, KH, 0, KW};
+    if (p.bx_w == 0) return t;
+    int h0 = KH, h1 = 0, w0 = KW, w1 = 0;
+    for (int i = 0; i < 2; ++i) {
+        int ow, oh, img;
+        tc_box(p, p0 / TC_BP + i, &ow, &oh, &img);
+        h0 = min(h0, max(0, p.cv_pad - oh - (p.bx_h - 1))); h1 = max(h1, min(KH, p.lw_H + p.cv_pad - oh));
+        w0 = min(w0, max(0, p.cv_pad - ow - (p.bx_w - 1))); w1 = max(w1, min(KW, p.lw_W + p.cv_pad - ow));
+    }
+    if (h0 < h1 && w0 < w1) t = {h0, h1, w0, w1};
+    return t;
 }
 
 // What an epilogue warp needs for the exchange of a shared tile.  The weight ring holds,
@@ -288,7 +331,8 @@ __device__ __forceinline__ void stager_loop(const TcParams &p, int *thr_s, uint6
 // Per-unit epilogue shared by both kernels: waits for the unit's thresholds and for its
 // accumulators, processes this warp's part, then releases the threshold buffer (the
 // caller releases the accumulators).  Returns false if a wait ran out.
-template <int OUT_MODE, int OUT_BITS>
+// BOX: tiles may be boxes of an implicit convolution's pixels.
+template <int OUT_MODE, int OUT_BITS, bool BOX = false>
 __device__ __forceinline__ bool epilogue_tile(const TcParams &p, const int *thr_s, uint64_t *thr_full,
                                               uint64_t *thr_empty, uint32_t thr_parity,
                                               uint64_t *tmem_full, uint32_t full_parity,
@@ -333,7 +377,7 @@ __device__ __forceinline__ bool epilogue_tile(const TcParams &p, const int *thr_
         }
     }
     epilogue_cols<OUT_MODE, OUT_BITS>(p, thr_s, t_acc + ((uint32_t)(quad * 32) << 16), c_begin, c_end,
-                                      p0 + quad * 32 + lane, c0, xw, lane);
+                                      BOX ? tc_pixel(p, p0, quad * 32 + lane) : p0 + quad * 32 + lane, c0, xw, lane);
     tc_fence_before();
     __syncwarp();
     if (OUT_MODE != OUT_RAW && lane == 0) mbar_arrive(thr_empty);
@@ -1150,24 +1194,34 @@ qgemm_tc2_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_const
                 // narrower last tile uses the first half-width of them)
                 const int c0 = ct + (int)rank * (CONV ? pair_tile_width(p, ct) >> 1 : 128);
                 int cv_w = 0, cv_h = 0, cv_n = 0;          // CONV: base pixel of this CTA's first output pixel
-                if (CONV) {
+                if (CONV && p.bx_w) {
+                    tc_box(p, p0 / TC_BP, &cv_w, &cv_h, &cv_n);
+                    cv_w -= p.cv_pad; cv_h -= p.cv_pad;
+                } else if (CONV) {
                     cv_n = p0 / p.cv_OHW;
                     const int r = p0 - cv_n * p.cv_OHW, oh = r / p.cv_OW;
                     cv_h = oh * p.cv_stride - p.cv_pad;
                     cv_w = (r - oh * p.cv_OW) * p.cv_stride - p.cv_pad;
                 }
-                int tap = 0, cc = 0, kh = 0, kw = 0;       // CONV: k-block = (filter tap, channel chunk)
-                for (int kb = un.kb_lo; kb < un.kb_hi; ++kb, ++it) {
+                TcTaps tp = {0, 0, 0, 0};
+                if (CONV) tp = tc_taps(p, p0 - (int)rank * 128);
+                int cc = 0, kh = tp.h0, kw = tp.w0;        // CONV: k-block = (filter tap, channel chunk)
+                const int kb_hi = CONV ? (tp.h1 - tp.h0) * (tp.w1 - tp.w0) * p.cchunks : un.kb_hi;
+                for (int kb = un.kb_lo; kb < kb_hi; ++kb, ++it) {
                     const int s = it % T2_STAGES;
                     const uint32_t ph = (it / T2_STAGES) & 1;
                     if (!(ok = mbar_wait(&sm.empty[s], ph ^ 1, abort_flag))) break;
-                    if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], PAIR_STAGE_BYTES);
+                    if (rank == 0)
+                        mbar_arrive_expect_tx(&sm.full[s], CONV && p.bx_w ? 2u * (uint32_t)(p.bx_w * p.bx_h * p.bx_n + 128) * TC_BK : PAIR_STAGE_BYTES);
                     const uint32_t leader_full = map_to_cta(smem_u32(&sm.full[s]), 0);
                     if (CONV) {
-                        tma_load_im2col_pair(sm.act[s], &map_act, leader_full, cc * TC_BK, cv_w, cv_h, cv_n,
-                                             (uint16_t)kw, (uint16_t)kh);
-                        tma_load_2d_pair(sm.wgt[s], &map_wgt, leader_full, tap * p.cv_C + cc * TC_BK, c0);
-                        if (++cc == p.cchunks) { cc = 0; ++tap; if (++kw == p.cv_KW) { kw = 0; ++kh; } }
+                        if (p.bx_w)
+                            tma_load_4d_pair(sm.act[s], &map_act, leader_full, cc * TC_BK, cv_w + kw, cv_h + kh, cv_n);
+                        else
+                            tma_load_im2col_pair(sm.act[s], &map_act, leader_full, cc * TC_BK, cv_w, cv_h, cv_n,
+                                                 (uint16_t)kw, (uint16_t)kh);
+                        tma_load_2d_pair(sm.wgt[s], &map_wgt, leader_full, (kh * p.cv_KW + kw) * p.cv_C + cc * TC_BK, c0);
+                        if (++cc == p.cchunks) { cc = 0; if (++kw == tp.w1) { kw = tp.w0; ++kh; } }
                     } else {
                         tma_load_2d_pair(sm.act[s], &map_act, leader_full, kb * TC_BK, p0);
                         tma_load_2d_pair(sm.wgt[s], &map_wgt, leader_full, kb * TC_BK, c0);
@@ -1194,7 +1248,11 @@ qgemm_tc2_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_const
             for (int u = pair; ok && u < num_units; u += num_pairs, ++tcount) {
                 const PairUnit un = pair_unit<KIND>(p, u, num_tiles);
                 const int tile = un.tile;
-                const int unit_kb = un.kb_hi - un.kb_lo;   // all k-blocks, or (a split tile) one half of them
+                int unit_kb = un.kb_hi - un.kb_lo;         // all k-blocks, or (a split tile) one half of them
+                if (CONV) {
+                    const TcTaps tp = tc_taps(p, (tile % p.tiles_p) * 256);
+                    unit_kb = (tp.h1 - tp.h0) * (tp.w1 - tp.w0) * p.cchunks;
+                }
                 const uint32_t buf = tcount & 1, acc_ph = (tcount >> 1) & 1;
                 if (!(ok = mbar_wait(&sm.tmem_empty[buf], acc_ph ^ 1, abort_flag))) break;
                 tc_fence_after();
@@ -1254,7 +1312,7 @@ qgemm_tc2_kernel(const __grid_constant__ CUtensorMap map_act, const __grid_const
                                                              &sm.tmem_full[buf], acc_ph, tmem_base + buf * T2_BN, p0, c0, un,
                                                              rank, warp, lane, abort_flag))
                     break;
-            } else if (!epilogue_tile<OUT_MODE, OUT_BITS>(p, sm.thr[buf], &sm.thr_full[buf], &sm.thr_empty[buf], acc_ph,
+            } else if (!epilogue_tile<OUT_MODE, OUT_BITS, CONV>(p, sm.thr[buf], &sm.thr_full[buf], &sm.thr_empty[buf], acc_ph,
                                                           &sm.tmem_full[buf], acc_ph, tmem_base + buf * T2_BN,
                                                           CONV ? pair_tile_width(p, c0) : T2_BN, p0, c0, -1, TcExchange{}, warp,
                                                           lane, abort_flag))
@@ -1338,6 +1396,56 @@ static bool make_im2col_map(CUtensorMap *map, const void *base, const qnn_conv_d
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(base), dims, strides, lower, upper,
               (cuuint32_t)TC_BK, (cuuint32_t)TC_BP, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The same map as boxes of w x h pixels of n images x 128 channel bytes.
+static bool make_box_map(CUtensorMap *map, const void *base, const qnn_conv_desc *d, int pitch, int w, int h, int n) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {(cuuint64_t)d->C, (cuuint64_t)d->W, (cuuint64_t)d->H, (cuuint64_t)d->B};
+    cuuint64_t strides[3] = {(cuuint64_t)pitch, (cuuint64_t)pitch * d->W, (cuuint64_t)pitch * d->W * d->H};
+    cuuint32_t box[4] = {(cuuint32_t)TC_BK, (cuuint32_t)w, (cuuint32_t)h, (cuuint32_t)n};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Boxes of output pixels for the CTA-pair kernel (0: im2col loads).  A box knows which filter taps fall outside
+// the image for all of its pixels, and the pair leaves them out: with boxes of single pixels of 128 images, 9 %
+// of the k-blocks of a padded 27 x 27 map (5 x 5 taps), 10 % of a 13 x 13 one (3 x 3).  Chosen: the extents with
+// the fewest (box, tap) pairs; taken where that is less than the raster tiles' (batch 256: 112.5 -> 103 us and
+// 42.7 / 56.8 / 37.9 -> 40 / 52 / 35.2; batch 64 of the former the same, 36 to 37).  A k-block takes the same
+// time with either load.
+static long long conv_boxes(const qnn_conv_desc *cv, int *w, int *h, int *n) {
+    const int OH = qnn_conv_out_h(cv), OW = qnn_conv_out_w(cv), taps = cv->KH * cv->KW;
+    const char *force = getenv("QNN_CONV_BOX");                // "0": never, "1": wherever the kernel can (tests)
+    if (cv->stride != 1 || (force && force[0] == '0') || (cv->pad == 0 && !(force && force[0] == '1'))) return 0;
+    const long long raster = ((long long)cv->B * OH * OW + TC_BP - 1) / TC_BP * taps;
+    // taps of one dimension that meet the image, summed over the boxes of `size` pixels along it
+    auto met = [&](int out, int size, int in, int k) {
+        long long sum = 0;
+        for (int o = 0; o < out; o += size) {
+            const int lo = cv->pad - o - (size - 1) > 0 ? cv->pad - o - (size - 1) : 0, hi = in + cv->pad - o < k ? in + cv->pad - o : k;
+            sum += hi > lo ? hi - lo : k;
+        }
+        return sum;
+    };
+    long long best = 0, boxes = 0;
+    // the smallest extents that make nw x nh boxes of an image, larger ones first
+    for (int nw = ceil_div(OW, TC_BP), bw = 0; nw <= OW; ++nw) {
+        if (ceil_div(OW, nw) == bw) continue;
+        bw = ceil_div(OW, nw);
+        const long long met_w = met(OW, bw, cv->W, cv->KW);
+        for (int nh = ceil_div(OH, TC_BP / bw), bh = 0; nh <= OH; ++nh) {
+            if (ceil_div(OH, nh) == bh) continue;
+            bh = ceil_div(OH, nh);
+            const int bn = cv->B < TC_BP / (bw * bh) ? cv->B : TC_BP / (bw * bh);
+            const long long nn = ceil_div(cv->B, bn), pairs = met_w * met(OH, bh, cv->H, cv->KH) * nn;
+            if (best == 0 || pairs < best) { best = pairs; boxes = nn * ceil_div(OW, bw) * ceil_div(OH, bh); *w = bw; *h = bh; *n = bn; }
+        }
+    }
+    return best < raster || (force && force[0] == '1') ? boxes : 0;
 }
 
 // Shared memory of a LOWER kernel besides its two staging buffers.
@@ -1541,9 +1649,20 @@ static qnn_status tc_launch(const qnn_gemm_desc *d, const qnn_conv_desc *cv, con
                             const int32_t *thr, void *out, void *ws, size_t ws_bytes, cudaStream_t s) {
     const int ld = round_up(d->K, 16);
     const int sms = sm_count();
-    const bool pair = choose_pair_kernel(d, sms);
-
     TcParams p;
+    p.bx_w = p.bx_h = p.bx_n = p.nb_w = p.nb_h = p.nb_n = 0;
+    const bool pair = choose_pair_kernel(d, sms);
+    int columns = d->N;                   // rows of the activation operand's tiles: those of boxes may not be full
+    if (cv && pair) {
+        const long long boxes = conv_boxes(cv, &p.bx_w, &p.bx_h, &p.bx_n);
+        if (boxes > 0 && boxes <= 0x7fffffff / TC_BP) {
+            p.nb_w = ceil_div(qnn_conv_out_w(cv), p.bx_w); p.nb_h = ceil_div(qnn_conv_out_h(cv), p.bx_h); p.nb_n = ceil_div(cv->B, p.bx_n);
+            columns = (int)boxes * TC_BP;
+        } else {
+            p.bx_w = 0;
+        }
+    }
+
     p.thr = thr; p.out = out; p.M = d->M; p.N = d->N; p.K = d->K;
     p.num_kb = ceil_div(d->K, TC_BK);
     p.ld_out = round_up(d->M, 16);
@@ -1554,6 +1673,7 @@ static qnn_status tc_launch(const qnn_gemm_desc *d, const qnn_conv_desc *cv, con
         p.taps = cv->KH * cv->KW; p.cchunks = ceil_div(cv->C, TC_BK);
         p.cv_C = cv->C; p.cv_KW = cv->KW; p.cv_stride = cv->stride; p.cv_pad = cv->pad;
         p.cv_OW = qnn_conv_out_w(cv); p.cv_OHW = qnn_conv_out_h(cv) * p.cv_OW;
+        p.lw_H = cv->H; p.lw_W = cv->W;
         p.num_kb = p.taps * p.cchunks;
     }
     const double wmax = d->w_enc == QNN_ENC_BIPOLAR ? 1.0
@@ -1572,12 +1692,13 @@ static qnn_status tc_launch(const qnn_gemm_desc *d, const qnn_conv_desc *cv, con
     if (pair) {
         if (cv) {
             const int pitch = cv->in_pitch ? cv->in_pitch : round_up(cv->C, 16);
-            if (!make_im2col_map(&ma, A, cv, pitch)) return QNN_ERR_UNSUPPORTED;     // caller lowers explicitly
+            if (!(p.bx_w ? make_box_map(&ma, A, cv, pitch, p.bx_w, p.bx_h, p.bx_n) : make_im2col_map(&ma, A, cv, pitch)))
+                return QNN_ERR_UNSUPPORTED;                    // caller lowers explicitly
         } else if (!make_map(&ma, A, d->N, d->K, ld, TC_BP)) {
             return QNN_ERR_CUDA;
         }
         if (!make_map(&mw, W, d->M, d->K, ld, 128)) return QNN_ERR_CUDA;
-        p.tiles_p = ceil_div(d->N, 256); p.tiles_c = ceil_div(d->M, T2_BN);
+        p.tiles_p = ceil_div(columns, 256); p.tiles_c = ceil_div(d->M, T2_BN);
         p.units = p.full_units = p.tiles_p * p.tiles_c;
         p.idesc = idesc_base | ((uint32_t)(256 >> 4) << 24);          // the kernel adds the tile's N
         // a workspace from the caller lets the last, at most half-filled round be split between pairs
@@ -1692,7 +1813,7 @@ qnn_status gemm_tc_lower_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g,
     p.thr = thr; p.out = out; p.M = g->M; p.N = g->N; p.K = g->K;
     p.num_kb = ceil_div(g->K, TC_BK);
     p.ld_out = round_up(g->M, 16);
-    p.kb_half = 0; p.share = 0;
+    p.kb_half = 0; p.share = 0; p.bx_w = 0;
     p.taps = 0; p.cchunks = 1; p.cv_C = cv->C; p.cv_KW = cv->KW; p.cv_pad = cv->pad;
     p.cv_stride = cv->stride; p.cv_OW = OW; p.cv_OHW = OH * OW;
     p.lw_in = reinterpret_cast<const uint8_t *>(in);

@@ -175,6 +175,13 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
         "[%0], [%1, {%3, %4}], [%2];"
         ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(x), "r"(y) : "memory");
 }
+__device__ __forceinline__ void tma_load_4d_pair(void *dst, const CUtensorMap *map, uint32_t bar_cluster_addr, int c, int w,
+                                                 int h, int n) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c), "r"(w), "r"(h), "r"(n) : "memory");
+}
 // im2col-mode load of a CTA pair's kernel (see tma_load_im2col); completion bytes are counted on
 // the barrier at cluster address `bar_cluster_addr` (the pair leader's).  No multicast.
 __device__ __forceinline__ void tma_load_im2col_pair(void *dst, const CUtensorMap *map, uint32_t bar_cluster_addr,
