@@ -15,7 +15,8 @@ CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 OBJ_DIR = os.path.join(_HERE, "_build")
 LIB = os.path.join(_HERE, "libqnn_b200.so")
-FASTCALL = os.path.join(_HERE, "_fastcall.so")       # the binding's host path (csrc/fastcall.c)
+# the binding's host path (csrc/fastcall.c); the name carries the interpreter's ABI, so that no other one loads it
+FASTCALL = os.path.join(_HERE, "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -44,6 +45,27 @@ def _compile(src, verbose):
     return obj, r.stderr
 
 
+def _build_fastcall(force: bool = False) -> bool:
+    """The extension module, if there is a C compiler and the interpreter's headers; without it the binding
+    makes the same calls through ctypes."""
+    src = os.path.join(CSRC, "fastcall.c")
+    if not force and os.path.exists(FASTCALL) and os.path.getmtime(FASTCALL) >= os.path.getmtime(src):
+        return True
+    # what stands there was made from another source, or (without a tag) perhaps for another interpreter
+    for old in (FASTCALL, os.path.join(os.path.dirname(FASTCALL), "_fastcall.so")):
+        if os.path.exists(old):
+            os.remove(old)
+    cmd = ["gcc", "-O2", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"], src, "-o", FASTCALL]
+    try:
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        built, log = r.returncode == 0, r.stderr
+    except OSError as e:
+        built, log = False, str(e)
+    if not built:
+        print(f"{os.path.basename(FASTCALL)} not built, calls go through ctypes:\n{log}", file=sys.stderr)
+    return built
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ_DIR, exist_ok=True)
     hm = _headers_mtime()
@@ -62,9 +84,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if todo or not os.path.exists(LIB):
         cmd = ["nvcc", "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"]
         subprocess.run(cmd, check=True)
-    src = os.path.join(CSRC, "fastcall.c")
-    if force or not os.path.exists(FASTCALL) or os.path.getmtime(FASTCALL) < os.path.getmtime(src):
-        subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"], src, "-o", FASTCALL], check=True)
+    _build_fastcall(force)
     return LIB
 
 
