@@ -49,6 +49,9 @@ inline qnn_status launch_status() {
 // effect unless the next kernel asked for it), pdl_wait() is a no-op for a normally launched
 // kernel.  They are not launched that way themselves: early placement next to a draining kernel
 // packs the CTAs of a small grid onto few SMs, which halved the bit-serial kernel's speed.
+// A kernel launched this way is resident while the one ahead may still write what it will read, so it
+// reads global memory with plain loads only: ld.global.nc (__ldg, const __restrict__) is for data that
+// nothing writes as long as the kernel lives.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

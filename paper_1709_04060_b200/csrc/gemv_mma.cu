@@ -86,17 +86,18 @@ __device__ __forceinline__ void mv_mma16(int (&d)[4], const uint32_t (&a)[4], ui
 
 // V words of global memory.  volatile: the loads stay where they are written, all of a warp's first ones
 // ahead of everything that waits for one of them.  Whole 16-byte units of weights are streamed (nothing
-// reads them again); smaller ones leave the rest of their sector to the warp's next load.
+// reads them again); smaller ones leave the rest of their sector to the warp's next load.  Not .nc: the
+// kernel is resident while the one ahead may still write the activations.
 template <int V, bool STREAM>
 __device__ __forceinline__ void mv_load(uint32_t *w, const uint8_t *p) {
     if (V == 4 && STREAM)
         asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1 % V]), "=r"(w[2 % V]), "=r"(w[3 % V]) : "l"(p));
     else if (V == 4)
-        asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1 % V]), "=r"(w[2 % V]), "=r"(w[3 % V]) : "l"(p));
+        asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1 % V]), "=r"(w[2 % V]), "=r"(w[3 % V]) : "l"(p));
     else if (V == 2)
-        asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1 % V]) : "l"(p));
+        asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1 % V]) : "l"(p));
     else
-        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w[0]) : "l"(p));
+        asm volatile("ld.global.u32 %0, [%1];" : "=r"(w[0]) : "l"(p));
 }
 
 // A word of every plane of a weight row -> eight registers of four bytes, in pairs: pair k holds the
