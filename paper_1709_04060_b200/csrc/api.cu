@@ -437,11 +437,12 @@ qnn_status qnn_qconv_maxpool(const qnn_conv_desc *d, int k, int stride, const vo
     if (st != QNN_OK) return st;
     qnn_gemm_desc g;
     conv_to_gemm(d, &g);
-    st = check_gemm_desc(&g, true, nullptr);
+    int path = 0;
+    st = check_gemm_desc(&g, true, &path);
     if (st != QNN_OK) return st;
     if (!Wpacked || !in || !thr || !out || k <= 0 || stride <= 0) return QNN_ERR_INVALID_ARG;
     if (!aligned16(Wpacked) || !aligned16(in) || !aligned16(out) || !aligned4(thr)) return QNN_ERR_ALIGNMENT;
-    if (!qnn_conv_maxpool_fuses(d, k, stride)) return QNN_ERR_UNSUPPORTED;
+    if (k != 3 || stride != 2 || path != QNN_PATH_TCGEN05_I8) return QNN_ERR_UNSUPPORTED;
     return conv_direct_launch(d, &g, Wpacked, in, thr, out, true, (cudaStream_t)stream);
 }
 

@@ -25,8 +25,6 @@
 // are contiguous); warps 2-5 turn them into ring slots; the next ones lay out the weights, then run the
 // epilogue, one 32 x 32 part of a tile per warp; with the pool in the kernel, four more take the maxima
 // from the codes of the last three tiles, which the epilogue leaves in shared memory.
-#include <stdlib.h>
-
 #include "tc_epilogue.cuh"
 #include "tc_ptx.cuh"
 
@@ -492,8 +490,7 @@ static bool dc_plan(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool pool, 
     }
     const long long tiles = (long long)cv->B * p->tiles_image;
     if (tiles > 0x3fffffff) return false;
-    const char *force = getenv("QNN_CONV_DIRECT");                 // "0": never, "1": whatever the size (tests)
-    if (force ? force[0] == '0' : tiles < (long long)DC_MIN_ROUNDS * sm_count()) return false;
+    if (tiles < (long long)DC_MIN_ROUNDS * sm_count()) return false;
     p->tiles = (int)tiles;
     p->per = ceil_div(p->tiles, sm_count());
     p->M = g->M; p->N = g->N; p->ld_out = round_up(g->M, 16);

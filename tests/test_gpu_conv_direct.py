@@ -20,11 +20,6 @@ def qb():
     return binding
 
 
-@pytest.fixture(autouse=True)
-def every_size(monkeypatch):
-    monkeypatch.setenv("QNN_CONV_DIRECT", "1")
-
-
 def layer(qb, B, H, W, OC, KH, KW, stride, w_bits, a_bits, out_bits, w_enc, a_enc, seed):
     case = synth.conv_case(seed, B, H, W, 3, OC, KH, KW, stride, 0, w_bits, a_bits, w_enc=w_enc, a_enc=a_enc, out_bits=out_bits)
     rows = np.zeros((OC, KH, round_up(KW * 3, 16)), dtype=np.int32)
@@ -34,15 +29,16 @@ def layer(qb, B, H, W, OC, KH, KW, stride, w_bits, a_bits, out_bits, w_enc, a_en
     return case, Wp, x, torch.from_numpy(case.thr).cuda()
 
 
+# (as many images as make five rounds of tiles on 148 SMs, from where the library takes this kernel)
 SHAPES = [
     # B, H, W, OC, KH, KW, stride, w_bits, a_bits, out_bits, w_enc, a_enc
-    (3, 227, 227, 96, 11, 11, 4, 8, 8, 2, 1, 0),      # the layer of the network; last tile half empty
-    (160, 15, 15, 20, 11, 11, 4, 4, 8, 2, 1, 0),      # four pixels an image, more images than SMs
-    (2, 61, 255, 128, 7, 5, 4, 2, 8, 1, 0, 0),        # 63 pixels a row, filter rows not a whole unit
-    (1, 40, 131, 33, 3, 3, 2, 8, 8, 3, 1, 1),         # stride 2, signed activations, 65 pixels a row
-    (2, 19, 100, 64, 3, 4, 1, 1, 8, 4, 2, 0),         # stride 1, +-1 weights against the pad bytes
-    (5, 33, 37, 1, 1, 1, 4, 8, 8, 2, 1, 0),           # a single tap
-    (2, 30, 29, 17, 9, 3, 2, 3, 4, 2, 1, 0),          # filter taller than wide
+    (28, 227, 227, 96, 11, 11, 4, 8, 8, 2, 1, 0),     # the layer of the network; last tile half empty
+    (760, 15, 15, 20, 11, 11, 4, 4, 8, 2, 1, 0),      # four pixels an image, several images a CTA
+    (125, 61, 255, 128, 7, 5, 4, 2, 8, 1, 0, 0),      # 63 pixels a row, filter rows not a whole unit
+    (40, 40, 131, 33, 3, 3, 2, 8, 8, 3, 1, 1),        # stride 2, signed activations, 65 pixels a row
+    (44, 19, 100, 64, 3, 4, 1, 1, 8, 4, 2, 0),        # stride 1, +-1 weights against the pad bytes
+    (250, 33, 37, 1, 1, 1, 4, 8, 8, 2, 1, 0),         # a single tap
+    (373, 30, 29, 17, 9, 3, 2, 3, 4, 2, 1, 0),        # filter taller than wide
 ]
 
 
@@ -68,11 +64,14 @@ def test_rows_read_in_place(qb, shape):
         assert np.array_equal(got, want_raw if raw else want)
 
 
-@pytest.mark.parametrize("shape", [s for s in SHAPES if s[2] in (227, 255, 131)] + [
-    (40, 143, 143, 96, 11, 11, 4, 8, 8, 2, 1, 0),     # 34 x 34 map, 16 pooled rows, CTAs that span images
-    (1, 19, 227, 32, 11, 11, 4, 8, 8, 4, 1, 0),       # three rows: one pooled row
+@pytest.mark.parametrize("shape,fuses", [(s, s[2] != 131) for s in SHAPES if s[2] in (227, 255, 131)] + [
+    ((47, 143, 143, 96, 11, 11, 4, 8, 8, 2, 1, 0), True),      # 34 x 34 map, 16 pooled rows, CTAs that span images
+    ((745, 19, 227, 32, 11, 11, 4, 8, 8, 4, 1, 0), True),      # three rows: one pooled row; 15 thresholds
+    ((93, 20, 50, 40, 3, 3, 1, 8, 8, 1, 1, 0), True),          # stride 1, 50 units a row; one threshold
+    ((107, 33, 101, 64, 5, 5, 2, 8, 8, 3, 1, 1), True),        # stride 2, 51 units a row; seven thresholds
+    ((93, 20, 40, 40, 3, 3, 1, 8, 8, 1, 1, 0), False),         # 40 units a row: three output rows a tile
 ])
-def test_pool_in_the_same_kernel(qb, shape):
+def test_pool_in_the_same_kernel(qb, shape, fuses):
     case, Wp, x, thr = layer(qb, *shape, seed=1900 + shape[1])
     OH, OW, PH, PW = case.OH, case.OW, (case.OH - 3) // 2 + 1, (case.OW - 3) // 2 + 1
     codes = orc.qconv(case.In, case.Wt, case.thr, case.stride, 0).reshape(case.B, OH, OW, case.OC)
@@ -80,7 +79,8 @@ def test_pool_in_the_same_kernel(qb, shape):
     for out_fmt in (INT8, BITPLANES):
         d = qb.qnn_conv_desc(case.B, case.H, case.Wd, 3, 3, case.OC, case.KH, case.KW, case.stride, 0, case.w_bits,
                              case.a_bits, case.out_bits, case.w_enc, case.a_enc, INT8, out_fmt, 0)
-        if not qb.qnn_conv_maxpool_fuses(d, 3, 2):
+        assert qb.qnn_conv_maxpool_fuses(d, 3, 2) == fuses
+        if not fuses:
             assert qb.qnn_qconv_maxpool(d, 3, 2, Wp, x, thr, x) == qb.QNN_ERR_UNSUPPORTED
             continue
         npix = case.B * PH * PW
@@ -96,7 +96,7 @@ def test_pool_in_the_same_kernel(qb, shape):
 
 def test_only_that_pool_and_those_layers_fuse(qb):
     def d(**kw):
-        v = dict(B=2, H=227, W=227, C=3, in_pitch=3, OC=96, KH=11, KW=11, stride=4, pad=0, w_bits=8, a_bits=8, out_bits=2,
+        v = dict(B=28, H=227, W=227, C=3, in_pitch=3, OC=96, KH=11, KW=11, stride=4, pad=0, w_bits=8, a_bits=8, out_bits=2,
                  w_enc=1, a_enc=0, fmt=INT8, out_fmt=INT8, path=0)
         v.update(kw)
         return qb.qnn_conv_desc(*v.values())
@@ -108,6 +108,7 @@ def test_only_that_pool_and_those_layers_fuse(qb):
     assert not qb.qnn_conv_maxpool_fuses(d(OC=129), 3, 2)
     assert not qb.qnn_conv_maxpool_fuses(d(stride=3), 3, 2)
     assert not qb.qnn_conv_maxpool_fuses(d(pad=1), 3, 2)
+    assert not qb.qnn_conv_maxpool_fuses(d(B=27), 3, 2)        # fewer than five rounds of pooled rows
     t = torch.zeros(64, dtype=torch.uint8, device="cuda")
     n0 = qb.qnn_launch_count()
     assert qb.qnn_qconv_maxpool(d(pad=1), 3, 2, t, t, t, t) == qb.QNN_ERR_UNSUPPORTED
