@@ -311,6 +311,8 @@ def measure_other_configs(torch, qb, synth, peaks, measured):
     macs = {"conv1": 1.054e8, "conv2": 4.479e8, "conv3": 1.495e8, "conv4": 2.243e8, "conv5": 1.495e8,
             "fc6": 3.77e7, "fc7": 1.68e7, "fc8": 4.10e6}
     for (kind, d, Wp, thr, out), name in zip(plan.steps, plan.names):
+        if out is None:              # one kernel with the pool behind it; timed alone here
+            out = torch.empty(qb.qnn_conv_out_bytes(d, True), dtype=torch.uint8, device="cuda")
         x_in = img if prev is None else prev
         if kind == "conv":
             f = lambda i: qb.check(qb.qnn_qconv(d, Wp, x_in, thr, out, plan.workspace, plan.workspace.numel()))
@@ -795,6 +797,8 @@ def run_extras(args):
             ms = _time_calls(torch, lambda i: plan.forward(img), 30 if B == 1 else 10)
             per_layer = {}
             for (kind, d, Wp, thr, out), name in zip(plan.steps, plan.names):
+                if out is None:              # one kernel with the pool behind it; timed alone here
+                    out = torch.empty(qb.qnn_conv_out_bytes(d, True), dtype=torch.uint8, device="cuda")
                 x_in = img if name == "conv1" else prev
                 if kind == "conv":
                     f = lambda i: qb.check(qb.qnn_qconv(d, Wp, x_in, thr, out, plan.workspace, plan.workspace.numel()))

@@ -36,7 +36,8 @@ class AlexNetPlan:
     def __init__(self, net, B: int, mode: str = "auto", hw: int = 227):
         assert mode in ("tensor", "bitserial", "auto")
         self.B, self.mode, self.layers, self.hw = B, mode, list(net.layers), hw
-        self.steps = []          # (kind, desc, tensors...)
+        self.steps = []          # (kind, desc, tensors...); the last one is the output
+        self._fused = set()      # convolutions that run together with the pool behind them
         self.names = []
         H, C = hw, 3
         fmt_in = INT8            # the image is uint8, pixel pitch 3
@@ -64,7 +65,12 @@ class AlexNetPlan:
                                      L.w_enc, qb.QNN_ENC_UNSIGNED, fmt, out_fmt, qb.QNN_PATH_AUTO)
                 Wflat = qb.conv_weight_rows(d, Wl)
                 Wp = qb.pack(qb.to_device_logical(Wflat, L.w_enc), L.w_bits, L.w_enc, fmt)
-                out = torch.empty(qb.qnn_conv_out_bytes(d, thr is not None), dtype=torch.uint8, device="cuda")
+                # together with the pool behind it, the convolution leaves no map of its own
+                if L.pool and thr is not None and qb.qnn_conv_maxpool_fuses(d, 3, 2):
+                    self._fused.add(len(self.steps))
+                    out = None
+                else:
+                    out = torch.empty(qb.qnn_conv_out_bytes(d, thr is not None), dtype=torch.uint8, device="cuda")
                 ws_bytes = max(ws_bytes, qb.qnn_conv_workspace_bytes(d))
                 OH = qb.qnn_conv_out_h(d)
                 self.steps.append(("conv", d, Wp, thr_d, out))
@@ -95,17 +101,12 @@ class AlexNetPlan:
                 flat = L.OC
             fmt_in = out_fmt
         self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
-        # convolutions that run together with the pool behind them
-        self._fused = {i for i in range(len(self.steps) - 1)
-                       if self.steps[i][0] == "conv" and self.steps[i + 1][0] == "pool" and self.steps[i][3] is not None
-                       and qb.qnn_conv_maxpool_fuses(self.steps[i][1], self.steps[i + 1][1].k, self.steps[i + 1][1].stride)}
-        self._image = None       # input of the last forward pass
         self.n_classes = self.layers[-1].OC
 
     def forward(self, image: torch.Tensor, stream=None):
         """image: uint8 device tensor [B][H][W][3].  Returns int32 logits [B][n_classes]
         (a view of the plan's last buffer).  Enqueues only; does not synchronise."""
-        x = self._image = image
+        x = image
         for i, (kind, d, Wp, thr, out) in enumerate(self.steps):
             if i in self._fused:
                 _, pool, _, _, pooled = self.steps[i + 1]
@@ -140,16 +141,19 @@ class AlexNetPlan:
             logits = self.forward(image)
         return graph, logits
 
-    def intermediates(self):
-        """{step name: (output buffer, descriptor kind, descriptor)} for tests.  A convolution that runs
-        together with its pool leaves no map of its own: it is computed here from its present input (for
-        the first layer the image of the last forward pass)."""
-        for i in sorted(self._fused):
-            if i > 0 or self._image is not None:
-                _, d, Wp, thr, out = self.steps[i]
-                x = self.steps[i - 1][4] if i > 0 else self._image
+    def intermediates(self, image=None):
+        """{step name: (output buffer, descriptor kind, descriptor)} for tests, once a forward pass is
+        complete.  A convolution that runs together with its pool leaves no map of its own: given the image
+        of that pass, it is computed here, on the current stream; without it that entry is left out."""
+        maps = {n: (s[4], s[0], s[1]) for n, s in zip(self.names, self.steps) if s[4] is not None}
+        for i in self._fused:
+            _, d, Wp, thr, _ = self.steps[i]
+            x = self.steps[i - 1][4] if i > 0 else image
+            if x is not None:
+                out = torch.empty(qb.qnn_conv_out_bytes(d, True), dtype=torch.uint8, device="cuda")
                 qb.check(qb.qnn_qconv(d, Wp, x, thr, out, self.workspace, self.workspace.numel()))
-        return {n: (s[4], s[0], s[1]) for n, s in zip(self.names, self.steps)}
+                maps[self.names[i]] = (out, "conv", d)
+        return maps
 
     def launches_per_forward(self) -> int:
         """Kernels one forward pass launches (counted by the library on a dry call)."""

@@ -213,6 +213,28 @@ def test_alexnet_chain_per_layer(qb, mode, B):
     assert np.array_equal(logits.cpu().numpy().astype(np.int64), logits_ref)
 
 
+def test_alexnet_plan_keeps_neither_the_image_nor_a_map_it_does_not_write(qb):
+    """Batch 32 runs the first layer and its pool in one kernel."""
+    import weakref
+    from paper_1709_04060_b200.alexnet import AlexNetPlan
+    net = synth.alexnet_case(32)
+    plan = AlexNetPlan(net, 32)
+    img = torch.from_numpy(net.image.astype(np.uint8)).cuda()
+    plan.forward(img)
+    torch.cuda.synchronize()
+    assert plan.steps[0][4] is None
+    assert "conv1" not in plan.intermediates()
+    inter = plan.intermediates(img)
+    d = inter["conv1"][2]
+    codes = decode_out(inter["conv1"][0].cpu().numpy(), d.out_fmt, 2, 32 * 55 * 55, 96, False).reshape(32, 55, 55, 96)
+    pooled = np.max([codes[:, i:i + 53:2, j:j + 53:2] for i in range(3) for j in range(3)], axis=0)
+    got = decode_out(inter["conv1_pool"][0].cpu().numpy(), inter["conv1_pool"][2].fmt, 2, 32 * 27 * 27, 96, False)
+    assert np.array_equal(got, pooled.reshape(-1, 96))
+    gone = weakref.ref(img)
+    del img
+    assert gone() is None
+
+
 def test_alexnet_chain_graph_replay(qb):
     """The chain recorded into a CUDA graph gives the oracle's logits on replay, also after
     the input buffer has been overwritten with another batch."""
