@@ -286,6 +286,11 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
                      const int32_t *thr, void *out,
                      void *workspace, size_t workspace_bytes, void *stream);
 
+/* The boxes of w x h output pixels of n images that the CTA-pair kernel cuts a large padded layer of stride 1 on
+ * an 8-bit map into, so as to leave out filter taps that lie outside the image: their number; 0 where the layer
+ * takes consecutive pixels or another kernel.  Host only. */
+int qnn_conv_boxes(const qnn_conv_desc *d, int *w, int *h, int *n);
+
 /* Convolution and the max-pool behind it (Section 4.2) in one kernel: the un-pooled map never reaches
  * global memory.  Arguments as for qnn_qconv, without a workspace, thr required; `out` is the pooled map,
  * [B][(OH-k)/stride+1][(OW-k)/stride+1][...] in d->out_fmt, i.e. what qnn_maxpool makes of qnn_qconv's output.

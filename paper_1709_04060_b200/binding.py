@@ -36,7 +36,7 @@ EXPORTS = (
     "qnn_packed_ld", "qnn_packed_bytes", "qnn_pack", "qnn_planes_to_int8", "qnn_gemm_workspace_bytes",
     "qnn_gemm_out_bytes", "qnn_qgemm", "qnn_qgemm_kernel", "qnn_qgemm_kernel_name", "qnn_conv_out_h", "qnn_conv_out_w",
     "qnn_conv_lowered_k", "qnn_conv_lowered_bytes", "qnn_conv_workspace_bytes",
-    "qnn_conv_out_bytes", "qnn_im2col", "qnn_qconv", "qnn_conv_maxpool_fuses", "qnn_qconv_maxpool", "qnn_qconv_static", "qnn_maxpool",
+    "qnn_conv_out_bytes", "qnn_im2col", "qnn_qconv", "qnn_conv_boxes", "qnn_conv_maxpool_fuses", "qnn_qconv_maxpool", "qnn_qconv_static", "qnn_maxpool",
     "qnn_streamline", "qnn_peak_mma_i8", "qnn_peak_popc", "qnn_peak_popc_sink_bytes", "qnn_validate_thresholds", "qnn_device_status", "qnn_launch_count",
     "qnn_status_string", "qnn_version",
 )
@@ -99,6 +99,8 @@ _lib.qnn_im2col.restype = _ci
 _lib.qnn_im2col.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp]
 _lib.qnn_qconv.restype = _ci
 _lib.qnn_qconv.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp]
+_lib.qnn_conv_boxes.restype = _ci
+_lib.qnn_conv_boxes.argtypes = [_P(qnn_conv_desc), _P(_ci), _P(_ci), _P(_ci)]
 _lib.qnn_conv_maxpool_fuses.restype = _ci
 _lib.qnn_conv_maxpool_fuses.argtypes = [_P(qnn_conv_desc), _ci, _ci]
 _lib.qnn_qconv_maxpool.restype = _ci
@@ -285,6 +287,14 @@ def qnn_im2col(d, inp, lowered, stream=None) -> int:
 
 def qnn_qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream=None) -> int:
     return _qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream)
+
+
+def qnn_conv_boxes(d):
+    """Boxes of output pixels that the CTA-pair kernel cuts this layer into: (number, width, height, images), or
+    None where it takes consecutive pixels or another kernel takes the layer."""
+    w, h, n = _ci(), _ci(), _ci()
+    boxes = _lib.qnn_conv_boxes(ctypes.byref(d), ctypes.byref(w), ctypes.byref(h), ctypes.byref(n))
+    return (boxes, w.value, h.value, n.value) if boxes else None
 
 
 def qnn_conv_maxpool_fuses(d, k: int, stride: int) -> bool:

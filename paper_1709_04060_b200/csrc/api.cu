@@ -422,6 +422,15 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
     return qnn_qgemm(&g, Wpacked, workspace, thr, out, nullptr, 0, stream);
 }
 
+int qnn_conv_boxes(const qnn_conv_desc *d, int *w, int *h, int *n) {
+    qnn_gemm_desc g;
+    int path = 0;
+    if (check_conv_desc(d) != QNN_OK || !w || !h || !n) return 0;
+    conv_to_gemm(d, &g);
+    if (check_gemm_desc(&g, false, &path) != QNN_OK || path != QNN_PATH_TCGEN05_I8) return 0;
+    return gemm_tc_conv_boxes(d, &g, w, h, n);
+}
+
 int qnn_conv_maxpool_fuses(const qnn_conv_desc *d, int k, int stride) {
     qnn_gemm_desc g;
     int path = 0;

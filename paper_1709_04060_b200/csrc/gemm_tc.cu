@@ -1411,28 +1411,77 @@ static bool make_box_map(CUtensorMap *map, const void *base, const qnn_conv_desc
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Boxes of output pixels for the CTA-pair kernel (0: im2col loads).  A box knows which filter taps fall outside
-// the image for all of its pixels, and the pair leaves them out: with boxes of single pixels of 128 images, 9 %
-// of the k-blocks of a padded 27 x 27 map (5 x 5 taps), 10 % of a 13 x 13 one (3 x 3).  Chosen: the extents with
-// the fewest (box, tap) pairs; taken where that is less than the raster tiles' (batch 256: 112.5 -> 103 us and
-// 42.7 / 56.8 / 37.9 -> 40 / 52 / 35.2; batch 64 of the former the same, 36 to 37).  A k-block takes the same
-// time with either load.
-static long long conv_boxes(const qnn_conv_desc *cv, int *w, int *h, int *n) {
-    const int OH = qnn_conv_out_h(cv), OW = qnn_conv_out_w(cv), taps = cv->KH * cv->KW;
-    const char *force = getenv("QNN_CONV_BOX");                // "0": never, "1": wherever the kernel can (tests)
-    if (cv->stride != 1 || (force && force[0] == '0') || (cv->pad == 0 && !(force && force[0] == '1'))) return 0;
-    const long long raster = ((long long)cv->B * OH * OW + TC_BP - 1) / TC_BP * taps;
-    // taps of one dimension that meet the image, summed over the boxes of `size` pixels along it
+// Filter taps of one dimension (`in` image pixels, `k` taps) that meet the image for the box of `size` output pixels
+// that starts at pixel o: [lo, hi); all of them where none do.
+static void box_taps(const qnn_conv_desc *cv, int size, int in, int k, int o, int *lo, int *hi) {
+    *lo = cv->pad - o - (size - 1) > 0 ? cv->pad - o - (size - 1) : 0;
+    *hi = in + cv->pad - o < k ? in + cv->pad - o : k;
+    if (*lo >= *hi) { *lo = 0; *hi = k; }
+}
+
+struct BoxPlan { int w, h, n; long long boxes; };
+
+// What a pair of SMs spends on a tile of kb k-blocks, in us: the main loop (0.43 a k-block with either load), or
+// the epilogue of the tile before where that takes longer.
+static double pair_tile_us(double kb) { return kb * 0.43 > 4.0 ? kb * 0.43 : 4.0; }
+
+// Tiles of one channel tile, and pairs, that boxes_us goes through.
+constexpr int BOX_TILES = 4096, BOX_PAIRS = 128;
+
+// Time of the busiest of `pairs` pairs of SMs, tiles dealt in turn as the kernel does, each with the taps that
+// its two boxes meet.
+static double boxes_us(const qnn_conv_desc *cv, const BoxPlan &b, int tiles_c, int pairs) {
+    const int nw = ceil_div(qnn_conv_out_w(cv), b.w), nn = ceil_div(cv->B, b.n), chunks = ceil_div(cv->C, TC_BK);
+    const int tiles_p = (int)((b.boxes + 1) / 2);
+    float tile[BOX_TILES], load[BOX_PAIRS] = {0.0f};
+    int h0, h1, w0, w1;
+    for (int t = 0; t < tiles_p; ++t) {
+        const int q0 = 2 * t / nn, q1 = (int)(2 * t + 1 < b.boxes ? 2 * t + 1 : b.boxes - 1) / nn;
+        box_taps(cv, b.h, cv->H, cv->KH, q0 / nw * b.h, &h0, &h1);
+        box_taps(cv, b.w, cv->W, cv->KW, q0 % nw * b.w, &w0, &w1);
+        if (q1 != q0) {
+            int lo, hi;
+            box_taps(cv, b.h, cv->H, cv->KH, q1 / nw * b.h, &lo, &hi);
+            h0 = lo < h0 ? lo : h0; h1 = hi > h1 ? hi : h1;
+            box_taps(cv, b.w, cv->W, cv->KW, q1 % nw * b.w, &lo, &hi);
+            w0 = lo < w0 ? lo : w0; w1 = hi > w1 ? hi : w1;
+        }
+        tile[t] = (float)pair_tile_us((double)(h1 - h0) * (w1 - w0) * chunks);
+    }
+    int at = 0;
+    for (int c = 0; c < tiles_c; ++c)
+        for (int t = 0; t < tiles_p; ++t) { load[at] += tile[t]; if (++at == pairs) at = 0; }
+    float most = 0.0f;
+    for (int i = 0; i < pairs; ++i) most = load[i] > most ? load[i] : most;
+    return most;
+}
+
+// Boxes of output pixels for the CTA-pair kernel (false: im2col loads of consecutive pixels).  A box knows which
+// filter taps fall outside the image for all of its pixels, and the pair leaves them out: with boxes of single pixels
+// of 128 images, 9 % of the k-blocks of a padded 27 x 27 map (5 x 5 taps), 10 % of a 13 x 13 one (3 x 3).  But
+// boxes rarely fill their 128 rows, and tiles are dealt in whole rounds: a round more costs what many taps save.
+// So of the extents with the smallest rounds times mean tile, the one whose busiest pair of SMs is done first, and
+// that only if consecutive pixels take longer.
+static bool conv_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan *plan) {
+    const int OH = qnn_conv_out_h(cv), OW = qnn_conv_out_w(cv), chunks = ceil_div(cv->C, TC_BK);
+    if (cv->stride != 1 || cv->pad == 0) return false;
+    auto rounds_us = [&](long long tiles_p, double kb) { return (double)((tiles_p * tiles_c + pairs - 1) / pairs) * pair_tile_us(kb); };
     auto met = [&](int out, int size, int in, int k) {
         long long sum = 0;
         for (int o = 0; o < out; o += size) {
-            const int lo = cv->pad - o - (size - 1) > 0 ? cv->pad - o - (size - 1) : 0, hi = in + cv->pad - o < k ? in + cv->pad - o : k;
-            sum += hi > lo ? hi - lo : k;
+            int lo, hi;
+            box_taps(cv, size, in, k, o, &lo, &hi);
+            sum += hi - lo;
         }
         return sum;
     };
-    long long best = 0, boxes = 0;
-    // the smallest extents that make nw x nh boxes of an image, larger ones first
+    constexpr double MARGIN = 0.98;
+    constexpr int KEPT = 4;
+    const double raster = rounds_us(((long long)cv->B * OH * OW + 255) / 256, (double)cv->KH * cv->KW * chunks);
+    BoxPlan best[KEPT];
+    double us[KEPT];
+    for (int i = 0; i < KEPT; ++i) us[i] = MARGIN * raster;
+    // the smallest extents that make nw x nh boxes of an image
     for (int nw = ceil_div(OW, TC_BP), bw = 0; nw <= OW; ++nw) {
         if (ceil_div(OW, nw) == bw) continue;
         bw = ceil_div(OW, nw);
@@ -1441,11 +1490,21 @@ static long long conv_boxes(const qnn_conv_desc *cv, int *w, int *h, int *n) {
             if (ceil_div(OH, nh) == bh) continue;
             bh = ceil_div(OH, nh);
             const int bn = cv->B < TC_BP / (bw * bh) ? cv->B : TC_BP / (bw * bh);
-            const long long nn = ceil_div(cv->B, bn), pairs = met_w * met(OH, bh, cv->H, cv->KH) * nn;
-            if (best == 0 || pairs < best) { best = pairs; boxes = nn * ceil_div(OW, bw) * ceil_div(OH, bh); *w = bw; *h = bh; *n = bn; }
+            const long long places = (long long)ceil_div(OW, bw) * ceil_div(OH, bh), boxes = places * ceil_div(cv->B, bn);
+            const double t = rounds_us((boxes + 1) / 2, (double)met_w * met(OH, bh, cv->H, cv->KH) / places * chunks);
+            if (t >= us[KEPT - 1] || boxes > 0x7fffff) continue;
+            int i = KEPT - 1;
+            for (; i > 0 && t < us[i - 1]; --i) { us[i] = us[i - 1]; best[i] = best[i - 1]; }
+            us[i] = t; best[i] = {bw, bh, bn, boxes};
         }
     }
-    return best < raster || (force && force[0] == '1') ? boxes : 0;
+    double least = MARGIN * raster;
+    for (int i = 0; i < KEPT && us[i] < MARGIN * raster; ++i) {
+        // (of many rounds every pair gets about the same)
+        const double t = best[i].boxes > 2 * BOX_TILES || pairs > BOX_PAIRS ? us[i] : boxes_us(cv, best[i], tiles_c, pairs);
+        if (t < least) { least = t; *plan = best[i]; }
+    }
+    return least < MARGIN * raster;
 }
 
 // Shared memory of a LOWER kernel besides its two staging buffers.
@@ -1654,12 +1713,11 @@ static qnn_status tc_launch(const qnn_gemm_desc *d, const qnn_conv_desc *cv, con
     const bool pair = choose_pair_kernel(d, sms);
     int columns = d->N;                   // rows of the activation operand's tiles: those of boxes may not be full
     if (cv && pair) {
-        const long long boxes = conv_boxes(cv, &p.bx_w, &p.bx_h, &p.bx_n);
-        if (boxes > 0 && boxes <= 0x7fffffff / TC_BP) {
+        BoxPlan b;
+        if (conv_boxes(cv, ceil_div(d->M, T2_BN), sms / 2, &b)) {
+            p.bx_w = b.w; p.bx_h = b.h; p.bx_n = b.n;
             p.nb_w = ceil_div(qnn_conv_out_w(cv), p.bx_w); p.nb_h = ceil_div(qnn_conv_out_h(cv), p.bx_h); p.nb_n = ceil_div(cv->B, p.bx_n);
-            columns = (int)boxes * TC_BP;
-        } else {
-            p.bx_w = 0;
+            columns = (int)b.boxes * TC_BP;
         }
     }
 
@@ -1750,6 +1808,12 @@ bool gemm_tc_conv_takes(const qnn_conv_desc *cv) {
     const int pitch = cv->in_pitch ? cv->in_pitch : round_up(cv->C, 16);
     if (cv->fmt != QNN_FMT_INT8 || (cv->C % 16) != 0 || (pitch % 16) != 0) return false;
     return cv->KH <= 255 && cv->KW <= 255 && cv->stride <= 8;
+}
+int gemm_tc_conv_boxes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, int *w, int *h, int *n) {
+    BoxPlan b;
+    if (!gemm_tc_conv_takes(cv) || !choose_pair_kernel(g, sm_count()) || !conv_boxes(cv, ceil_div(g->M, T2_BN), sm_count() / 2, &b)) return 0;
+    *w = b.w; *h = b.h; *n = b.n;
+    return (int)b.boxes;
 }
 qnn_status gemm_tc_conv_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
                                const int32_t *thr, void *out, bool any_size, cudaStream_t s) {

@@ -22,3 +22,67 @@ def test_the_environment_does_not_decide_what_fuses(qb, monkeypatch):
             monkeypatch.setenv("QNN_CONV_DIRECT", value)
         assert qb.qnn_conv_maxpool_fuses(big, 3, 2)
         assert not qb.qnn_conv_maxpool_fuses(small, 3, 2)
+
+
+def busiest_pair(cv, boxes):
+    """k-blocks (one channel chunk) of the SM pair with the most, of 74: tiles of two boxes, or of 256
+    consecutive pixels that meet every tap, dealt in turn."""
+    B, H, W, OC, KH, KW, pad = cv.B, cv.H, cv.W, cv.OC, cv.KH, cv.KW, cv.pad
+    OH, OW, tiles_c = H + 2 * pad - KH + 1, W + 2 * pad - KW + 1, -(-OC // 256)
+    if boxes is None:
+        tiles = [KH * KW] * -(-B * OH * OW // 256)
+    else:
+        count, w, h, n = boxes
+        nn, nw = -(-B // n), -(-OW // w)
+        assert count == nn * nw * -(-OH // h) and w * h * n <= 128
+
+        def taps(q):
+            oh, ow = q // nw * h, q % nw * w
+            rows = {k for o in range(oh, oh + h) for k in range(KH) if 0 <= o + k - pad < H}
+            cols = {k for o in range(ow, ow + w) for k in range(KW) if 0 <= o + k - pad < W}
+            return rows or set(range(KH)), cols or set(range(KW))
+        tiles = []
+        for t in range(-(-count // 2)):
+            (r0, c0), (r1, c1) = taps(2 * t // nn), taps(min(2 * t + 1, count - 1) // nn)
+            r, c = r0 | r1, c0 | c1
+            tiles.append((max(r) - min(r) + 1) * (max(c) - min(c) + 1))
+    load = [0] * 74
+    for u in range(len(tiles) * tiles_c):
+        load[u % 74] += tiles[u % len(tiles)]
+    return max(load)
+
+
+@pytest.mark.parametrize("B,H,C,OC,k,boxes", [
+    (64, 21, 512, 512, 3, False), (64, 17, 256, 512, 3, False), (14, 45, 96, 512, 3, False),      # a round more, or
+    (21, 30, 128, 512, 3, False), (18, 56, 64, 256, 5, False), (64, 27, 96, 256, 5, False),       # nothing gained
+    (256, 27, 96, 256, 5, True), (256, 13, 256, 384, 3, True), (256, 13, 384, 384, 3, True), (256, 13, 384, 256, 3, True),
+])
+def test_boxes_by_rounds(qb, B, H, C, OC, k, boxes):
+    cv = conv(qb, B, H, H, C, OC, k, k, 1, k // 2)
+    plan = qb.qnn_conv_boxes(cv)
+    assert (plan is not None) == boxes
+    if boxes:
+        assert busiest_pair(cv, plan) < busiest_pair(cv, None)
+
+
+def test_boxes_never_keep_a_pair_of_sms_busier(qb):
+    import random
+    rng, taken = random.Random(5), 0
+    for _ in range(1500):
+        k = rng.choice([3, 3, 5, 7])
+        B, H, W, OC = rng.choice([8, 16, 33, 64, 128, 250]), rng.randint(4, 60), rng.randint(4, 60), rng.choice([256, 384, 512, 1000])
+        if B * H * W > 300000:
+            continue
+        cv = conv(qb, B, H, W, rng.choice([96, 128, 256]), OC, k, k, 1, rng.choice([1, k // 2]))
+        plan = qb.qnn_conv_boxes(cv)
+        if plan is not None:
+            taken += 1
+            assert busiest_pair(cv, plan) <= 0.98 * busiest_pair(cv, None), (B, H, W, OC, k, plan)
+    assert taken > 100
+
+
+def test_only_padded_layers_of_stride_one_take_boxes(qb):
+    assert qb.qnn_conv_boxes(conv(qb, 256, 27, 27, 96, 256, 5, 5, 1, 0)) is None
+    assert qb.qnn_conv_boxes(conv(qb, 256, 27, 27, 96, 256, 5, 5, 2, 2)) is None
+    assert qb.qnn_conv_boxes(conv(qb, 1, 27, 27, 96, 256, 5, 5, 1, 2)) is None          # too small for SM pairs
+    assert qb.qnn_conv_boxes(conv(qb, 256, 27, 27, 90, 256, 5, 5, 1, 2)) is None        # not the tensor-map loader's

@@ -15,18 +15,17 @@ pytestmark = pytest.mark.gpu
 BITPLANES, INT8 = 0, 1
 
 
-@pytest.mark.parametrize("shape", [
-    # B, H, W, C, OC, KH, KW, stride, pad, w_bits, a_bits
-    (130, 5, 6, 96, 256, 5, 5, 1, 2, 1, 2),       # single pixels of 128 images, and of the last two
-    (300, 4, 4, 144, 300, 3, 3, 1, 1, 2, 2),      # 128 + 16 channel bytes, a channel tile of 64
-    (3, 13, 13, 256, 384, 3, 3, 1, 1, 1, 2),      # boxes of a few images: rows and columns
-    (1, 33, 50, 32, 64, 5, 3, 1, 1, 4, 3),        # one image, rectangular filter
-    (7, 9, 9, 64, 70, 3, 3, 1, 2, 2, 4),          # padding of two with three taps
-    (5, 12, 7, 48, 130, 1, 1, 1, 0, 3, 1),        # a single tap
+@pytest.mark.parametrize("shape,boxes", [
+    # B, H, W, C, OC, KH, KW, stride, pad, w_bits, a_bits; number, width, height, images
+    ((257, 5, 4, 96, 256, 5, 5, 1, 2, 1, 2), (60, 1, 1, 128)),       # single pixels of 128 images, and of the last one
+    ((300, 2, 3, 144, 300, 3, 3, 1, 1, 2, 2), (20, 2, 1, 64)),       # 128 + 16 channel bytes, a channel tile of 44
+    ((257, 17, 9, 48, 70, 5, 5, 1, 2, 4, 3), (405, 1, 4, 32)),       # an odd number; cut by the last row and image
+    ((130, 10, 18, 144, 70, 3, 3, 1, 3, 2, 4), (385, 2, 3, 21)),     # boxes outside the image; cut at all edges
+    ((3, 19, 3, 256, 300, 3, 5, 1, 1, 3, 1), (7, 1, 3, 3)),          # all images in a box, rectangular filter
+    ((65, 11, 2, 96, 300, 3, 5, 1, 2, 1, 2), (17, 2, 13, 4)),        # whole images
 ])
-def test_box_tiles(qb, monkeypatch, shape):  # noqa: F811
+def test_box_tiles(qb, monkeypatch, shape, boxes):  # noqa: F811
     monkeypatch.setenv("QNN_TC_KERNEL", "pair")
-    monkeypatch.setenv("QNN_CONV_BOX", "1")
     monkeypatch.setenv("QNN_CONV_LOWER", "0")
     monkeypatch.setenv("QNN_CONV_IMPLICIT", "1")
     case = synth.conv_case(1500 + shape[0], *shape)
@@ -37,6 +36,7 @@ def test_box_tiles(qb, monkeypatch, shape):  # noqa: F811
     want = (want_raw[:, :, None] >= case.thr[None]).sum(2)
     for out_fmt, raw in ((INT8, False), (BITPLANES, False), (INT8, True)):
         d = conv_desc(qb, case, INT8, out_fmt, pitch)
+        assert qb.qnn_conv_boxes(d) == boxes
         nb = qb.qnn_conv_out_bytes(d, not raw)
         out = torch.full((nb + 64,), 0xEE, dtype=torch.uint8, device="cuda")
         ws = torch.zeros(qb.qnn_conv_workspace_bytes(d), dtype=torch.uint8, device="cuda")
