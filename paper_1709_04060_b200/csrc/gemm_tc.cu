@@ -44,6 +44,7 @@
 // resident by construction, so neither can wait for one that is not running.
 #include <cuda.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include "common.cuh"
 #include "planes.cuh"
@@ -1462,9 +1463,8 @@ static double boxes_us(const qnn_conv_desc *cv, const BoxPlan &b, int tiles_c, i
 // boxes rarely fill their 128 rows, and tiles are dealt in whole rounds: a round more costs what many taps save.
 // So of the extents with the smallest rounds times mean tile, the one whose busiest pair of SMs is done first, and
 // that only if consecutive pixels take longer.
-static bool conv_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan *plan) {
+static bool search_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan *plan) {
     const int OH = qnn_conv_out_h(cv), OW = qnn_conv_out_w(cv), chunks = ceil_div(cv->C, TC_BK);
-    if (cv->stride != 1 || cv->pad == 0) return false;
     auto rounds_us = [&](long long tiles_p, double kb) { return (double)((tiles_p * tiles_c + pairs - 1) / pairs) * pair_tile_us(kb); };
     auto met = [&](int out, int size, int in, int k) {
         long long sum = 0;
@@ -1477,6 +1477,9 @@ static bool conv_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan 
     };
     constexpr double MARGIN = 0.98;
     constexpr int KEPT = 4;
+    // single pixels leave out the most: too little in a large map (224 x 224, 3 x 3: 1.2 %)
+    const double fewest = (double)met(OW, 1, cv->W, cv->KW) * met(OH, 1, cv->H, cv->KH) / ((double)OW * OH) * chunks;
+    if (pair_tile_us(fewest) >= MARGIN * pair_tile_us((double)cv->KH * cv->KW * chunks)) return false;
     const double raster = rounds_us(((long long)cv->B * OH * OW + 255) / 256, (double)cv->KH * cv->KW * chunks);
     BoxPlan best[KEPT];
     double us[KEPT];
@@ -1505,6 +1508,25 @@ static bool conv_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan 
         if (t < least) { least = t; *plan = best[i]; }
     }
     return least < MARGIN * raster;
+}
+
+// The same, searched once per shape and thread (the search takes 5 to 15 us for maps of 13 to 56 pixels, up to 50
+// for larger ones; a call of the library some 2).
+static bool conv_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan *plan) {
+    if (cv->stride != 1 || cv->pad == 0) return false;
+    struct Entry { int key[9]; bool found; BoxPlan plan; };
+    constexpr int ENTRIES = 32;                               // a shape displaces another of the same slot
+    static thread_local Entry table[ENTRIES] = {};
+    const int key[9] = {cv->B, cv->H, cv->W, cv->KH, cv->KW, cv->pad, ceil_div(cv->C, TC_BK), tiles_c, pairs};
+    unsigned slot = 0;
+    for (int k : key) slot = slot * 31 + (unsigned)k;
+    Entry &e = table[slot % ENTRIES];
+    if (memcmp(e.key, key, sizeof(key)) != 0) {
+        e.found = search_boxes(cv, tiles_c, pairs, &e.plan);
+        memcpy(e.key, key, sizeof(key));
+    }
+    *plan = e.plan;
+    return e.found;
 }
 
 // Shared memory of a LOWER kernel besides its two staging buffers.
