@@ -291,6 +291,9 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
  * takes consecutive pixels or another kernel.  Host only. */
 int qnn_conv_boxes(const qnn_conv_desc *d, int *w, int *h, int *n);
 
+/* Whether qnn_qconv runs this layer on the kernel that reads the rows of a three-channel map in place.  Host only. */
+int qnn_conv_in_place(const qnn_conv_desc *d, int has_thresholds);
+
 /* Convolution and the max-pool behind it (Section 4.2) in one kernel: the un-pooled map never reaches
  * global memory.  Arguments as for qnn_qconv, without a workspace, thr required; `out` is the pooled map,
  * [B][(OH-k)/stride+1][(OW-k)/stride+1][...] in d->out_fmt, i.e. what qnn_maxpool makes of qnn_qconv's output.

@@ -36,7 +36,7 @@ EXPORTS = (
     "qnn_packed_ld", "qnn_packed_bytes", "qnn_pack", "qnn_planes_to_int8", "qnn_gemm_workspace_bytes",
     "qnn_gemm_out_bytes", "qnn_qgemm", "qnn_qgemm_kernel", "qnn_qgemm_kernel_name", "qnn_conv_out_h", "qnn_conv_out_w",
     "qnn_conv_lowered_k", "qnn_conv_lowered_bytes", "qnn_conv_workspace_bytes",
-    "qnn_conv_out_bytes", "qnn_im2col", "qnn_qconv", "qnn_conv_boxes", "qnn_conv_maxpool_fuses", "qnn_qconv_maxpool", "qnn_qconv_static", "qnn_maxpool",
+    "qnn_conv_out_bytes", "qnn_im2col", "qnn_qconv", "qnn_conv_boxes", "qnn_conv_in_place", "qnn_conv_maxpool_fuses", "qnn_qconv_maxpool", "qnn_qconv_static", "qnn_maxpool",
     "qnn_streamline", "qnn_peak_mma_i8", "qnn_peak_popc", "qnn_peak_popc_sink_bytes", "qnn_validate_thresholds", "qnn_device_status", "qnn_launch_count",
     "qnn_status_string", "qnn_version",
 )
@@ -101,6 +101,8 @@ _lib.qnn_qconv.restype = _ci
 _lib.qnn_qconv.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp]
 _lib.qnn_conv_boxes.restype = _ci
 _lib.qnn_conv_boxes.argtypes = [_P(qnn_conv_desc), _P(_ci), _P(_ci), _P(_ci)]
+_lib.qnn_conv_in_place.restype = _ci
+_lib.qnn_conv_in_place.argtypes = [_P(qnn_conv_desc), _ci]
 _lib.qnn_conv_maxpool_fuses.restype = _ci
 _lib.qnn_conv_maxpool_fuses.argtypes = [_P(qnn_conv_desc), _ci, _ci]
 _lib.qnn_qconv_maxpool.restype = _ci
@@ -295,6 +297,11 @@ def qnn_conv_boxes(d):
     w, h, n = _ci(), _ci(), _ci()
     boxes = _lib.qnn_conv_boxes(ctypes.byref(d), ctypes.byref(w), ctypes.byref(h), ctypes.byref(n))
     return (boxes, w.value, h.value, n.value) if boxes else None
+
+
+def qnn_conv_in_place(d, has_thresholds: bool = True) -> bool:
+    """Whether qnn_qconv reads the rows of this three-channel map in place."""
+    return bool(_lib.qnn_conv_in_place(ctypes.byref(d), int(has_thresholds)))
 
 
 def qnn_conv_maxpool_fuses(d, k: int, stride: int) -> bool:

@@ -431,6 +431,15 @@ int qnn_conv_boxes(const qnn_conv_desc *d, int *w, int *h, int *n) {
     return gemm_tc_conv_boxes(d, &g, w, h, n);
 }
 
+int qnn_conv_in_place(const qnn_conv_desc *d, int has_thresholds) {
+    qnn_gemm_desc g;
+    int path = 0;
+    if (check_conv_desc(d) != QNN_OK) return 0;
+    conv_to_gemm(d, &g);
+    if (check_gemm_desc(&g, has_thresholds != 0, &path) != QNN_OK || path != QNN_PATH_TCGEN05_I8) return 0;
+    return conv_direct_takes(d, &g, has_thresholds != 0, false) ? 1 : 0;
+}
+
 int qnn_conv_maxpool_fuses(const qnn_conv_desc *d, int k, int stride) {
     qnn_gemm_desc g;
     int path = 0;

@@ -25,6 +25,8 @@
 // are contiguous); warps 2-5 turn them into ring slots; the next ones lay out the weights, then run the
 // epilogue, one 32 x 32 part of a tile per warp; with the pool in the kernel, four more take the maxima
 // from the codes of the last three tiles, which the epilogue leaves in shared memory.
+#include <math.h>
+
 #include "tc_epilogue.cuh"
 #include "tc_ptx.cuh"
 
@@ -432,13 +434,32 @@ conv_direct_kernel(const __grid_constant__ DcParams p) {
 }
 
 // ------------------------------------------------------------------- host side
-// From five rounds of tiles (pooled rows) per SM on: setting up (weights laid out, first rows) takes 7 us of a
-// launch.  227 x 227 -> 96, 11 x 11, us with the pool, the other kernels -> this one: batch 16 15.8 -> 15.0,
-// 24 19.6 -> 20.4, 32 26.4 -> 22.4, 64 42.8 -> 33.9, 256 151 -> 101; batch 1 8.7 -> 10.3.
+// Where this kernel is the faster one.  From five rounds of tiles (pooled rows) per SM on: setting up (weights laid
+// out, first rows) takes 7 us of a launch.  227 x 227 -> 96, 11 x 11, us with the pool, the other kernels -> this
+// one: batch 16 15.8 -> 15.0, 24 19.6 -> 20.4, 32 26.4 -> 22.4, 64 42.8 -> 33.9, 256 151 -> 101; batch 1 8.7 -> 10.3.
+// And where enough of the 128 operand rows of a tile carry a pixel: the kernel with lowering warps packs its tiles
+// densely and spends the same epilogue on each, but lowers every row (40 x 40 -> 8, 7 x 7, batch 78, half of the
+// rows used: 9.3 there, 20.9 here; 19 x 91 -> 32, 11 x 11, stride 2, batch 398: 16.5 and 47).  The share that is
+// enough depends on how long the epilogue takes (output bits, 32-channel parts).  The logarithm of the two times'
+// ratio is fitted to 835 random layers and, with the pool, 1702, those near 1 weighing most; below 0.92 (with the
+// pool 0.87) it is taken.  Raw sums are bound by their stores: 1.2 times as long here.
 constexpr int DC_MIN_ROUNDS = 5;
+static bool dc_faster(const DcParams &p, const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, bool pool) {
+    if (p.tiles < (long long)DC_MIN_ROUNDS * sm_count()) return false;
+    // +-1 weights against pad bytes: the kernel with lowering warps does not take them (0.5 of the time)
+    if (g->w_enc == QNN_ENC_BIPOLAR && cv->KW * 3 % 16 != 0) return true;
+    if (!has_thr) return false;
+    static const double bits[2][4] = {{0.173, 0.112, 0.091, 0.0}, {0.038, 0.007, 0.038, 0.0}};
+    static const double parts[2][4] = {{0.074, -0.049, -0.084, 0.0}, {0.095, -0.114, -0.079, 0.0}};
+    static const double base[2] = {-0.292, -0.080}, tile[2] = {0.5, -0.547}, slope[2] = {0.477, 0.419};
+    // row steps of a CTA: its tiles, and what the last one of an image reads beyond
+    const double steps = p.per + ((double)p.per / p.tiles_image + 1.0) * (p.extra + (pool ? 1 : 0));
+    const double used = (double)p.N / (128.0 * p.tiles) * p.per / steps;
+    return base[pool] + bits[pool][g->out_bits - 1] + parts[pool][p.chunks - 1] + tile[pool] / p.per < slope[pool] * log(used);
+}
 // The layers this kernel takes: three channels in contiguous pixels, no padding, up to 128 output channels,
 // a stride that divides 4, rows of up to 128 units.
-static bool dc_plan(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool pool, DcParams *p) {
+static bool dc_plan(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, bool pool, DcParams *p) {
     const int pitch = cv->in_pitch ? cv->in_pitch : round_up(cv->C, 16);
     if (cv->fmt != QNN_FMT_INT8 || cv->C != 3 || pitch != 3 || cv->pad != 0 || cv->OC > 128) return false;
     if (cv->stride != 1 && cv->stride != 2 && cv->stride != 4) return false;
@@ -490,10 +511,10 @@ static bool dc_plan(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool pool, 
     }
     const long long tiles = (long long)cv->B * p->tiles_image;
     if (tiles > 0x3fffffff) return false;
-    if (tiles < (long long)DC_MIN_ROUNDS * sm_count()) return false;
     p->tiles = (int)tiles;
     p->per = ceil_div(p->tiles, sm_count());
     p->M = g->M; p->N = g->N; p->ld_out = round_up(g->M, 16);
+    if (!dc_faster(*p, cv, g, has_thr, pool)) return false;
     p->w_ld = round_up(g->K, 16); p->w_run = round_up(cv->KW * 3, 16);
     p->w_total = (long long)g->M * p->w_ld;
     const double wmax = g->w_enc == QNN_ENC_BIPOLAR ? 1.0
@@ -528,14 +549,14 @@ static qnn_status dc_launch(const DcParams &p, size_t smem, cudaStream_t s) {
 
 bool conv_direct_takes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, bool pool) {
     DcParams p = {};
-    return dc_plan(cv, g, pool, &p) && (has_thr || !pool) && dc_smem_bytes(p, has_thr ? g->out_bits : 0, pool) <= SMEM_LIMIT;
+    return dc_plan(cv, g, has_thr, pool, &p) && (has_thr || !pool) && dc_smem_bytes(p, has_thr ? g->out_bits : 0, pool) <= SMEM_LIMIT;
 }
 
 // The convolution (UNSUPPORTED: the layer needs another kernel), with `pool` its 3 x 3, stride 2 max-pool too.
 qnn_status conv_direct_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
                               const int32_t *thr, void *out, bool pool, cudaStream_t s) {
     DcParams p = {};
-    if (!dc_plan(cv, g, pool, &p) || (pool && !thr)) return QNN_ERR_UNSUPPORTED;
+    if (!dc_plan(cv, g, thr != nullptr, pool, &p) || (pool && !thr)) return QNN_ERR_UNSUPPORTED;
     const size_t smem = dc_smem_bytes(p, thr ? g->out_bits : 0, pool);
     if (smem > SMEM_LIMIT) return QNN_ERR_UNSUPPORTED;
     p.in = (const uint8_t *)in; p.W = (const uint8_t *)W; p.thr = thr; p.out = out;

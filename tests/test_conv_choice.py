@@ -24,6 +24,38 @@ def test_the_environment_does_not_decide_what_fuses(qb, monkeypatch):
         assert not qb.qnn_conv_maxpool_fuses(small, 3, 2)
 
 
+def first_layer(qb, B, H, W, OC, k, stride, out_bits, w_enc=1):
+    return qb.qnn_conv_desc(B, H, W, 3, 3, OC, k, k, stride, 0, 1 if w_enc == 2 else 8, 8, out_bits, w_enc, 0, 1, 1, 0)
+
+
+@pytest.mark.parametrize("layer,in_place", [
+    # us, the kernel with lowering warps -> this one
+    ((398, 91, 19, 32, 11, 2, 1), False),       # 16.5 -> 47.1
+    ((78, 40, 40, 8, 7, 1, 1), False),          # 9.3 -> 20.9
+    ((147, 197, 20, 96, 7, 1, 1), False),       # 32.9 -> 81.6
+    ((425, 40, 40, 20, 11, 2, 3), False),       # 20.0 -> 32.5
+    ((424, 256, 256, 48, 7, 4, 2), True),       # 264 -> 100
+    ((479, 97, 23, 64, 1, 1, 2), True),         # 148 -> 68
+    ((256, 227, 227, 96, 11, 4, 2), True),      # 128 -> 97
+])
+def test_first_layers_in_place_where_tiles_are_full(qb, layer, in_place):
+    assert qb.qnn_conv_in_place(first_layer(qb, *layer)) == in_place
+    assert not qb.qnn_conv_in_place(first_layer(qb, *layer), False)                  # sums
+    assert qb.qnn_conv_in_place(first_layer(qb, *layer, w_enc=2), False)             # no other kernel lowers these inside
+
+
+@pytest.mark.parametrize("layer,fuses", [
+    ((162, 201, 137, 8, 11, 4, 3), False),      # 43.6 -> 84.0
+    ((201, 82, 82, 20, 5, 2, 4), False),        # 55.8 -> 87.0
+    ((500, 133, 133, 32, 5, 4, 1), False),      # 38.4 -> 66.8
+    ((342, 159, 216, 64, 1, 4, 2), True),       # 109 -> 58
+    ((32, 227, 227, 96, 11, 4, 2), True),       # 26.4 -> 22.4
+    ((256, 227, 227, 96, 11, 4, 2), True),      # 151 -> 101
+])
+def test_first_layers_fuse_with_their_pool_where_tiles_are_full(qb, layer, fuses):
+    assert qb.qnn_conv_maxpool_fuses(first_layer(qb, *layer), 3, 2) == fuses
+
+
 def busiest_pair(cv, boxes):
     """k-blocks (one channel chunk) of the SM pair with the most, of 74: tiles of two boxes, or of 256
     consecutive pixels that meet every tap, dealt in turn."""

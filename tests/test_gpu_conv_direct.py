@@ -29,16 +29,19 @@ def layer(qb, B, H, W, OC, KH, KW, stride, w_bits, a_bits, out_bits, w_enc, a_en
     return case, Wp, x, torch.from_numpy(case.thr).cuda()
 
 
-# (as many images as make five rounds of tiles on 148 SMs, from where the library takes this kernel)
+# Layers that the library itself runs this way: five rounds of tiles on 148 SMs and full ones, or +-1 weights, which
+# the kernel with lowering warps does not take.
 SHAPES = [
     # B, H, W, OC, KH, KW, stride, w_bits, a_bits, out_bits, w_enc, a_enc
     (28, 227, 227, 96, 11, 11, 4, 8, 8, 2, 1, 0),     # the layer of the network; last tile half empty
-    (760, 15, 15, 20, 11, 11, 4, 4, 8, 2, 1, 0),      # four pixels an image, several images a CTA
-    (125, 61, 255, 128, 7, 5, 4, 2, 8, 1, 0, 0),      # 63 pixels a row, filter rows not a whole unit
-    (40, 40, 131, 33, 3, 3, 2, 8, 8, 3, 1, 1),        # stride 2, signed activations, 65 pixels a row
-    (44, 19, 100, 64, 3, 4, 1, 1, 8, 4, 2, 0),        # stride 1, +-1 weights against the pad bytes
-    (250, 33, 37, 1, 1, 1, 4, 8, 8, 2, 1, 0),         # a single tap
-    (373, 30, 29, 17, 9, 3, 2, 3, 4, 2, 1, 0),        # filter taller than wide
+    (760, 15, 15, 20, 11, 11, 4, 1, 8, 2, 2, 0),      # four pixels an image, several images a CTA
+    (125, 61, 255, 128, 7, 5, 4, 1, 8, 1, 2, 0),      # 63 pixels a row, filter rows not a whole unit
+    (40, 40, 131, 33, 3, 3, 2, 1, 8, 3, 2, 1),        # stride 2, signed activations, 65 pixels a row
+    (44, 19, 100, 64, 3, 4, 1, 1, 8, 4, 2, 0),        # stride 1
+    (250, 33, 37, 1, 1, 1, 4, 1, 8, 2, 2, 0),         # a single tap
+    (373, 30, 29, 17, 9, 3, 2, 1, 4, 2, 2, 0),        # filter taller than wide
+    (96, 26, 207, 100, 1, 5, 2, 8, 8, 3, 1, 1),       # signed operands, stride 2
+    (223, 52, 210, 33, 2, 2, 2, 2, 8, 4, 0, 0),
 ]
 
 
@@ -51,6 +54,7 @@ def test_rows_read_in_place(qb, shape):
     for out_fmt, raw in ((INT8, False), (BITPLANES, False), (INT8, True)):
         d = qb.qnn_conv_desc(case.B, case.H, case.Wd, 3, 3, case.OC, case.KH, case.KW, case.stride, 0, case.w_bits,
                              case.a_bits, case.out_bits, case.w_enc, case.a_enc, INT8, out_fmt, 0)
+        assert qb.qnn_conv_in_place(d, not raw) == (not raw or case.w_enc == 2)       # sums: only +-1 weights
         nb = qb.qnn_conv_out_bytes(d, not raw)
         out = torch.full((nb + 64,), 0xEE, dtype=torch.uint8, device="cuda")
         ws = torch.zeros(qb.qnn_conv_workspace_bytes(d), dtype=torch.uint8, device="cuda")
@@ -65,11 +69,14 @@ def test_rows_read_in_place(qb, shape):
 
 
 @pytest.mark.parametrize("shape,fuses", [(s, s[2] != 131) for s in SHAPES if s[2] in (227, 255, 131)] + [
-    ((47, 143, 143, 96, 11, 11, 4, 8, 8, 2, 1, 0), True),      # 34 x 34 map, 16 pooled rows, CTAs that span images
-    ((745, 19, 227, 32, 11, 11, 4, 8, 8, 4, 1, 0), True),      # three rows: one pooled row; 15 thresholds
-    ((93, 20, 50, 40, 3, 3, 1, 8, 8, 1, 1, 0), True),          # stride 1, 50 units a row; one threshold
-    ((107, 33, 101, 64, 5, 5, 2, 8, 8, 3, 1, 1), True),        # stride 2, 51 units a row; seven thresholds
-    ((93, 20, 40, 40, 3, 3, 1, 8, 8, 1, 1, 0), False),         # 40 units a row: three output rows a tile
+    ((47, 143, 143, 96, 11, 11, 4, 1, 8, 2, 2, 0), True),      # 34 x 34 map, 16 pooled rows, CTAs that span images
+    ((745, 19, 227, 32, 11, 11, 4, 1, 8, 4, 2, 0), True),      # three rows: one pooled row; 15 thresholds
+    ((93, 20, 50, 40, 3, 3, 1, 1, 8, 1, 2, 0), True),          # stride 1, 48 pixels a row; one threshold
+    ((107, 33, 101, 64, 5, 5, 2, 1, 8, 3, 2, 1), True),        # stride 2, 49 pixels a row; seven thresholds
+    ((48, 142, 55, 70, 2, 3, 1, 8, 8, 4, 1, 0), True),         # stride 1, 8-bit weights, 15 thresholds
+    ((59, 83, 115, 70, 3, 7, 2, 8, 8, 4, 1, 1), True),
+    ((71, 65, 126, 70, 2, 7, 2, 8, 8, 1, 1, 0), True),
+    ((93, 20, 40, 40, 3, 3, 1, 1, 8, 1, 2, 0), False),         # 40 units a row: three output rows a tile
 ])
 def test_pool_in_the_same_kernel(qb, shape, fuses):
     case, Wp, x, thr = layer(qb, *shape, seed=1900 + shape[1])
