@@ -276,7 +276,7 @@ qnn_status qnn_im2col(const qnn_conv_desc *d, const void *in, void *lowered, voi
  * when C and in_pitch are multiples of 16 (the CTA-pair kernel for large layers,
  * the one-CTA kernel otherwise); by the operand descriptors of a kernel that keeps image rows
  * in shared memory when C is 3, pixels are contiguous, pad == 0, OC <= 128, the stride is 1, 2
- * or 4 and the layer has many tiles; by lowering warps when pixels are contiguous and either C
+ * or 4 and the layer has many tiles with few empty rows (qnn_conv_in_place); by lowering warps when pixels are contiguous and either C
  * is not a multiple of 16, pad == 0, OC <= 128 and the weights are not BIPOLAR, or C is a multiple of 16 but not of 128, the layer has many tiles and
  * the CTA-pair kernel does not apply.  All routes give the same integer results.
  * The pad columns of the weight rows (see qnn_conv_lowered_k) must be zero bytes
@@ -298,8 +298,9 @@ int qnn_conv_in_place(const qnn_conv_desc *d, int has_thresholds);
  * global memory.  Arguments as for qnn_qconv, without a workspace, thr required; `out` is the pooled map,
  * [B][(OH-k)/stride+1][(OW-k)/stride+1][...] in d->out_fmt, i.e. what qnn_maxpool makes of qnn_qconv's output.
  * Which layers fuse: qnn_conv_maxpool_fuses (host only; 1 or 0), i.e. large three-channel 8-bit maps
- * with contiguous pixels and no padding, a filter stride of 1, 2 or 4 and rows of 33 to 64 units (output
- * pixels plus ceil(KW / stride) - 1), with a 3 x 3 pool of stride 2.  The others return
+ * with contiguous pixels and no padding, a filter stride of 1, 2 or 4, rows of 41 to 64 units (output pixels plus
+ * ceil(KW / stride) - 1; from 33 at stride 4) that leave few operand rows empty, and filters that are not too
+ * deep for its buffers, with a 3 x 3 pool of stride 2.  The others return
  * QNN_ERR_UNSUPPORTED: call qnn_qconv and qnn_maxpool. */
 int qnn_conv_maxpool_fuses(const qnn_conv_desc *d, int k, int stride);
 qnn_status qnn_qconv_maxpool(const qnn_conv_desc *d, int k, int stride, const void *Wpacked, const void *in,
