@@ -446,8 +446,9 @@ conv_direct_kernel(const __grid_constant__ DcParams p) {
 constexpr int DC_MIN_ROUNDS = 5;
 static bool dc_faster(const DcParams &p, const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, bool pool) {
     if (p.tiles < (long long)DC_MIN_ROUNDS * sm_count()) return false;
-    // +-1 weights against pad bytes: the kernel with lowering warps does not take them (0.5 of the time)
-    if (g->w_enc == QNN_ENC_BIPOLAR && cv->KW * 3 % 16 != 0) return true;
+    // +-1 weights against pad bytes: the kernel with lowering warps does not take them (0.5 of the time; with a pool
+    // behind it the same, but up to 1.3 times as long where the epilogue counts 7 or 15 thresholds)
+    if (g->w_enc == QNN_ENC_BIPOLAR && cv->KW * 3 % 16 != 0 && (!pool || g->out_bits <= 2)) return true;
     if (!has_thr) return false;
     static const double bits[2][4] = {{0.173, 0.112, 0.091, 0.0}, {0.038, 0.007, 0.038, 0.0}};
     static const double parts[2][4] = {{0.074, -0.049, -0.084, 0.0}, {0.095, -0.114, -0.079, 0.0}};

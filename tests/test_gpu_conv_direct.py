@@ -70,9 +70,10 @@ def test_rows_read_in_place(qb, shape):
 
 @pytest.mark.parametrize("shape,fuses", [(s, s[2] != 131) for s in SHAPES if s[2] in (227, 255, 131)] + [
     ((47, 143, 143, 96, 11, 11, 4, 1, 8, 2, 2, 0), True),      # 34 x 34 map, 16 pooled rows, CTAs that span images
-    ((745, 19, 227, 32, 11, 11, 4, 1, 8, 4, 2, 0), True),      # three rows: one pooled row; 15 thresholds
+    ((745, 19, 227, 32, 11, 11, 4, 1, 8, 2, 2, 0), True),      # three rows: one pooled row
     ((93, 20, 50, 40, 3, 3, 1, 1, 8, 1, 2, 0), True),          # stride 1, 48 pixels a row; one threshold
-    ((107, 33, 101, 64, 5, 5, 2, 1, 8, 3, 2, 1), True),        # stride 2, 49 pixels a row; seven thresholds
+    ((107, 33, 101, 64, 5, 5, 2, 1, 8, 2, 2, 1), True),        # stride 2, 49 pixels a row
+    ((257, 17, 94, 33, 2, 5, 2, 8, 8, 3, 1, 0), True),         # seven thresholds
     ((48, 142, 55, 70, 2, 3, 1, 8, 8, 4, 1, 0), True),         # stride 1, 8-bit weights, 15 thresholds
     ((59, 83, 115, 70, 3, 7, 2, 8, 8, 4, 1, 1), True),
     ((71, 65, 126, 70, 2, 7, 2, 8, 8, 1, 1, 0), True),
