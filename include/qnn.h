@@ -289,7 +289,7 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
 /* The boxes of w x h output pixels of n images that the CTA-pair kernel cuts a large padded layer of stride 1 on
  * an 8-bit map into, so as to leave out filter taps that lie outside the image: their number; 0 where the layer
  * takes consecutive pixels or another kernel.  Host only. */
-int qnn_conv_boxes(const qnn_conv_desc *d, int *w, int *h, int *n);
+int qnn_conv_boxes(const qnn_conv_desc *d, int has_thresholds, int *w, int *h, int *n);
 
 /* Whether qnn_qconv runs this layer on the kernel that reads the rows of a three-channel map in place.  Host only. */
 int qnn_conv_in_place(const qnn_conv_desc *d, int has_thresholds);

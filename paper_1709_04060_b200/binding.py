@@ -100,7 +100,7 @@ _lib.qnn_im2col.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp]
 _lib.qnn_qconv.restype = _ci
 _lib.qnn_qconv.argtypes = [_P(qnn_conv_desc), _vp, _vp, _vp, _vp, _vp, _sz, _vp]
 _lib.qnn_conv_boxes.restype = _ci
-_lib.qnn_conv_boxes.argtypes = [_P(qnn_conv_desc), _P(_ci), _P(_ci), _P(_ci)]
+_lib.qnn_conv_boxes.argtypes = [_P(qnn_conv_desc), _ci, _P(_ci), _P(_ci), _P(_ci)]
 _lib.qnn_conv_in_place.restype = _ci
 _lib.qnn_conv_in_place.argtypes = [_P(qnn_conv_desc), _ci]
 _lib.qnn_conv_maxpool_fuses.restype = _ci
@@ -291,11 +291,11 @@ def qnn_qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream=None
     return _qconv(d, Wpacked, inp, thr, out, workspace, workspace_bytes, stream)
 
 
-def qnn_conv_boxes(d):
+def qnn_conv_boxes(d, has_thresholds: bool = True):
     """Boxes of output pixels that the CTA-pair kernel cuts this layer into: (number, width, height, images), or
     None where it takes consecutive pixels or another kernel takes the layer."""
     w, h, n = _ci(), _ci(), _ci()
-    boxes = _lib.qnn_conv_boxes(ctypes.byref(d), ctypes.byref(w), ctypes.byref(h), ctypes.byref(n))
+    boxes = _lib.qnn_conv_boxes(ctypes.byref(d), int(has_thresholds), ctypes.byref(w), ctypes.byref(h), ctypes.byref(n))
     return (boxes, w.value, h.value, n.value) if boxes else None
 
 

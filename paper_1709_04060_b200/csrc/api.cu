@@ -155,8 +155,7 @@ enum Route {
 static Route gemm_route(const qnn_gemm_desc *d, bool has_thr, int path) {
     if (d->w_fmt == QNN_FMT_FIELDS) {
         if (!getenv("QNN_FIELDS_KERNEL") && gemv_mma_takes(d, has_thr)) return ROUTE_FIELDS_MMA;
-        // one column: byte dot products on the CUDA cores; columns that do not fit an SM's shared
-        // memory: the tcgen05 form
+        // one column: byte dot products on the CUDA cores, where it fits their shared memory; else the tcgen05 form
         return gemv_fields_dp4a_fits(d) ? ROUTE_FIELDS_DP4A : ROUTE_FIELDS_TENSOR;
     }
     // 8-bit containers with a handful of columns and no path forced: the weights are streamed once
@@ -422,13 +421,13 @@ qnn_status qnn_qconv(const qnn_conv_desc *d, const void *Wpacked, const void *in
     return qnn_qgemm(&g, Wpacked, workspace, thr, out, nullptr, 0, stream);
 }
 
-int qnn_conv_boxes(const qnn_conv_desc *d, int *w, int *h, int *n) {
+int qnn_conv_boxes(const qnn_conv_desc *d, int has_thresholds, int *w, int *h, int *n) {
     qnn_gemm_desc g;
     int path = 0;
     if (check_conv_desc(d) != QNN_OK || !w || !h || !n) return 0;
     conv_to_gemm(d, &g);
-    if (check_gemm_desc(&g, false, &path) != QNN_OK || path != QNN_PATH_TCGEN05_I8) return 0;
-    return gemm_tc_conv_boxes(d, &g, w, h, n);
+    if (check_gemm_desc(&g, has_thresholds != 0, &path) != QNN_OK || path != QNN_PATH_TCGEN05_I8) return 0;
+    return gemm_tc_conv_boxes(d, &g, has_thresholds != 0, w, h, n);
 }
 
 int qnn_conv_in_place(const qnn_conv_desc *d, int has_thresholds) {

@@ -123,7 +123,7 @@ bool gemm_tc_uses_pair_kernel(const qnn_gemm_desc *d);
 qnn_status gemm_tc_conv_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
                                const int32_t *thr, void *out, bool any_size, cudaStream_t s);
 bool gemm_tc_conv_takes(const qnn_conv_desc *cv);       // what the tensor-map loader can lower
-int gemm_tc_conv_boxes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, int *w, int *h, int *n);
+int gemm_tc_conv_boxes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, int *w, int *h, int *n);
 qnn_status gemm_tc_lower_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *in,
                                 const int32_t *thr, void *out, cudaStream_t s);
 qnn_status gemm_tc_planes_launch(const qnn_conv_desc *cv, const qnn_gemm_desc *g, const void *W, const void *A,

@@ -1462,8 +1462,10 @@ static double boxes_us(const qnn_conv_desc *cv, const BoxPlan &b, int tiles_c, i
 // of 128 images, 9 % of the k-blocks of a padded 27 x 27 map (5 x 5 taps), 10 % of a 13 x 13 one (3 x 3).  But
 // boxes rarely fill their 128 rows, and tiles are dealt in whole rounds: a round more costs what many taps save.
 // So of the extents with the smallest rounds times mean tile, the one whose busiest pair of SMs is done first, and
-// that only if consecutive pixels take longer.
-static bool search_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan *plan) {
+// that only if consecutive pixels take longer.  Sums, and codes of three or four bits, are stored at a pace that an
+// epilogue of scattered pixels does not keep up with: there the saving has to be larger (1 x 1 boxes estimated at
+// 0.9 to 0.95: 16 x 16 x 80 -> 384, 5 x 5, batch 241, 3 bits 121 -> 129 us; 34 x 34 x 32 -> 256, 4 bits 85 -> 100).
+static bool search_boxes(const qnn_conv_desc *cv, bool light, int tiles_c, int pairs, BoxPlan *plan) {
     const int OH = qnn_conv_out_h(cv), OW = qnn_conv_out_w(cv), chunks = ceil_div(cv->C, TC_BK);
     auto rounds_us = [&](long long tiles_p, double kb) { return (double)((tiles_p * tiles_c + pairs - 1) / pairs) * pair_tile_us(kb); };
     auto met = [&](int out, int size, int in, int k) {
@@ -1475,15 +1477,15 @@ static bool search_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPla
         }
         return sum;
     };
-    constexpr double MARGIN = 0.98;
+    const double margin = light ? 0.98 : 0.88;
     constexpr int KEPT = 4;
     // single pixels leave out the most: too little in a large map (224 x 224, 3 x 3: 1.2 %)
     const double fewest = (double)met(OW, 1, cv->W, cv->KW) * met(OH, 1, cv->H, cv->KH) / ((double)OW * OH) * chunks;
-    if (pair_tile_us(fewest) >= MARGIN * pair_tile_us((double)cv->KH * cv->KW * chunks)) return false;
+    if (pair_tile_us(fewest) >= margin * pair_tile_us((double)cv->KH * cv->KW * chunks)) return false;
     const double raster = rounds_us(((long long)cv->B * OH * OW + 255) / 256, (double)cv->KH * cv->KW * chunks);
     BoxPlan best[KEPT];
     double us[KEPT];
-    for (int i = 0; i < KEPT; ++i) us[i] = MARGIN * raster;
+    for (int i = 0; i < KEPT; ++i) us[i] = margin * raster;
     // the smallest extents that make nw x nh boxes of an image
     for (int nw = ceil_div(OW, TC_BP), bw = 0; nw <= OW; ++nw) {
         if (ceil_div(OW, nw) == bw) continue;
@@ -1501,28 +1503,28 @@ static bool search_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPla
             us[i] = t; best[i] = {bw, bh, bn, boxes};
         }
     }
-    double least = MARGIN * raster;
-    for (int i = 0; i < KEPT && us[i] < MARGIN * raster; ++i) {
+    double least = margin * raster;
+    for (int i = 0; i < KEPT && us[i] < margin * raster; ++i) {
         // (of many rounds every pair gets about the same)
         const double t = best[i].boxes > 2 * BOX_TILES || pairs > BOX_PAIRS ? us[i] : boxes_us(cv, best[i], tiles_c, pairs);
         if (t < least) { least = t; *plan = best[i]; }
     }
-    return least < MARGIN * raster;
+    return least < margin * raster;
 }
 
 // The same, searched once per shape and thread (the search takes 5 to 15 us for maps of 13 to 56 pixels, up to 50
-// for larger ones; a call of the library some 2).
-static bool conv_boxes(const qnn_conv_desc *cv, int tiles_c, int pairs, BoxPlan *plan) {
+// for larger ones; a call of the library some 2).  light: codes of one or two bits.
+static bool conv_boxes(const qnn_conv_desc *cv, bool light, int tiles_c, int pairs, BoxPlan *plan) {
     if (cv->stride != 1 || cv->pad == 0) return false;
-    struct Entry { int key[9]; bool found; BoxPlan plan; };
+    struct Entry { int key[10]; bool found; BoxPlan plan; };
     constexpr int ENTRIES = 32;                               // a shape displaces another of the same slot
     static thread_local Entry table[ENTRIES] = {};
-    const int key[9] = {cv->B, cv->H, cv->W, cv->KH, cv->KW, cv->pad, ceil_div(cv->C, TC_BK), tiles_c, pairs};
+    const int key[10] = {cv->B, cv->H, cv->W, cv->KH, cv->KW, cv->pad, ceil_div(cv->C, TC_BK), tiles_c, pairs, light};
     unsigned slot = 0;
     for (int k : key) slot = slot * 31 + (unsigned)k;
     Entry &e = table[slot % ENTRIES];
     if (memcmp(e.key, key, sizeof(key)) != 0) {
-        e.found = search_boxes(cv, tiles_c, pairs, &e.plan);
+        e.found = search_boxes(cv, light, tiles_c, pairs, &e.plan);
         memcpy(e.key, key, sizeof(key));
     }
     *plan = e.plan;
@@ -1736,7 +1738,7 @@ static qnn_status tc_launch(const qnn_gemm_desc *d, const qnn_conv_desc *cv, con
     int columns = d->N;                   // rows of the activation operand's tiles: those of boxes may not be full
     if (cv && pair) {
         BoxPlan b;
-        if (conv_boxes(cv, ceil_div(d->M, T2_BN), sms / 2, &b)) {
+        if (conv_boxes(cv, thr && d->out_bits <= 2, ceil_div(d->M, T2_BN), sms / 2, &b)) {
             p.bx_w = b.w; p.bx_h = b.h; p.bx_n = b.n;
             p.nb_w = ceil_div(qnn_conv_out_w(cv), p.bx_w); p.nb_h = ceil_div(qnn_conv_out_h(cv), p.bx_h); p.nb_n = ceil_div(cv->B, p.bx_n);
             columns = (int)b.boxes * TC_BP;
@@ -1831,9 +1833,10 @@ bool gemm_tc_conv_takes(const qnn_conv_desc *cv) {
     if (cv->fmt != QNN_FMT_INT8 || (cv->C % 16) != 0 || (pitch % 16) != 0) return false;
     return cv->KH <= 255 && cv->KW <= 255 && cv->stride <= 8;
 }
-int gemm_tc_conv_boxes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, int *w, int *h, int *n) {
+int gemm_tc_conv_boxes(const qnn_conv_desc *cv, const qnn_gemm_desc *g, bool has_thr, int *w, int *h, int *n) {
     BoxPlan b;
-    if (!gemm_tc_conv_takes(cv) || !choose_pair_kernel(g, sm_count()) || !conv_boxes(cv, ceil_div(g->M, T2_BN), sm_count() / 2, &b)) return 0;
+    if (!gemm_tc_conv_takes(cv) || !choose_pair_kernel(g, sm_count())) return 0;
+    if (!conv_boxes(cv, has_thr && g->out_bits <= 2, ceil_div(g->M, T2_BN), sm_count() / 2, &b)) return 0;
     *w = b.w; *h = b.h; *n = b.n;
     return (int)b.boxes;
 }

@@ -56,6 +56,14 @@ def test_first_layers_fuse_with_their_pool_where_tiles_are_full(qb, layer, fuses
     assert qb.qnn_conv_maxpool_fuses(first_layer(qb, *layer), 3, 2) == fuses
 
 
+def test_layers_of_plus_minus_one_fuse_where_few_thresholds_are_counted(qb):
+    """36 x 47 -> 16, 3 x 3, batch 356, seven thresholds: 81 us apart, 106 in one kernel."""
+    for layer in ((356, 43, 47, 16, 3, 1, 3), (131, 130, 130, 8, 5, 4, 3)):
+        assert not qb.qnn_conv_maxpool_fuses(first_layer(qb, *layer, w_enc=2), 3, 2)
+        assert qb.qnn_conv_maxpool_fuses(first_layer(qb, *layer[:6], 2, w_enc=2), 3, 2)
+        assert qb.qnn_conv_in_place(first_layer(qb, *layer, w_enc=2))
+
+
 def busiest_pair(cv, boxes):
     """k-blocks (one channel chunk) of the SM pair with the most, of 74: tiles of two boxes, or of 256
     consecutive pixels that meet every tap, dealt in turn."""
@@ -111,6 +119,16 @@ def test_boxes_never_keep_a_pair_of_sms_busier(qb):
             taken += 1
             assert busiest_pair(cv, plan) <= 0.98 * busiest_pair(cv, None), (B, H, W, OC, k, plan)
     assert taken > 100
+
+
+def test_boxes_save_more_where_the_epilogue_is_longer(qb):
+    """Sums and codes of three or four bits: 34 x 34 x 32 -> 256, 5 x 5, 85 -> 100 us with single pixels."""
+    cv = conv(qb, 118, 34, 34, 32, 256, 5, 5, 1, 2)
+    assert qb.qnn_conv_boxes(cv) is not None and qb.qnn_conv_boxes(cv, False) is None
+    cv.out_bits = 4
+    assert qb.qnn_conv_boxes(cv) is None
+    deep = conv(qb, 127, 10, 10, 32, 600, 7, 7, 1, 3)           # three taps of ten: 0.71 of the time
+    assert qb.qnn_conv_boxes(deep, False) is not None
 
 
 def test_only_padded_layers_of_stride_one_take_boxes(qb):

@@ -36,7 +36,7 @@ def test_box_tiles(qb, monkeypatch, shape, boxes):  # noqa: F811
     want = (want_raw[:, :, None] >= case.thr[None]).sum(2)
     for out_fmt, raw in ((INT8, False), (BITPLANES, False), (INT8, True)):
         d = conv_desc(qb, case, INT8, out_fmt, pitch)
-        assert qb.qnn_conv_boxes(d) == boxes
+        assert qb.qnn_conv_boxes(d, not raw) == boxes
         nb = qb.qnn_conv_out_bytes(d, not raw)
         out = torch.full((nb + 64,), 0xEE, dtype=torch.uint8, device="cuda")
         ws = torch.zeros(qb.qnn_conv_workspace_bytes(d), dtype=torch.uint8, device="cuda")
