@@ -36,8 +36,8 @@
 //                robin; group 0 then runs the epilogue
 //   warp 10      TMA loads of the slice's activation k-blocks (16 rows x 128 bytes each, all
 //                resident)
-// The library takes this kernel where the columns do not fit the shared memory of gemv_mma.cu's CTA
-// (16 columns: depths beyond 9 700 to 12 200, by field width), which is the faster one otherwise.
+// The library takes this kernel where the columns are deeper than gemv_mma.cu takes (209 KB of column
+// bytes: 16 columns of 13 376, 8 of 26 752), which is the faster one otherwise.
 // Every wait is bounded; on expiry the CTA records QNN_ERR_DEVICE_TIMEOUT and drains.
 #include <cuda.h>
 

@@ -504,11 +504,12 @@ static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
     return true;
 }
 
-// What this kernel is taken for: deeper products with several columns, whose activations would be loaded
-// in many passes, are left to the others.
+// What this kernel is taken for.  Deep products are walked in passes, up to the 209 KB of column bytes (elements, times
+// columns) that fitted an SM's shared memory when the columns were staged there.  Past it the kernels that take over
+// need 2 to 8 times as long (5 to 8 columns: planes 7.5; 9 to 16: planes 3.8, fields 2.2).
 static bool mv_fits(const qnn_gemm_desc *d) {
     if (d->N > (d->w_fmt == QNN_FMT_INT8 ? 8 : MV_COLS) || (d->w_fmt == QNN_FMT_BITPLANES && (d->w_bits > 4 || d->a_bits > 4))) return false;
-    return (long long)d->N * round_up(d->K, 32) <= 192 * 1024;
+    return (long long)d->N * round_up(d->K, 32) <= 209 * 1024;
 }
 
 // Sums, and 8-bit codes without pad bytes: whether this kernel beats the one that counts bits
