@@ -504,39 +504,35 @@ static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
     return true;
 }
 
-// What this kernel is taken for.  Deep products are walked in passes, up to the 209 KB of column bytes (elements, times
-// columns) that fitted an SM's shared memory when the columns were staged there.  Past it the kernels that take over
-// need 2 to 8 times as long (5 to 8 columns: planes 7.5; 9 to 16: planes 3.8, fields 2.2).
-static bool mv_fits(const qnn_gemm_desc *d) {
-    if (d->N > (d->w_fmt == QNN_FMT_INT8 ? 8 : MV_COLS) || (d->w_fmt == QNN_FMT_BITPLANES && (d->w_bits > 4 || d->a_bits > 4))) return false;
-    return (long long)d->N * round_up(d->K, 32) <= 209 * 1024;
-}
-
-// Sums, and 8-bit codes without pad bytes: whether this kernel beats the one that counts bits
-// (gemv_planes.cu), by an estimate of both.  That one costs a load latency per staged column and plane, one
-// per depth step of a lane, its CTAs and its population counts; this one its fill and drain, the columns it
-// widens, the rounds of tiles and the weights.  The terms' shares are fitted to random problems; the factor
-// is the point below which counting is the better choice: of 860 problems with 2 to 16 columns (up to 12000
-// x 9216, every width and encoding, replayed as a graph) the choice costs 1.0 % of the faster one's time (at
-// 0.96, as for one column, 10.5 %; always this kernel 0.6 %, but up to 1.4 times as long for little work, call
-// after call); 960 x 64, N = 5, W2A1: 2.7 us there, 2.9 here.
-static bool mv_planes_faster(const qnn_gemm_desc *d) {
-    const int kw = ceil_div(d->K, 32), cols = d->N < 4 ? d->N : 4, pairs = d->w_bits * d->a_bits;
+// Bit planes: whether this kernel beats the one that counts bits (gemv_planes.cu), by an estimate of both in
+// microseconds.  That one costs a load latency per staged column and plane, one per depth step of a lane, its CTAs
+// and its population counts; this one its fill and drain, the products of the warp with the most, the weights, the
+// columns it widens and the partial sums it exchanges.  The terms' shares are a non-negative least-squares fit to
+// 7623 random problems timed with both kernels (half of them with one column; up to 12000 x 9216, every width,
+// encoding and output), replayed as a graph; call after call this kernel takes a little longer, hence the factor.
+// Twelve plane pairs and more of 2^22 weights are never counted: the estimate is up to a fifth off there (8192 x
+// 8192 W4A4, one column: 14.6 us counted, 11.5 here).  The choice costs 1.6 % (graph) and 1.4 % (calls) of the
+// faster one's time on average; always this kernel 5.1 % and 6.1 %, always counting 72 % and 53 %.
+static bool mv_planes_faster(const qnn_gemm_desc *d, bool has_thr) {
+    if (d->w_bits * d->a_bits >= 12 && (long long)d->M * d->K >= (1ll << 22)) return true;
+    MvPlan pl;
+    if (!mv_plan(d, has_thr, &pl)) return false;
+    const int kw = ceil_div(d->K, 32), cols = d->N < 4 ? d->N : 4, pairs = d->w_bits * d->a_bits, nt = d->N > 8 ? 2 : 1;
     const double ctas = (double)ceil_div(d->M, 8) * ceil_div(d->N, 4), words = (double)d->M * kw;
-    const double staged = d->w_enc == QNN_ENC_BIPOLAR && d->a_enc != QNN_ENC_BIPOLAR ? 0.48 : 0.32;   // with column sums
-    const double counted = 0.89 + staged * d->a_bits * cols * ceil_div(kw, 256) +
-                           (kw % 4 == 0 ? 0.83 * ceil_div(kw, 128) : 0.23 * ceil_div(kw, 32)) +
-                           0.011 * pairs * cols * ceil_div(kw, 32) + 2.3e-7 * words * pairs * d->N + 2.44e-3 * ctas;
-    const double here = (d->w_bits <= 2 ? 4.8 : 4.0) + (d->N > 8 ? 0.25 : 0.0) + 1.9e-3 * d->N * kw +
-                        1.5 * ((ceil_div(d->M, 32) - 1) / sm_count()) + 0.8e-6 * words * d->w_bits;
-    return counted > (d->N >= 2 ? 0.65 : 0.96) * here;
+    const double staged = d->w_enc == QNN_ENC_BIPOLAR && d->a_enc != QNN_ENC_BIPOLAR ? 0.43 : 0.285;   // with column sums
+    const double counted = 1.42 + staged * d->a_bits * cols * ceil_div(kw, 256) +
+                           (kw % 4 == 0 ? 0.616 * ceil_div(kw, 128) : 0.183 * ceil_div(kw, 32)) +
+                           0.0113 * pairs * cols * ceil_div(kw, 32) + 2.38e-7 * words * pairs * d->N + (1.56e-3 + 2.4e-4 * cols) * ctas;
+    const double waves = (double)ceil_div(ceil_div(pl.groups, pl.per), sm_count());
+    const double rounds = waves * pl.passes * ceil_div(ceil_div(pl.per, 3 - nt), pl.rsplit) * pl.u;
+    const double here = 2.60 + rounds * (0.172 + 0.0142 * pl.v * d->w_bits) + 1.04e-6 * words * d->w_bits +
+                        1.74e-4 * d->N * kw * d->a_bits + (nt == 2 ? 0.2 : 0.0) + 1.3e-3 * pl.dsplit * pl.per * d->N;
+    return counted > 1.1 * here;
 }
 
 // Where this kernel is the faster one of those that take the format (8192 x 8192, us, the other -> this):
 //   fields  two columns on: W2A2 N = 2 10.2 -> 7.2, N = 4 13.0 -> 7.3, N = 16 15.4 -> 9.5 (N = 1 6.0 -> 7.1)
-//   planes  two columns on, or one where there are twelve or more plane pairs to count (8192 x 8192, weights
-//           in L2: W2A2 N = 4 12.9 -> 7.2, N = 16 38 -> 9.1; W4A4 N = 1 14.6 -> 11.5), but for small problems:
-//           mv_planes_faster
+//   planes  mv_planes_faster (W2A2 N = 4 12.9 -> 7.2, N = 16 38 -> 9.1; W4A4 N = 1 14.6 -> 11.5)
 //   bytes   three columns on from 2^23 weights, four from 3 x 2^20: N = 4 26 -> 11.6, N = 8 35 -> 12.1 (N = 2
 //           4805 x 5120 5.4 -> 6.2); 11841 x 512 N = 7 6.1 -> 2.9, 416 x 7424 N = 6 6.8 -> 4.0.  Below, where
 //           either takes 2 to 3 us, a call of the host takes longer than both, and of this one longest
@@ -545,17 +541,19 @@ static bool mv_planes_faster(const qnn_gemm_desc *d) {
 //           they set bit by bit; pad bytes that they do not write): the host's second launch decides, call
 //           after call (fields N = 1 10.2 -> 8.1, bytes 4096 x 9216 N = 1 12.8 -> 11.4); bytes only below 2^26
 //           elements (8192 x 8192: 16.1 there, 17 here)
-//   planes whose output is bit planes or padded: two columns on (240 random problems with two columns: 0.76 of
-//           the time on average, more columns 0.51); one column below 2^24 weights (210 problems: 0.95,
-//           between 0.4 and 1.6)
+// Deep products are walked in passes, up to the 209 KB of column bytes (elements, times columns) that fitted an SM's
+// shared memory when the columns were staged there.  Past it the kernels that take over need 2 to 8 times as long
+// (5 to 8 columns: planes 7.5; 9 to 16: planes 3.8, fields 2.2).
 bool gemv_mma_takes(const qnn_gemm_desc *d, bool has_thr) {
-    if (!mv_fits(d)) return false;
+    if (d->N > (d->w_fmt == QNN_FMT_INT8 ? 8 : MV_COLS)) return false;
+    const long long size = (long long)d->M * d->K, column_bytes = (long long)d->N * round_up(d->K, 32);
+    if (column_bytes > 209 * 1024) return false;
+    if (d->w_fmt == QNN_FMT_BITPLANES) {
+        if (d->w_bits > 4 || d->a_bits > 4) return false;
+        return mv_planes_faster(d, has_thr);
+    }
     const bool padded = has_thr && (d->out_fmt == QNN_FMT_BITPLANES || (d->w_fmt != QNN_FMT_FIELDS && d->M % 16 != 0));
     if (d->w_fmt == QNN_FMT_FIELDS) return d->N >= 2 || padded;
-    const long long size = (long long)d->M * d->K;
-    if (d->w_fmt == QNN_FMT_BITPLANES)
-        return padded ? d->N >= 2 || d->w_bits * d->a_bits >= 12 || size < (1ll << 24)
-                      : (d->N >= 2 || d->w_bits * d->a_bits >= 12) && mv_planes_faster(d);
     return (d->N >= 3 && size >= (1ll << 23)) || (d->N >= 4 && size >= (3ll << 20)) || (padded && size < (1ll << 26));
 }
 

@@ -9,9 +9,9 @@
 // One warp per weight row: lanes stride over the depth words, partial sums meet in
 // a shuffle reduction, then lane n counts the thresholds of column n (Section 2.1.1).
 // Columns are handled four at a time (blockIdx.y); more than four columns re-read
-// the weights from L2.  The library takes this kernel for one column and fewer than twelve plane pairs,
-// for small products where little is counted (mv_planes_faster in gemv_mma.cu), on the forced
-// bit-serial path, and where plane pairs are left out; else gemv_mma.cu.
+// the weights from L2.  The library takes this kernel where little is counted (few plane pairs, mostly
+// one column: mv_planes_faster in gemv_mma.cu), on the forced bit-serial path, and where plane pairs
+// are left out; else gemv_mma.cu.
 #include "common.cuh"
 
 namespace qnn {

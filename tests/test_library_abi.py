@@ -241,22 +241,23 @@ def test_kernel_names_on_both_sides_of_every_rule(qb):
     assert k(8200, 1, 8192, I8, out=PL) == "gemv_i8_kernel"
     assert k(4096, 9, 4096, I8) == tc
     assert k(4096, 4096, 4096, I8) == "qgemm_tc2_kernel"
-    # planes, few columns: two columns on; one with twelve plane pairs, or cleared below 2^24 weights
+    # planes, few columns: the estimate of both kernels, twelve plane pairs and more of 2^22 weights aside; neither
+    # needs a clearing launch, so pad bytes and the output's format do not matter
     assert k(8192, 1, 8192, PL) == popc
     assert k(8192, 2, 8192, PL) == mma
     assert k(8192, 1, 8192, PL, w=3, a=4) == mma
+    assert k(8192, 1, 8192, PL, w=4, a=4) == mma
     assert k(8192, 1, 8192, PL, w=3, a=3) == popc
-    # ... but not where little is counted: few activation planes, few rows, a shallow depth
-    assert k(960, 5, 64, PL, w=2, a=1) == popc
-    assert k(961, 5, 64, PL, w=2, a=1) == mma                 # pad bytes to clear
-    assert k(960, 5, 64, PL, w=2, a=1, out=PL) == mma         # bit-plane output
-    assert k(961, 5, 64, PL, w=2, a=1, thr=False) == popc
     assert k(12000, 16, 64, PL, w=2, a=1) == mma
     assert k(960, 5, 64, PL, w=2, a=4) == mma
     assert k(5, 12, 647, PL, w=1, a=1, w_enc=B, thr=False) == popc
-    assert k(352, 1, 512, PL, w=4, a=4) == popc
-    assert k(4095, 1, 4096, PL) == mma
-    assert k(4096, 1, 4096, PL, out=PL) == popc
+    for out, thr in ((I8, True), (PL, True), (I8, False)):
+        assert k(4095, 1, 4096, PL, out=out, thr=thr) == popc
+        assert k(4096, 1, 4096, PL, out=out, thr=thr) == popc
+        assert k(101, 16, 64, PL, w=1, a=1, out=out, thr=thr) == popc
+        assert k(961, 5, 64, PL, w=2, a=1, out=out, thr=thr) == mma
+        assert k(1000, 1, 4096, PL, w=4, a=4, out=out, thr=thr) == mma
+        assert k(352, 1, 512, PL, w=2, a=2, out=out, thr=thr) == popc
     assert k(8192, 2, 8192, PL, path=qb.QNN_PATH_BITSERIAL) == popc
     assert k(8192, 2, 8192, PL, skip=1) == popc
     # planes, tiled: sixteen plane pairs up to 2^30, a single pair between 2^24 and 2^27, the forced path
