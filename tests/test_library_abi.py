@@ -229,7 +229,7 @@ def test_kernel_names_on_both_sides_of_every_rule(qb):
     assert k(8192, 16, 9216, FL) == mma
     assert k(8192, 16, 13376, FL) == mma                      # 209 KB of column bytes
     assert k(8192, 16, 13377, FL) == "gemv_fields_kernel"
-    assert k(8192, 8, 26000, FL, w=4, a=4) == mma
+    assert k(8192, 8, 25000, FL, w=4, a=4) == mma
     assert k(8192, 8, 26000, PL) == mma
     assert k(8192, 16, 16384, FL) == "gemv_fields_kernel"
     # bytes: three columns on from 2^23 weights; fewer where pad bytes need clearing, below 2^26 weights
