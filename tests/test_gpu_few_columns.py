@@ -29,6 +29,9 @@ def qb():
     (2500, 9, 1000), (321, 16, 9120),          # two blocks of columns; passes
     (4100, 5, 33), (1200, 3, 2080),            # shallow: several groups at a time
     (19000, 2, 512),                           # more groups a CTA than warps
+    (4100, 4, 4097), (1200, 7, 2080),          # ... of few plane pairs too
+    (4100, 8, 1025), (3000, 5, 9729),          # bytes as sums; three quarters of the steps of a warp
+    (1000, 16, 11000), (500, 6, 20000),        # deeper than 16 warps hold
 ])
 def test_plan_edges(qb, fmt, w, a, w_enc, a_enc, M, N, K):
     if fmt == INT8 and N > 8:
@@ -42,6 +45,11 @@ def test_plan_edges(qb, fmt, w, a, w_enc, a_enc, M, N, K):
     codes = (sums[:, :, None] >= case.thr[None]).sum(2)
     for out_fmt, raw in ((INT8, False), (BITPLANES, False), (INT8, True)):
         d = qb.qnn_gemm_desc(M, N, K, w, a, 3, w_enc, a_enc, fmt, a_fmt, out_fmt, 0, 0)
+        name = qb.qnn_qgemm_kernel_name(d, not raw)
+        if fmt == FIELDS or (fmt == BITPLANES and (a > 1 or N > 3)):
+            assert name == "gemv_mma_kernel"
+        elif fmt == INT8 and K <= 12288:                   # what the byte dot products stage
+            assert (name == "gemv_mma_kernel") == ((not raw and (out_fmt == BITPLANES or M % 16 != 0)) or (N >= 4 and M * K >= 3 << 20))
         nb = qb.qnn_gemm_out_bytes(d, not raw)
         out = torch.full((nb + 64,), 0xEE, dtype=torch.uint8, device="cuda")
         qb.check(qb.qnn_qgemm(d, Wp, Ap, None if raw else thr, out))
