@@ -135,6 +135,9 @@ __device__ __forceinline__ void mv_expand(const uint32_t *w, uint32_t (&o)[4][2]
         for (int i = 0; i < 2; ++i) o[k][i] = x[2 * (k >> 1) + i] & (k & 1 ? 0xF0F0F0F0u : 0x0F0F0F0Fu);
 }
 
+// Steps of a buffer: the largest power of two up to `most` that divides the steps of a product.
+__host__ __device__ constexpr int mv_buffer_steps(int most, int steps) { return most > steps || steps % most != 0 ? mv_buffer_steps(most / 2, steps) : most; }
+
 // Activation registers of a product: for each half of its depth, the column g and (NT == 2) g + 8.
 #define MV_AT(HALF_, BLOCK_) ((HALF_) * NT + (BLOCK_))
 // Ints between the rows of a group's partial sums: two blocks of columns are stored column by column.
@@ -156,8 +159,8 @@ gemv_mma_kernel(const MvParams p) {
     // (of few: a launch that runs a product or two per warp waits for every line of code it fetches, also of
     // the products it skips)
     constexpr int FIT = 16 / (G * PL * V), STEPS = FIT >= 8 ? 8 : (FIT >= 4 ? 4 : (FIT >= 2 ? 2 : 1)), MOST = AP >= 8 ? 2 : 4;
-    constexpr int UB = STEPS < U ? STEPS : U, Q = STEPS / UB < MOST ? STEPS / UB : MOST, NB = U / UB;
-    constexpr int TURN = NB == 1 ? 2 : NB;                         // buffers per turn of the loop (even)
+    constexpr int UB = mv_buffer_steps(STEPS, U), Q = U > UB ? 1 : (STEPS / UB < MOST ? STEPS / UB : MOST), NB = U / UB;
+    constexpr int TURN = NB == 1 ? 2 : (NB % 2 ? 2 * NB : NB);     // buffers per turn of the loop (even)
     constexpr int FIELD = SRC == MV_PLANES ? mv_field<B> : (SRC == MV_FIELDS ? B : 0);
     extern __shared__ __align__(16) uint8_t mv_smem[];
     int *part = reinterpret_cast<int *>(mv_smem);                  // [group][depth slice][8 rows][PITCH: 8 NT columns]
@@ -409,12 +412,12 @@ gemv_mma_kernel(const MvParams p) {
                 }
             }
         };
-        for (int gi = 0; G * (r0 + gi * p.rsplit) < ng; gi += NB == 1 ? 2 * Q : 1) {
+        for (int gi = 0; G * (r0 + gi * p.rsplit) < ng; gi += NB == 1 ? 2 * Q : TURN / NB) {
 #pragma unroll
             for (int i = 0; i < TURN; ++i) {
-                multiply(w[i & 1], NB == 1 ? gi + i * Q : gi, NB == 1 ? 0 : i);
+                multiply(w[i & 1], NB == 1 ? gi + i * Q : gi + i / NB, NB == 1 ? 0 : i % NB);
                 if (NB == 1) load(w[i & 1], gi + (i + 2) * Q, 0);
-                else load(w[i & 1], i + 2 < NB ? gi : gi + 1, (i + 2) % NB);
+                else load(w[i & 1], gi + (i + 2) / NB, (i + 2) % NB);
             }
         }
     }
@@ -455,10 +458,12 @@ gemv_mma_kernel(const MvParams p) {
 struct MvPlan { int src, b, v, units, u, dsplit, rsplit, passes, groups, per, threads; size_t smem; };
 
 // Activation registers per lane and step, and the steps of a warp per product that kernels are built for:
-// as many as 64 such registers allow, and fewer for shallow depths and few rows.
+// as many as 64 such registers allow, three quarters of that (depths that leave warps idle otherwise), and fewer for
+// shallow depths and few rows.
 static int mv_act_regs(const MvPlan &pl, int nt) { return nt * (pl.src == MV_PLANES ? 8 * pl.v : 4 * (8 / pl.b)); }
 constexpr int mv_steps_least(int regs) { return regs >= 16 ? 1 : (regs == 8 ? 2 : 4); }
 constexpr int mv_steps_most(int regs) { return 64 / regs; }
+constexpr int mv_steps_mid(int regs) { return mv_steps_most(regs) >= 4 ? mv_steps_most(regs) * 3 / 4 : mv_steps_most(regs); }
 
 static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
     if (d->N > MV_COLS) return false;
@@ -487,7 +492,10 @@ static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
     // 4101 x 9063 N = 11: 11.1 -> 10.2; three of one -> two of two, W2 6154 x 8805 N = 16: 10.8 -> 12.5)
     const int steps = ceil_div(pl->units, 4), regs = mv_act_regs(*pl, nt), most = mv_steps_most(regs);
     long long best = 0;
-    for (int u = mv_steps_least(regs); u <= most; u = u < most ? most : most + 1) {
+    // (three quarters of the steps only where a row's depth takes more than half of the warps: 3597 x 9725 bytes, N = 5,
+    // ten of sixteen 10.1 -> 7.6; where the rows are shared between warps the other two are the better ones)
+    for (int u : {mv_steps_least(regs), mv_steps_mid(regs), most}) {
+        if (u == mv_steps_mid(regs) && u < most && 2 * ceil_div(steps, most) <= MV_WARPS) continue;
         const int passes = ceil_div(steps, MV_WARPS * u), ds = ceil_div(steps, u * passes), rs = MV_WARPS / ds;
         const int fit = (int)((MV_SMEM_MAX - 1024) / (ds * 32 * mv_part_pitch(nt) + 8 * 15 * 4));
         const int waves = ceil_div(pl->groups, sms * fit), per = ceil_div(pl->groups, sms * waves);
@@ -572,8 +580,9 @@ static qnn_status mv_launch(const MvParams &p, const MvPlan &pl, cudaStream_t s)
 
 template <int SRC, int B, int V, int NT, bool W_SIGNED, bool A_SIGNED>
 static qnn_status mv_launch_u(const MvParams &p, const MvPlan &pl, cudaStream_t s) {
-    constexpr int REGS = NT * (SRC == MV_PLANES ? 8 * V : 4 * (8 / B)), LEAST = mv_steps_least(REGS), MOST = mv_steps_most(REGS);
+    constexpr int REGS = NT * (SRC == MV_PLANES ? 8 * V : 4 * (8 / B)), LEAST = mv_steps_least(REGS), MID = mv_steps_mid(REGS), MOST = mv_steps_most(REGS);
     if (pl.u == LEAST) return mv_launch<SRC, B, V, NT, LEAST, W_SIGNED, A_SIGNED>(p, pl, s);
+    if (pl.u == MID) return mv_launch<SRC, B, V, NT, MID, W_SIGNED, A_SIGNED>(p, pl, s);
     return mv_launch<SRC, B, V, NT, MOST, W_SIGNED, A_SIGNED>(p, pl, s);
 }
 
