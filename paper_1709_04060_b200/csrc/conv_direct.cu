@@ -24,7 +24,8 @@
 // table's latency takes 89 cycles an MMA); warp 1 asks for the image rows of later steps by bulk copies (they
 // are contiguous); warps 2-5 turn them into ring slots; the next ones lay out the weights, then run the
 // epilogue, one 32 x 32 part of a tile per warp; with the pool in the kernel, four more take the maxima
-// from the codes of the last three tiles, which the epilogue leaves in shared memory.
+// from the codes of the last three tiles, which the epilogue leaves in shared memory.  Up to 832 threads leave 72 or 80 registers
+// each: with two output bits 4 to 48 bytes are spilled, else none.
 #include <math.h>
 
 #include "tc_epilogue.cuh"

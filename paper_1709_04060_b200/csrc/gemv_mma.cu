@@ -31,6 +31,9 @@
 // reads whole (131 KB each, 19 MB from L2).  8192 x 8192, us, activations staged through shared memory by the
 // whole CTA -> here: planes W2A2 N = 2 8.4 -> 7.0, 4 9.1 -> 7.2, 16 14.8 -> 9.1, W4A4 N = 1 13.5 -> 11.5;
 // fields W2 N = 2 7.8 -> 7.2, 16 12.3 -> 10.1, W4 N = 16 13.1 -> 11.9; bytes 1000 x 4096 N = 7 5.2 -> 3.3.
+//
+// 512 threads leave 128 registers a thread; of the 90 kernels the 29 with all 64 activation registers spill, 4 to 104
+// bytes each (planes W1 word by word most, bytes 52, W2 fields 40 to 60, W4 fields 4 to 20).
 #include "common.cuh"
 #include "planes.cuh"
 
