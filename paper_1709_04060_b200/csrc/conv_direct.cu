@@ -102,7 +102,7 @@ __device__ __forceinline__ void dc_words(const uint8_t *base, long long at, long
     if (a + 16 <= total) {
         const uint32_t *q = reinterpret_cast<const uint32_t *>(base + a);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = q[i];
+        for (int i = 0; i < 4; ++i) x[i] = ld_global(q + i);
     } else {
         const uint4 v = dc_words_end(base, a, total);
         x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;

@@ -269,7 +269,7 @@ gemv_fields_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
             // thresholds of this thread's row: in registers long before they are needed
 #pragma unroll
             for (int i = 0; i < 15; ++i)
-                t[i] = (i < n_thr && m < p.M && r < p.R) ? p.thr[(size_t)m * n_thr + i] : 0x7fffffff;
+                t[i] = (i < n_thr && m < p.M && r < p.R) ? ld_global(p.thr + (size_t)m * n_thr + i) : 0x7fffffff;
         }
         // Lane R of tensor memory (the first one past the block's rows) carries a row of ones: its
         // accumulators collect sum_k a[n][k], the column sums that the weight encoding's offset

@@ -171,7 +171,7 @@ gemv_fields_dp4a_kernel(const FdParams p) {
                     reinterpret_cast<int32_t *>(p.out)[(size_t)n * p.M + mr] = a;
                 } else {
                     int code = 0;
-                    for (int q = 0; q < n_thr; ++q) code += (a >= p.thr[(size_t)mr * n_thr + q]) ? 1 : 0;
+                    for (int q = 0; q < n_thr; ++q) code += (a >= ld_global(p.thr + (size_t)mr * n_thr + q)) ? 1 : 0;
                     if (p.out_fmt == QNN_FMT_INT8) {
                         uint8_t *o = reinterpret_cast<uint8_t *>(p.out) + (size_t)n * p.ld_out;
                         o[mr] = (uint8_t)code;

@@ -109,7 +109,7 @@ gemv_i8_kernel(const G8Params p) {
                 reinterpret_cast<int32_t *>(p.out)[(size_t)n * p.M + m] = a;
             } else {
                 int code = 0;
-                for (int q = 0; q < n_thr; ++q) code += (a >= p.thr[(size_t)m * n_thr + q]) ? 1 : 0;
+                for (int q = 0; q < n_thr; ++q) code += (a >= ld_global(p.thr + (size_t)m * n_thr + q)) ? 1 : 0;
                 if (p.out_fmt == QNN_FMT_INT8) {
                     reinterpret_cast<uint8_t *>(p.out)[(size_t)n * p.ld_out + m] = (uint8_t)code;
                 } else {

@@ -169,7 +169,7 @@ gemv_planes_kernel(const GvParams p) {
             } else {
                 int code = 0;
                 if (row_ok)
-                    for (int q = 0; q < n_thr; ++q) code += (a >= p.thr[(size_t)m * n_thr + q]) ? 1 : 0;
+                    for (int q = 0; q < n_thr; ++q) code += (a >= ld_global(p.thr + (size_t)m * n_thr + q)) ? 1 : 0;
                 if (p.out_fmt == QNN_FMT_INT8) {
                     if (m < p.ld_out) reinterpret_cast<uint8_t *>(p.out)[(size_t)n * p.ld_out + m] = (uint8_t)code;
                 } else {

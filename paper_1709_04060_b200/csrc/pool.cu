@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256) maxpool_u8_kernel(const PoolParams p) {
             const uint4 *row = in + (((size_t)b * p.H + oh * p.stride + i) * p.W + ow * p.stride) * cu + u;
 #pragma unroll
             for (int j = 0; j < k; ++j) {
-                const uint4 v = row[(size_t)j * cu];
+                const uint4 v = ld_global(row + (size_t)j * cu);
                 best.x = __vmaxu4(best.x, v.x); best.y = __vmaxu4(best.y, v.y);
                 best.z = __vmaxu4(best.z, v.z); best.w = __vmaxu4(best.w, v.w);
             }

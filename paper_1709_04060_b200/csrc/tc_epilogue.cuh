@@ -76,7 +76,7 @@ __device__ __forceinline__ void stage_thresholds(const Params &p, int *thr_s, in
         for (int q = 0; q < NT; ++q) t[q] = 0x7fffffff;
         if (m < p.M) {
 #pragma unroll
-            for (int q = 0; q < N_THR; ++q) t[q] = p.thr[(size_t)m * N_THR + q];
+            for (int q = 0; q < N_THR; ++q) t[q] = ld_global(p.thr + (size_t)m * N_THR + q);
         }
         if (SORT) {
             // odd-even transposition sort; the pads are the largest value and stay last
