@@ -219,10 +219,12 @@ static bool gv_dispatch(int wb, int ab, const GvParams &p, dim3 grid, size_t sme
     return false;
 }
 
-// N <= 16 and the activation columns of one CTA fit the default 48 KB of shared memory.
+// N <= 16 and the activation columns of one CTA fit the default 48 KB of shared memory beside the kernel's own
+// arrays (corr_s, code_s).
+constexpr size_t GV_STATIC_SMEM = GV_COLS * sizeof(int) + 2 * GV_COLS * (GV_THREADS / 32);
 bool gemv_planes_fits(const qnn_gemm_desc *d) {
     const int kw_pad = round_up(ceil_div(d->K, 32), 4);
-    return d->N <= 16 && (size_t)d->a_bits * GV_COLS * kw_pad * 4 <= 48 * 1024;
+    return d->N <= 16 && (size_t)d->a_bits * GV_COLS * kw_pad * 4 + GV_STATIC_SMEM <= 48 * 1024;
 }
 
 qnn_status gemv_planes_launch(const qnn_gemm_desc *d, const void *W, const void *A,

@@ -84,3 +84,19 @@ def test_counting_kernel_writes_whole_rows(qb, w, a, w_enc, a_enc, M, N, K):
             assert (buf[:nb].reshape(N, -1)[:, M:] == 0).all()
         elif M % 32:
             assert (buf[:nb].view(np.uint32).reshape(3 * N, -1)[:, -1] >> (M % 32) == 0).all()
+
+
+@pytest.mark.parametrize("K,a,kernel", [
+    (24448, 4, "gemv_planes_kernel"), (24449, 4, "qgemm_bitserial_kernel"), (24576, 4, "qgemm_bitserial_kernel"),
+    (97920, 1, "gemv_planes_kernel"), (98176, 1, "qgemm_bitserial_kernel"),
+])
+def test_deepest_columns_that_the_counting_kernel_stages(qb, K, a, kernel):
+    """Columns and the kernel's own arrays share 48 KB; deeper ones go to the tiled kernel."""
+    case = synth.gemm_case(4900 + K, 9, 2, K, 1, a, 0, 0, out_bits=2)
+    Wp = qb.pack(qb.to_device_logical(case.W, 0), 1, 0, BITPLANES)
+    Ap = qb.pack(qb.to_device_logical(case.At, 0), a, 0, BITPLANES)
+    d = qb.qnn_gemm_desc(9, 2, K, 1, a, 2, 0, 0, BITPLANES, BITPLANES, INT8, qb.QNN_PATH_BITSERIAL, 0)
+    assert qb.qnn_qgemm_kernel_name(d, False) == kernel
+    out = torch.zeros(qb.qnn_gemm_out_bytes(d, False), dtype=torch.uint8, device="cuda")
+    qb.check(qb.qnn_qgemm(d, Wp, Ap, None, out))
+    assert np.array_equal(out.cpu().numpy().view(np.int32).reshape(2, 9), orc.qgemm(case.W, case.At, None).T)
