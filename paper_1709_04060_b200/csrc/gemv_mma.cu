@@ -522,12 +522,13 @@ static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
 // 7623 random problems timed with both kernels (half of them with one column; up to 12000 x 9216, every width,
 // encoding and output), replayed as a graph; call after call this kernel takes a little longer, hence the factor.
 // Twelve plane pairs and more of 2^22 weights are never counted: the estimate is up to a fifth off there (8192 x
-// 8192 W4A4, one column: 14.6 us counted, 11.5 here).  The choice costs 1.6 % (graph) and 1.4 % (calls) of the
+// 8192 W4A4, one column: 14.6 us counted, 11.5 here); one column in several passes is (2021 problems 6000 to 60000
+// deep: this kernel 1.25 times as long on average).  The choice costs 1.6 % (graph) and 1.4 % (calls) of the
 // faster one's time on average; always this kernel 5.1 % and 6.1 %, always counting 72 % and 53 %.
 static bool mv_planes_faster(const qnn_gemm_desc *d, bool has_thr) {
     if (d->w_bits * d->a_bits >= 12 && (long long)d->M * d->K >= (1ll << 22)) return true;
     MvPlan pl;
-    if (!mv_plan(d, has_thr, &pl)) return false;
+    if (!mv_plan(d, has_thr, &pl) || (d->N == 1 && pl.passes > 1)) return false;
     const int kw = ceil_div(d->K, 32), cols = d->N < 4 ? d->N : 4, pairs = d->w_bits * d->a_bits, nt = d->N > 8 ? 2 : 1;
     const double ctas = (double)ceil_div(d->M, 8) * ceil_div(d->N, 4), words = (double)d->M * kw;
     const double staged = d->w_enc == QNN_ENC_BIPOLAR && d->a_enc != QNN_ENC_BIPOLAR ? 0.43 : 0.285;   // with column sums
@@ -537,7 +538,8 @@ static bool mv_planes_faster(const qnn_gemm_desc *d, bool has_thr) {
     const double waves = (double)ceil_div(ceil_div(pl.groups, pl.per), sm_count());
     const double rounds = waves * pl.passes * ceil_div(ceil_div(pl.per, 3 - nt), pl.rsplit) * pl.u;
     const double here = 2.60 + rounds * (0.172 + 0.0142 * pl.v * d->w_bits) + 1.04e-6 * words * d->w_bits +
-                        1.74e-4 * d->N * kw * d->a_bits + (nt == 2 ? 0.2 : 0.0) + 1.3e-3 * pl.dsplit * pl.per * d->N;
+                        1.74e-4 * d->N * kw * d->a_bits + (nt == 2 ? 0.2 : 0.0) + 1.3e-3 * pl.dsplit * pl.per * d->N +
+                        2.0 * (waves * pl.passes - 1.0);
     return counted > 1.1 * here;
 }
 
