@@ -522,10 +522,13 @@ static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
 // 7623 random problems timed with both kernels (half of them with one column; up to 12000 x 9216, every width,
 // encoding and output), replayed as a graph; call after call this kernel takes a little longer, hence the factor.
 // Twelve plane pairs and more of 2^22 weights are never counted: the estimate is up to a fifth off there (8192 x
-// 8192 W4A4, one column: 14.6 us counted, 11.5 here); one column in several passes is (2021 problems 6000 to 60000
-// deep: this kernel 1.25 times as long on average).  The choice costs 1.6 % (graph) and 1.4 % (calls) of the
+// 8192 W4A4, one column: 14.6 us counted, 11.5 here).  One column of fewer pairs always is: a call by itself is up to
+// 7 % faster here, but in a chain the layers around it weigh more (fully connected layers of the AlexNet-shaped
+// network at batch 1: 68.7 us here, 65.6 counted); and so is one column in several passes (2021 problems 6000 to
+// 60000 deep: this kernel 1.25 times as long on average).  The choice costs 1.6 % (graph) and 1.4 % (calls) of the
 // faster one's time on average; always this kernel 5.1 % and 6.1 %, always counting 72 % and 53 %.
 static bool mv_planes_faster(const qnn_gemm_desc *d, bool has_thr) {
+    if (d->N == 1 && d->w_bits * d->a_bits < 12) return false;
     if (d->w_bits * d->a_bits >= 12 && (long long)d->M * d->K >= (1ll << 22)) return true;
     MvPlan pl;
     if (!mv_plan(d, has_thr, &pl) || (d->N == 1 && pl.passes > 1)) return false;

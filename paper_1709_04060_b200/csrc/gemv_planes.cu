@@ -18,6 +18,7 @@ namespace qnn {
 
 constexpr int GV_THREADS = 256;
 constexpr int GV_COLS = 4;          // columns per CTA
+constexpr size_t GV_COLUMN_SMEM = 48 * 1024;        // activation columns of a CTA
 
 struct GvParams {
     const uint32_t *W;     // [WB][M][kw]
@@ -194,15 +195,23 @@ gemv_planes_kernel(const GvParams p) {
 
 // Programmatic dependent launch: the kernel ahead releases its dependents at its end, so the CTAs
 // spread over all SMs (8192 x 8192 W1A2, one column, call after call: 8.1 -> 6.1 us).
-template <int WB, int AB, int MODE>
-static void gv_launch_one(const GvParams &p, dim3 grid, size_t smem, cudaStream_t s) {
-    if ((p.kw & 3) == 0) launch_pdl(gemv_planes_kernel<WB, AB, MODE, true>, grid, GV_THREADS, smem, s, p);
-    else launch_pdl(gemv_planes_kernel<WB, AB, MODE, false>, grid, GV_THREADS, smem, s, p);
+template <int WB, int AB, int MODE, bool VEC>
+static bool gv_launch_one(const GvParams &p, dim3 grid, size_t smem, cudaStream_t s) {
+    auto kern = gemv_planes_kernel<WB, AB, MODE, VEC>;
+    static std::atomic<bool> attr_done[QNN_MAX_DEVICES];           // per instantiation and device
+    // columns of nearly 48 KB pass the default limit together with the kernel's own arrays (corr_s, code_s)
+    if (smem > GV_COLUMN_SMEM - 1024) {
+        const int dev = current_device();
+        if (dev < 0 || !allow_smem(kern, GV_COLUMN_SMEM, attr_done[dev])) return false;
+    }
+    return launch_pdl(kern, grid, GV_THREADS, smem, s, p) == cudaSuccess;
 }
 
 template <int MODE>
-static bool gv_dispatch(int wb, int ab, const GvParams &p, dim3 grid, size_t smem, cudaStream_t s) {
-#define QNN_GV_CASE(W_, A_) if (wb == W_ && ab == A_) { gv_launch_one<W_, A_, MODE>(p, grid, smem, s); return true; }
+static qnn_status gv_dispatch(int wb, int ab, const GvParams &p, dim3 grid, size_t smem, cudaStream_t s) {
+#define QNN_GV_CASE(W_, A_)                                                                                              \
+    if (wb == W_ && ab == A_)                                                                                            \
+        return ((p.kw & 3) == 0 ? gv_launch_one<W_, A_, MODE, true>(p, grid, smem, s) : gv_launch_one<W_, A_, MODE, false>(p, grid, smem, s)) ? QNN_OK : QNN_ERR_CUDA;
     if (MODE == GV_REGULAR) {
         QNN_GV_CASE(1, 1) QNN_GV_CASE(1, 2) QNN_GV_CASE(1, 3) QNN_GV_CASE(1, 4)
         QNN_GV_CASE(2, 1) QNN_GV_CASE(2, 2) QNN_GV_CASE(2, 3) QNN_GV_CASE(2, 4)
@@ -216,15 +225,13 @@ static bool gv_dispatch(int wb, int ab, const GvParams &p, dim3 grid, size_t sme
         QNN_GV_CASE(1, 1)
     }
 #undef QNN_GV_CASE
-    return false;
+    return QNN_ERR_UNSUPPORTED;
 }
 
-// N <= 16 and the activation columns of one CTA fit the default 48 KB of shared memory beside the kernel's own
-// arrays (corr_s, code_s).
-constexpr size_t GV_STATIC_SMEM = GV_COLS * sizeof(int) + 2 * GV_COLS * (GV_THREADS / 32);
+// N <= 16 and the activation columns of one CTA fit 48 KB of shared memory.
 bool gemv_planes_fits(const qnn_gemm_desc *d) {
     const int kw_pad = round_up(ceil_div(d->K, 32), 4);
-    return d->N <= 16 && (size_t)d->a_bits * GV_COLS * kw_pad * 4 + GV_STATIC_SMEM <= 48 * 1024;
+    return d->N <= 16 && (size_t)d->a_bits * GV_COLS * kw_pad * 4 <= GV_COLUMN_SMEM;
 }
 
 qnn_status gemv_planes_launch(const qnn_gemm_desc *d, const void *W, const void *A,
@@ -255,21 +262,21 @@ qnn_status gemv_planes_launch(const qnn_gemm_desc *d, const void *W, const void 
     for (int i = 0; i < 4; ++i)
         for (int j = 0; j < 4; ++j)
             if (i + j < skip) p.coef[i][j] = 0;
-    bool ok;
+    qnn_status st;
     if (wb && ab) {
         p.coef[0][0] = skip > 0 ? 0 : -2;
         if (skip > 0) p.K = 0;                       // the pair's K - 2 popc(xor) goes as a whole
-        ok = gv_dispatch<GV_BOTH_BIPOLAR>(1, 1, p, grid, smem, s);
+        st = gv_dispatch<GV_BOTH_BIPOLAR>(1, 1, p, grid, smem, s);
     } else if (wb) {
         for (int j = 0; j < 4; ++j) { p.coef[0][j] = j < skip ? 0 : 2 * ca[j]; p.corr[j] = j < skip ? 0 : ca[j]; }
-        ok = gv_dispatch<GV_W_BIPOLAR>(1, d->a_bits, p, grid, smem, s);
+        st = gv_dispatch<GV_W_BIPOLAR>(1, d->a_bits, p, grid, smem, s);
     } else if (ab) {
         for (int i = 0; i < 4; ++i) { p.coef[i][0] = i < skip ? 0 : 2 * cw[i]; p.corr[i] = i < skip ? 0 : cw[i]; }
-        ok = gv_dispatch<GV_A_BIPOLAR>(d->w_bits, 1, p, grid, smem, s);
+        st = gv_dispatch<GV_A_BIPOLAR>(d->w_bits, 1, p, grid, smem, s);
     } else {
-        ok = gv_dispatch<GV_REGULAR>(d->w_bits, d->a_bits, p, grid, smem, s);
+        st = gv_dispatch<GV_REGULAR>(d->w_bits, d->a_bits, p, grid, smem, s);
     }
-    if (!ok) return QNN_ERR_UNSUPPORTED;
+    if (st != QNN_OK) return st;
     count_launch();
     return launch_status();
 }

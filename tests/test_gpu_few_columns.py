@@ -46,7 +46,7 @@ def test_plan_edges(qb, fmt, w, a, w_enc, a_enc, M, N, K):
     for out_fmt, raw in ((INT8, False), (BITPLANES, False), (INT8, True)):
         d = qb.qnn_gemm_desc(M, N, K, w, a, 3, w_enc, a_enc, fmt, a_fmt, out_fmt, 0, 0)
         name = qb.qnn_qgemm_kernel_name(d, not raw)
-        if fmt == FIELDS or (fmt == BITPLANES and (a > 1 or N > 3)):
+        if fmt == FIELDS or (fmt == BITPLANES and (a > 1 or (N > 3 and M > 1000))):
             assert name == "gemv_mma_kernel"
         elif fmt == INT8 and K <= 12288:                   # what the byte dot products stage
             assert (name == "gemv_mma_kernel") == ((not raw and (out_fmt == BITPLANES or M % 16 != 0)) or (N >= 4 and M * K >= 3 << 20))
@@ -87,11 +87,11 @@ def test_counting_kernel_writes_whole_rows(qb, w, a, w_enc, a_enc, M, N, K):
 
 
 @pytest.mark.parametrize("K,a,kernel", [
-    (24448, 4, "gemv_planes_kernel"), (24449, 4, "qgemm_bitserial_kernel"), (24576, 4, "qgemm_bitserial_kernel"),
-    (97920, 1, "gemv_planes_kernel"), (98176, 1, "qgemm_bitserial_kernel"),
+    (24576, 4, "gemv_planes_kernel"), (24577, 4, "qgemm_bitserial_kernel"),
+    (98304, 1, "gemv_planes_kernel"), (98176, 1, "gemv_planes_kernel"), (98305, 1, "qgemm_bitserial_kernel"),
 ])
 def test_deepest_columns_that_the_counting_kernel_stages(qb, K, a, kernel):
-    """Columns and the kernel's own arrays share 48 KB; deeper ones go to the tiled kernel."""
+    """48 KB of columns, the kernel's own arrays beside them; deeper ones go to the tiled kernel."""
     case = synth.gemm_case(4900 + K, 9, 2, K, 1, a, 0, 0, out_bits=2)
     Wp = qb.pack(qb.to_device_logical(case.W, 0), 1, 0, BITPLANES)
     Ap = qb.pack(qb.to_device_logical(case.At, 0), a, 0, BITPLANES)
