@@ -525,8 +525,9 @@ static bool mv_plan(const qnn_gemm_desc *d, bool has_thr, MvPlan *pl) {
 // 8192 W4A4, one column: 14.6 us counted, 11.5 here).  One column of fewer pairs always is: a call by itself is up to
 // 7 % faster here, but in a chain the layers around it weigh more (fully connected layers of the AlexNet-shaped
 // network at batch 1: 68.7 us here, 65.6 counted); and so is one column in several passes (2021 problems 6000 to
-// 60000 deep: this kernel 1.25 times as long on average).  The choice costs 1.6 % (graph) and 1.4 % (calls) of the
-// faster one's time on average; always this kernel 5.1 % and 6.1 %, always counting 72 % and 53 %.
+// 60000 deep: this kernel 1.25 times as long on average).  On average the choice costs 0.6 % (graph) and 0.9 %
+// (calls) of the faster one's time with two columns and more, 6.6 % and 3.0 % with one; always this kernel 0.4 % and
+// 1.6 %, with one column 10 % and 11 %; always counting 128 % and 98 %, with one column 11 % and 3.7 %.
 static bool mv_planes_faster(const qnn_gemm_desc *d, bool has_thr) {
     if (d->N == 1 && d->w_bits * d->a_bits < 12) return false;
     if (d->w_bits * d->a_bits >= 12 && (long long)d->M * d->K >= (1ll << 22)) return true;
