@@ -1462,7 +1462,8 @@ static double boxes_us(const qnn_conv_desc *cv, const BoxPlan &b, int tiles_c, i
 // of 128 images, 9 % of the k-blocks of a padded 27 x 27 map (5 x 5 taps), 10 % of a 13 x 13 one (3 x 3).  But
 // boxes rarely fill their 128 rows, and tiles are dealt in whole rounds: a round more costs what many taps save.
 // So of the extents with the smallest rounds times mean tile, the one whose busiest pair of SMs is done first, and
-// that only if consecutive pixels take longer.  Sums, and codes of three or four bits, are stored at a pace that an
+// that only if consecutive pixels take longer (28 such layers of random sizes 0.71 to 1.01 of the time of consecutive
+// pixels, mean 0.91; 62 whose busiest pair would be done no sooner 0.92 to 1.08, mean 1.02).  Sums, and codes of three or four bits, are stored at a pace that an
 // epilogue of scattered pixels does not keep up with: there the saving has to be larger (1 x 1 boxes estimated at
 // 0.9 to 0.95: 16 x 16 x 80 -> 384, 5 x 5, batch 241, 3 bits 121 -> 129 us; 34 x 34 x 32 -> 256, 4 bits 85 -> 100).
 static bool search_boxes(const qnn_conv_desc *cv, bool light, int tiles_c, int pairs, BoxPlan *plan) {
